@@ -173,9 +173,6 @@ struct WalkParams {
     uint32_t reuse;          // passes over each walk's pairs (>= 1)
     uint64_t R;              // record stride (K + 2)
     int32_t* rec;            // rec[s R], rec[s R + 1] = the pair of sample t0 + s
-    uint64_t* items;         // nullable: grouping items of slots 0 and 1
-    uint32_t ctx_off;        // row offset of the context table in the items
-    uint32_t slot_bits;      // item value = (s << slot_bits) | slot
 };
 size_t walk_smem_bytes(int L);
 // row_ptr[n+1]: first arc of each node, from the sorted src.

@@ -51,16 +51,12 @@
 #include <cstring>
 #include <vector>
 
-#include <cooperative_groups.h>
-
 #include "bulk.cuh"
 #include "line_internal.cuh"
 #include "rows.cuh"
 #include "scan.cuh"
 
 namespace line {
-
-namespace cg = cooperative_groups;
 
 // Programmatic dependent launch: let the next kernel of the stream start its
 // prologue, and wait until the previous kernel's writes are visible.
@@ -76,7 +72,8 @@ constexpr uint32_t kLongBit = 1u << 31;  // in mdesc.y: summed by a CTA
 // Sort item value: (sample within the chunk) << kSlotBits | slot.
 constexpr uint32_t kSlotBits = 6;
 constexpr uint32_t kSlotMask = (1u << kSlotBits) - 1u;
-// slot_info.x: sorted position within the batch, bit 31 set for a singleton segment.
+// slot_info: a shared row's position within the batch, or kSingleBit for a row
+// that the batch touches once.
 constexpr uint32_t kSingleBit = 1u << 31;
 
 // Fibonacci hashing: spreads the hot (low) row ids of skewed graphs.  The
@@ -108,7 +105,7 @@ struct DataParams {
     int64_t n_nodes;
     uint32_t row_bits;
     const int32_t* rec;      // [chunk samples][K+2]
-    const uint2* slot_info;  // [chunk samples][K+2]: {position | singleton bit, segment (first position)}
+    const uint32_t* slot_info;  // [chunk samples][K+2]: position, or the singleton bit
     const uint4* mdesc;      // [n_batches][mcap] shared segments: {first position, length | long bit, row, pair count}
     const uint32_t* mcount;  // [n_batches]
     uint32_t mcap;
@@ -136,9 +133,7 @@ struct DataParams {
 // Record entry idx of the group's sample: lane idx % L holds entries
 // idx < L in `held`; later ones are read from memory.
 __device__ __forceinline__ int32_t shfl_w(uint32_t gm, int32_t v, int src, int w) { return __shfl_sync(gm, v, src, w); }
-__device__ __forceinline__ uint2 shfl_w(uint32_t gm, uint2 v, int src, int w) {
-    return make_uint2(__shfl_sync(gm, v.x, src, w), __shfl_sync(gm, v.y, src, w));
-}
+__device__ __forceinline__ uint32_t shfl_w(uint32_t gm, uint32_t v, int src, int w) { return __shfl_sync(gm, v, src, w); }
 
 template <int L, typename T>
 __device__ __forceinline__ T rec_entry(uint32_t gm, T held, const T* row, int idx, bool active) {
@@ -158,8 +153,8 @@ __device__ __forceinline__ T rec_entry(uint32_t gm, T held, const T* row, int id
 // leaves room on every SM for the next chunk's pre-pass.
 template <int D, int DT, int JB = 8>
 __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bool active, float eta, uint64_t t0,
-                                                uint32_t gm, int32_t r0, uint2 i0, const int32_t* rec,
-                                                const uint2* info) {
+                                                uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
+                                                const uint32_t* info) {
     using G = Geom<D, DT>;
     const int32_t u = __shfl_sync(gm, r0, 0, G::L);
     float xu[G::E];
@@ -197,17 +192,17 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
         if (j > p.K) continue;
 #pragma unroll
         for (int e = 0; e < G::E; ++e) du[e] = fmaf(g[j], c[j][e], du[e]);
-        const uint2 inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
+        const uint32_t inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
         const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
         if (active) {
-            if (inf.x & kSingleBit) {
+            if (inf & kSingleBit) {
                 const float decay = 1.0f * etalam;
                 float x[G::E];
 #pragma unroll
                 for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[j][e], c[j][e]) + g[j] * xu[e];
                 store_row<D, DT>(p.C, y, lig, x, p.seed, t0, ctx_table);
             } else {
-                float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf.x * D + lig * G::E);
+                float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
 #pragma unroll
                 for (int q = 0; q < G::E / 4; ++q)
                     st_cg(dst + q, make_float4(g[j] * xu[4 * q], g[j] * xu[4 * q + 1], g[j] * xu[4 * q + 2],
@@ -215,15 +210,15 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
             }
         }
     }
-    const uint2 inf0 = shfl_w(gm, i0, 0, G::L);
+    const uint32_t inf0 = shfl_w(gm, i0, 0, G::L);
     if (active) {
-        if (inf0.x & kSingleBit) {
+        if (inf0 & kSingleBit) {
             const float decay = (float)(p.K + 1) * etalam;
 #pragma unroll
             for (int e = 0; e < G::E; ++e) xu[e] = fmaf(-decay, xu[e], xu[e]) + du[e];
             store_row<D, DT>(p.U, u, lig, xu, p.seed, t0, 0u);
         } else {
-            float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0.x * D + lig * G::E);
+            float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0 * D + lig * G::E);
 #pragma unroll
             for (int q = 0; q < G::E / 4; ++q) st_cg(dst + q, make_float4(du[4 * q], du[4 * q + 1], du[4 * q + 2], du[4 * q + 3]));
         }
@@ -235,8 +230,8 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
 // time.  Same arithmetic, in the same order, as the register body.
 template <int D, int DT>
 __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig, int lane, bool active, float eta,
-                                                   uint64_t t0, uint32_t gm, int32_t r0, uint2 i0, const int32_t* rec,
-                                                   const uint2* info, float* ctx_stage) {
+                                                   uint64_t t0, uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
+                                                   const uint32_t* info, float* ctx_stage) {
     using G = Geom<D, DT>;
     constexpr int CH = G::E <= 4 ? 8 : 4;  // context rows in flight per lane
     const int32_t u = __shfl_sync(gm, r0, 0, G::L);
@@ -306,10 +301,10 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
             const float g = j == 0 ? eta * (1.0f - sig) : -eta * p.alpha_neg * sig;
 #pragma unroll
             for (int e = 0; e < G::E; ++e) du[e] = fmaf(g, c[e], du[e]);
-            const uint2 inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
+            const uint32_t inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
             const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
             if (active) {
-                if (inf.x & kSingleBit) {
+                if (inf & kSingleBit) {
                     // the only reader of row y in this batch: write it now
                     const float decay = 1.0f * etalam;
                     float x[G::E];
@@ -317,7 +312,7 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
                     for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[e], c[e]) + g * xu[e];
                     store_row<D, DT>(p.C, y, lig, x, p.seed, t0, ctx_table);
                 } else {
-                    float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf.x * D + lig * G::E);
+                    float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
 #pragma unroll
                     for (int q = 0; q < G::E / 4; ++q)
                         st_cg(dst + q, make_float4(g * xu[4 * q], g * xu[4 * q + 1], g * xu[4 * q + 2], g * xu[4 * q + 3]));
@@ -325,15 +320,15 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
             }
         }
     }
-    const uint2 inf0 = shfl_w(gm, i0, 0, G::L);
+    const uint32_t inf0 = shfl_w(gm, i0, 0, G::L);
     if (active) {
-        if (inf0.x & kSingleBit) {
+        if (inf0 & kSingleBit) {
             const float decay = (float)(p.K + 1) * etalam;
 #pragma unroll
             for (int e = 0; e < G::E; ++e) xu[e] = fmaf(-decay, xu[e], xu[e]) + du[e];
             store_row<D, DT>(p.U, u, lig, xu, p.seed, t0, 0u);
         } else {
-            float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0.x * D + lig * G::E);
+            float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0 * D + lig * G::E);
 #pragma unroll
             for (int q = 0; q < G::E / 4; ++q) st_cg(dst + q, make_float4(du[4 * q], du[4 * q + 1], du[4 * q + 2], du[4 * q + 3]));
         }
@@ -347,10 +342,10 @@ __device__ __forceinline__ void sample_item(const DataParams& p, int64_t s_local
     const int R = p.K + 2;
     const int64_t sbase = (active ? s_local : 0) * R;
     const int32_t* rec = p.rec + sbase;
-    const uint2* info = p.slot_info + sbase;
+    const uint32_t* info = p.slot_info + sbase;
     const uint32_t gm = group_mask<G::L>(lane / G::L);
     const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
-    const uint2 i0 = (active && lig < R) ? info[lig] : make_uint2(0u, 0u);
+    const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
     if constexpr (PDL) pdl_wait();  // the tables' rows: written by the previous kernel
     if constexpr (G::E <= 4) {
         if (p.K < 6) {
@@ -660,8 +655,8 @@ __device__ __forceinline__ void slot_row(const unsigned char* set, int j, int li
 
 template <int D, int DT>
 __device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, bool active, float eta, uint64_t t0,
-                                                 uint32_t gm, int32_t r0, uint2 i0, const int32_t* rec,
-                                                 const uint2* info, const unsigned char* set) {
+                                                 uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
+                                                 const uint32_t* info, const unsigned char* set) {
     using G = Geom<D, DT>;
     constexpr int JB = 8;
     const int32_t u = __shfl_sync(gm, r0, 0, G::L);
@@ -698,17 +693,17 @@ __device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, b
             const float g = j == 0 ? eta * (1.0f - sig) : -eta * p.alpha_neg * sig;
 #pragma unroll
             for (int e = 0; e < G::E; ++e) du[e] = fmaf(g, c[e], du[e]);
-            const uint2 inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
+            const uint32_t inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
             const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
             if (active) {
-                if (inf.x & kSingleBit) {
+                if (inf & kSingleBit) {
                     const float decay = 1.0f * etalam;
                     float x[G::E];
 #pragma unroll
                     for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[e], c[e]) + g * xu[e];
                     store_row<D, DT>(p.C, y, lig, x, p.seed, t0, ctx_table);
                 } else {
-                    float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf.x * D + lig * G::E);
+                    float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
 #pragma unroll
                     for (int q = 0; q < G::E / 4; ++q)
                         st_cg(dst + q, make_float4(g * xu[4 * q], g * xu[4 * q + 1], g * xu[4 * q + 2], g * xu[4 * q + 3]));
@@ -716,15 +711,15 @@ __device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, b
             }
         }
     }
-    const uint2 inf0 = shfl_w(gm, i0, 0, G::L);
+    const uint32_t inf0 = shfl_w(gm, i0, 0, G::L);
     if (active) {
-        if (inf0.x & kSingleBit) {
+        if (inf0 & kSingleBit) {
             const float decay = (float)(p.K + 1) * etalam;
 #pragma unroll
             for (int e = 0; e < G::E; ++e) xu[e] = fmaf(-decay, xu[e], xu[e]) + du[e];
             store_row<D, DT>(p.U, u, lig, xu, p.seed, t0, 0u);
         } else {
-            float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0.x * D + lig * G::E);
+            float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0 * D + lig * G::E);
 #pragma unroll
             for (int q = 0; q < G::E / 4; ++q) st_cg(dst + q, make_float4(du[4 * q], du[4 * q + 1], du[4 * q + 2], du[4 * q + 3]));
         }
@@ -916,9 +911,9 @@ __global__ void __launch_bounds__(kPersistMaxWarps * 32, 1) k_persistent(DataPar
             const unsigned char* set = wslots + (size_t)sl * G::GPW * set_bytes + grp * set_bytes;
             const int64_t sbase = (active ? s_local : 0) * R;
             const int32_t* rec = p.rec + sbase;
-            const uint2* info = p.slot_info + sbase;
+            const uint32_t* info = p.slot_info + sbase;
             const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
-            const uint2 i0 = (active && lig < R) ? info[lig] : make_uint2(0u, 0u);
+            const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
             sample_body_slot<D, DT>(p, lig, active, eta, t0, gm, r0, i0, rec, info, set);
             // the slot's rows are read: it may be refilled by bulk copies
             fence_proxy_async_smem();
@@ -1014,38 +1009,57 @@ struct PrepassParams {
     int K, order;
     int walk;  // 1: slots 0 and 1 come from the walk sampler (no arc draw here)
     int32_t* rec;
-    uint64_t* items;  // null: records only (Hogwild schedule)
     uint64_t* t_out;  // receives t_chunk (read by graph replays of the data phase)
+    // per batch of the chunk (minibatch schedules): the learning rate, and
+    // the counters of the grouping, zeroed here
+    int n_batches;
+    float lr0, lr_floor;
+    int lr_schedule;
+    uint64_t lr_total;
+    float* eta;  // null: no per-batch outputs (Hogwild schedule)
+    uint32_t* mcount;
+    uint32_t* lcount;
+    uint32_t* pcount;
 };
 
 __device__ __forceinline__ uint64_t make_item(uint32_t rowid, uint32_t s_local, uint32_t slot) {
     return ((uint64_t)rowid << 32) | ((s_local << kSlotBits) | slot);
 }
 
+// eta of the batch starting at global sample t0: lr0 (schedule 0) or
+// lr0 * max(1 - t0/T, floor) (schedule 1), in FP32, 1 - t0/T as (T - t0) / T
+// from the exact integer difference.
+__device__ __forceinline__ float batch_eta(const PrepassParams& p, uint64_t t0) {
+    float f = 1.0f;
+    if (p.lr_schedule == 1) {
+        f = t0 >= p.lr_total ? 0.0f : (float)(p.lr_total - t0) / (float)p.lr_total;
+        if (f < p.lr_floor) f = p.lr_floor;
+    }
+    return p.lr0 * f;
+}
+
 __global__ void k_chunk_draws(PrepassParams p) {
-    if (blockIdx.x == 0 && threadIdx.x == 0 && p.t_out) *p.t_out = p.t_chunk;
+    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (tid == 0 && p.t_out) *p.t_out = p.t_chunk;
+    if (p.eta)
+        for (uint32_t b = tid; b < (uint32_t)p.n_batches; b += stride) {
+            p.eta[b] = batch_eta(p, p.t_chunk + (uint64_t)b * (uint64_t)p.batch);
+            p.mcount[b] = p.lcount[b] = p.pcount[b] = 0u;
+        }
     const uint32_t C1 = (uint32_t)p.K + 1u, R = (uint32_t)p.K + 2u;
     const uint32_t total = (uint32_t)p.chunk_samples * C1;
-    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
+    for (uint32_t q = tid; q < total; q += stride) {
         const uint32_t s = q / C1;
         const uint32_t c = q - s * C1;
         const uint4 w = draw_words(p.seed, 0u, p.t_chunk + (uint64_t)s, c);
-        const uint32_t ctx_off = p.order == 2 ? (uint32_t)p.n_nodes : 0u;
         const uint32_t base = s * R;
         if (c == 0) {
             if (p.walk) continue;
             const uint32_t e = alias_pick(p.edge_tab, (uint64_t)p.n_arcs, w);
-            const int32_t u = __ldg(p.src + e), v = __ldg(p.dst + e);
-            p.rec[base] = u;
-            p.rec[base + 1] = v;
-            if (p.items) {
-                p.items[base] = make_item((uint32_t)u, s, 0u);
-                p.items[base + 1] = make_item((uint32_t)v + ctx_off, s, 1u);
-            }
+            p.rec[base] = __ldg(p.src + e);
+            p.rec[base + 1] = __ldg(p.dst + e);
         } else {
-            const uint32_t y = alias_pick(p.neg_tab, (uint64_t)p.n_nodes, w);
-            p.rec[base + 1 + c] = (int32_t)y;
-            if (p.items) p.items[base + 1 + c] = make_item(y + ctx_off, s, 1u + c);
+            p.rec[base + 1 + c] = (int32_t)alias_pick(p.neg_tab, (uint64_t)p.n_nodes, w);
         }
     }
 }
@@ -1067,13 +1081,16 @@ struct GroupParams {
     int64_t chunk_samples;
     uint32_t R, K, parts;  // parts: bucketing CTAs per batch
     uint32_t row_bits;
-    const uint64_t* items;  // draws, (sample, slot) order
-    uint64_t* bucketed;     // items grouped by bucket within each batch
+    uint32_t R_magic;       // floor(2^32 / R) + 1: i / R = mulhi(i, R_magic) for i < 2^32 / R
+    uint32_t ctx_off;       // row id of the context table's first row
+    const int32_t* rec;     // draws, (sample, slot) order
+    uint64_t* bucketed;     // items grouped by bucket within each batch (k_group_parts: keys that exceed a CTA)
     uint64_t* tmp;          // scratch of the same size
     uint32_t* gcnt;         // [n_batches][parts][256] bucket counts of each part
     uint32_t* boff;         // [n_batches][257] bucket starts within the batch
+    uint32_t* pcount;       // [n_batches] positions handed out (k_group_parts)
     // outputs
-    uint2* slot_info;
+    uint32_t* slot_info;
     uint4* mdesc;
     uint32_t* mcount;
     uint32_t mcap;
@@ -1089,6 +1106,12 @@ __device__ __forceinline__ void batch_range(const GroupParams& q, int b, uint64_
     *n = (uint32_t)nb * q.R;
 }
 
+// Entry i of the chunk as an item: row id << 32 | (sample, slot).
+__device__ __forceinline__ uint64_t item_at(const GroupParams& q, uint64_t at) {
+    const uint32_t i = (uint32_t)at, s = i / q.R, slot = i - s * q.R;  // a chunk has fewer than 2^31 entries
+    return make_item((uint32_t)q.rec[i] + (slot ? q.ctx_off : 0u), s, slot);
+}
+
 __global__ void __launch_bounds__(kBucketThreads) k_bucket_count(GroupParams q) {
     __shared__ uint32_t cnt[kBuckets];
     const int part = blockIdx.x, b = blockIdx.y;
@@ -1099,7 +1122,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_count(GroupParams q) 
     batch_range(q, b, &base, &n);
     const uint32_t lo = min(n, (uint32_t)part * kPartItems), hi = min(n, lo + kPartItems);
     for (uint32_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const uint32_t rowid = (uint32_t)(q.items[base + i] >> 32);
+        const uint32_t rowid = (uint32_t)(item_at(q, base + i) >> 32);
         atomicAdd(&cnt[bucket_of(rowid)], 1u);
         if (q.depmap) {
             const uint32_t db = dep_bit(rowid);
@@ -1150,7 +1173,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_scatter(GroupParams q
     for (uint32_t r = wlo; r < whi; r += 32) {
         const uint32_t i = r + lane;
         const bool valid = i < whi;
-        const uint32_t d = valid ? bucket_of((uint32_t)(q.items[base + i] >> 32)) : 0xFFFFu;
+        const uint32_t d = valid ? bucket_of((uint32_t)(item_at(q, base + i) >> 32)) : 0xFFFFu;
         const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
         if (valid && (peers & lt) == 0) wcnt[warp][d] += __popc(peers);
         __syncwarp();
@@ -1168,7 +1191,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_scatter(GroupParams q
     for (uint32_t r = wlo; r < whi; r += 32) {
         const uint32_t i = r + lane;
         const bool valid = i < whi;
-        const uint64_t it = valid ? q.items[base + i] : 0ull;
+        const uint64_t it = valid ? item_at(q, base + i) : 0ull;
         const uint32_t d = valid ? bucket_of((uint32_t)(it >> 32)) : 0xFFFFu;
         const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
         const uint32_t before = valid ? wcnt[warp][d] : 0u;
@@ -1310,7 +1333,7 @@ __global__ void __launch_bounds__(kSortThreads) k_bucket_sort(GroupParams q) {
             const uint32_t slot = v & kSlotMask;
             cnt += slot == 0 ? q.K + 1 : 1u;
             const uint32_t pos = (uint32_t)(gpos + k);
-            q.slot_info[(v >> kSlotBits) * q.R + slot] = make_uint2(pos | (len == 1 ? kSingleBit : 0u), head);
+            q.slot_info[(v >> kSlotBits) * q.R + slot] = len == 1 ? kSingleBit : pos;
         }
         if (len > 1) {
             uint32_t flagged = len;
@@ -1325,22 +1348,40 @@ __global__ void __launch_bounds__(kSortThreads) k_bucket_sort(GroupParams q) {
     }
 }
 
-// ---- Grouping of a batch by one thread-block cluster (batches of up to 8 x
-// 3,584 items).  The items are split into P = 2^log_parts parts by the top
-// bits of hrow(row) (a part is a contiguous range of buckets) and each part
-// into 256 sub-buckets by the next 8 bits.  CTA rank r of batch b's cluster
-// counts the (part, sub-bucket) sizes of the r-th slice of the batch's draws;
-// after an exchange of counts every CTA knows where each of its keys
-// (hrow(row) << 32 | index) goes in the owner's shared memory (distributed
-// shared memory) and sends it there.  Each owner then sorts its sub-buckets
-// (about 14 keys each: one thread; larger ones: one warp) and emits its
-// segments.  The order, hence every position, is the same as the bucketed
-// path's: (hrow(row), index).
-constexpr int kGroupThreads = 512;
-constexpr uint32_t kGroupCap = 4096;  // keys of a part held in shared memory
-constexpr int kGroupMaxLog = 3;       // clusters of up to 8 CTAs (portable size)
-constexpr int kSub = 256;             // sub-buckets of a part
-constexpr int kGroupPerThread = 8;    // slice items per thread loaded at once
+// ---- Grouping of a batch by P = 2^log_parts independent CTAs (batches of up
+// to 16 x 16,384 items).  CTA `me` of batch b owns the rows whose hrow starts
+// with the bits `me`: it scans all of the batch's record entries (they are in
+// L2) and keeps its own, so no CTA waits for another.
+//   1. A row that occurs once needs no position: two bitmaps of 2^17 bits,
+//      indexed by hrow, record which bits are hit and which are hit twice.
+//      On R-MAT 20 73% of a batch's items are such rows; they (but for about
+//      one in ten, which shares its bit) get the singleton mark at once.
+//   2. The other items ("candidates") are counted into 1,024 sub-buckets by
+//      further hrow bits and placed there as keys (hrow(row) << 32 | sample,
+//      slot), in no particular order.
+//   3. One thread per key compares it with the keys of its sub-bucket (about
+//      five): the keys of smaller rows, of its own row, and those of its row
+//      that come before it give its position, its segment's head and length.
+//      Nothing is sorted.  Only a sub-bucket of more than kRankMax keys (a
+//      hub row) is sorted, by one warp.
+// Positions are unique within the batch and contiguous per row, in (sample,
+// slot) order; where a part begins depends on the order in which the parts
+// arrive, which no result depends on.
+// Bound: issue slots and the latency of the three scans.  A chunk of 64
+// batches of 28,672 items (R-MAT 20, d = 128, K = 5) takes 36 us with nothing
+// beside it and 38-41 beside the data phase, on 128 CTAs; the earlier form,
+// which sorted all items of a batch in an 8-CTA cluster, 107 and 118 on 512.
+// 16 batches of 114,688 items (8 parts each): 82 us against 276 for the
+// three kernels below.  One order at B = 4096 went from 8.74 to 7.80 ms for
+// 2^22 samples (BF16), both orders from 13.99 to 12.09 (FP32).  Beyond 16
+// parts every part's scan of the whole batch costs more than it saves.
+constexpr int kPartThreads = 1024;
+constexpr uint32_t kPartItems2 = 16384;  // a part's share of the items, at most
+constexpr uint32_t kPartCap = 15360;     // keys held in shared memory; more go to the scratch array
+constexpr int kPartMaxLog = 4;
+constexpr int kPartSub = 1024;           // sub-buckets of a part (one per thread)
+constexpr uint32_t kMapBits = 17;
+constexpr uint32_t kRankMax = 128;
 
 // In-place ascending sort of a[0 .. n) by one warp: a bitonic network whose
 // comparators all put the minimum first (per merge size k the mirror
@@ -1381,279 +1422,171 @@ __device__ __forceinline__ void warp_sort_keys(uint64_t* a, uint32_t n) {
     }
 }
 
-// The second half of the grouping of one part: sort its sub-buckets, write
-// its bucket starts and emit its segments.  `a` holds the part's nq keys
-// grouped by sub-bucket (s_start); inlined once for shared memory and once
-// for the global scratch, so that the common case uses shared-memory accesses.
-struct GroupShared {
-    uint32_t* start;  // [kSub + 1] sub-bucket starts
-    uint32_t* big;    // [kSub]
-    uint32_t* nbig;
-    uint32_t* mcnt;
-    uint32_t* lcnt;
-    uint32_t* mbase;
-    uint32_t* lbase;
-};
-
-__device__ __forceinline__ void group_tail(const GroupParams& q, uint64_t* a, uint32_t nq, uint32_t n,
-                                           uint32_t qbase, int b, uint32_t me, uint32_t P, int log_parts,
-                                           const GroupShared& sh) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kWarps = kGroupThreads / 32;
-    const uint32_t* s_start = sh.start;
-    const uint32_t gpos = qbase;  // position of the part's first key in the batch
-    // sort each sub-bucket by (hrow(row), index): up to 32 keys by ranks
-    // within a warp, larger ones (a hot row) by a warp bitonic sort
-    for (int sb = warp; sb < kSub; sb += kWarps) {
-        const uint32_t s0 = s_start[sb], c = s_start[sb + 1] - s0;
-        if (c <= 1) continue;
-        if (c <= 32) {
-            const uint64_t key = lane < (int)c ? a[s0 + lane] : ~0ull;
-            uint32_t rank = 0;
-            for (uint32_t l = 0; l < c; ++l) rank += __shfl_sync(0xFFFFFFFFu, key, l) < key;
-            __syncwarp();
-            if (lane < (int)c) a[s0 + rank] = key;
-            __syncwarp();
-        } else {
-            warp_sort_keys(a + s0, c);
-        }
+// Lists the shared segments of the warp's lanes with len > 1 (head: first
+// position, z: its source entries).  Called by whole warps.
+__device__ __forceinline__ void list_segments(const GroupParams& q, int b, bool is_head, uint32_t head, uint32_t len,
+                                              uint32_t hv, uint32_t z) {
+    const int lane = threadIdx.x & 31;
+    const bool m = is_head && len > 1, l = m && len > kChunk;
+    const uint32_t mm = __ballot_sync(0xFFFFFFFFu, m), lm = __ballot_sync(0xFFFFFFFFu, l);
+    if (!mm) return;
+    uint32_t base = 0;  // lane 0: mdesc entries, lane 1: ldesc entries
+    if (lane == 0) base = atomicAdd(q.mcount + b, (uint32_t)__popc(mm));
+    else if (lane == 1 && lm) base = atomicAdd(q.lcount + b, (uint32_t)__popc(lm));
+    const uint32_t mb = __shfl_sync(0xFFFFFFFFu, base, 0), lb = __shfl_sync(0xFFFFFFFFu, base, 1);
+    const uint32_t lt = (1u << lane) - 1u;
+    if (m) {
+        // pair count: K + 1 for a source entry, 1 otherwise
+        const uint4 d = make_uint4(head, l ? len | kLongBit : len, unhrow(hv), len + z * q.K);
+        q.mdesc[(size_t)b * q.mcap + mb + __popc(mm & lt)] = d;
+        if (l) q.ldesc[(size_t)b * q.lcap + lb + __popc(lm & lt)] = make_uint4(head, len, d.z, d.w);
     }
-    __syncthreads();
-    // bucket starts of the part's buckets: bucket (me, j) begins at
-    // sub-bucket j << log_parts
-    const uint32_t nbk = (uint32_t)kBuckets >> log_parts, d0 = me * nbk;
-    for (uint32_t j = threadIdx.x; j < nbk; j += blockDim.x)
-        q.boff[(size_t)b * (kBuckets + 1) + d0 + j] = qbase + s_start[j << log_parts];
-    if (me == P - 1u && threadIdx.x == 0) q.boff[(size_t)b * (kBuckets + 1) + kBuckets] = n;
-    // segments (a segment never crosses a sub-bucket).  Per sub-bucket, in
-    // rounds of 32 keys: lane l holds key s0 + r + l; starts come from a
-    // ballot, the carry is the open segment of the previous round.
-    // Pass 0 counts the shared and long segments, pass 1 writes.
-    for (int pass = 0; pass < 2; ++pass) {
-        uint32_t n_m = 0, n_l = 0;
-        for (int sb = warp; sb < kSub; sb += kWarps) {
-            const uint32_t s0 = s_start[sb], c = s_start[sb + 1] - s0;
-            for (uint32_t r = 0; r < c; r += 32) {
-                const uint32_t i = s0 + r + lane;
-                const bool valid = r + lane < c;
-                const uint64_t key = valid ? a[i] : ~0ull;
-                const uint32_t hk = (uint32_t)(key >> 32);
-                const uint32_t prev = (valid && i > s0) ? (uint32_t)(a[i - 1] >> 32) : ~hk;
-                const bool start = valid && prev != hk;
-                const uint32_t smask = __ballot_sync(0xFFFFFFFFu, start);
-                // each key's segment: first start at or below it (or the
-                // round's carry), next start above it (or the sub-bucket end)
-                const uint32_t below = smask & (0xFFFFFFFFu >> (31 - lane));
-                uint32_t head = below ? s0 + r + (31 - __clz(below)) : 0u;
-                uint32_t len = 0;
-                if (valid) {
-                    if (!below) {  // continues a segment of an earlier round (a hot row)
-                        uint32_t h0 = i;
-                        while (h0 > s0 && (uint32_t)(a[h0 - 1] >> 32) == hk) --h0;
-                        head = h0;
-                    }
-                    const uint32_t above = smask & ~(0xFFFFFFFFu >> (31 - lane));
-                    uint32_t end = above ? s0 + r + (__ffs(above) - 1) : 0u;
-                    if (!above) {
-                        end = s0 + min(c, r + 32);
-                        while (end < s0 + c && (uint32_t)(a[end] >> 32) == hk) ++end;
-                    }
-                    len = end - head;
-                }
-                const bool is_head = valid && i == head;
-                if (pass == 0) {
-                    n_m += is_head && len > 1;
-                    n_l += is_head && len > kChunk;
-                    continue;
-                }
-                const uint32_t hpos = (uint32_t)(gpos + head);
-                if (valid) {
-                    const uint32_t v = (uint32_t)key;
-                    const uint32_t slot = v & kSlotMask;
-                    const uint32_t pos = (uint32_t)(gpos + i);
-                    q.slot_info[(v >> kSlotBits) * q.R + slot] = make_uint2(pos | (len == 1 ? kSingleBit : 0u), hpos);
-                }
-                if (is_head) {
-                    if (len > 1) {
-                        // pair count of the segment: K + 1 for a source entry, 1 otherwise
-                        uint32_t cnt = 0;
-                        for (uint32_t k = head; k < head + len; ++k)
-                            cnt += ((uint32_t)a[k] & kSlotMask) == 0 ? q.K + 1 : 1u;
-                        const uint32_t key_row = unhrow(hk);
-                        uint32_t flagged = len;
-                        if (len > kChunk) {
-                            const uint32_t l = *sh.lbase + atomicAdd(sh.lcnt, 1u);
-                            q.ldesc[(size_t)b * q.lcap + l] = make_uint4(hpos, len, key_row, cnt);
-                            flagged |= kLongBit;
-                        }
-                        const uint32_t m = *sh.mbase + atomicAdd(sh.mcnt, 1u);
-                        q.mdesc[(size_t)b * q.mcap + m] = make_uint4(hpos, flagged, key_row, cnt);
-                    }
+}
+
+// Steps 2b and 3 for the part's nc keys, grouped by sub-bucket in a (shared
+// memory, or the scratch array; inlined for each).
+__device__ __forceinline__ void group_segments(const GroupParams& q, const uint64_t* a, uint64_t* aw, uint32_t nc,
+                                               const uint32_t* start, int log_parts, uint32_t pbase, int b,
+                                               const uint16_t* big, uint32_t nbig) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint32_t i0 = warp * 32; i0 < nc; i0 += kPartThreads) {
+        const uint32_t i = i0 + lane;
+        bool mine = i < nc;
+        const uint64_t key = mine ? a[i] : 0ull;
+        const uint32_t hv = (uint32_t)(key >> 32), v = (uint32_t)key;
+        const uint32_t sub = (hv << log_parts) >> (32 - 10);
+        const uint32_t s0 = start[sub], c = start[sub + 1] - s0;
+        mine = mine && c <= kRankMax;
+        uint32_t lower = 0, same = 0, before = 0, z = 0;
+        if (mine) {
+            for (uint32_t j = 0; j < c; ++j) {
+                const uint64_t k2 = a[s0 + j];
+                const uint32_t h2 = (uint32_t)(k2 >> 32), v2 = (uint32_t)k2;
+                lower += h2 < hv;
+                if (h2 == hv) {
+                    ++same;
+                    before += v2 < v;
+                    z += (v2 & kSlotMask) == 0;
                 }
             }
         }
-        if (pass == 0) {
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) {
-                n_m += __shfl_xor_sync(0xFFFFFFFFu, n_m, o);
-                n_l += __shfl_xor_sync(0xFFFFFFFFu, n_l, o);
+        const uint32_t head = pbase + s0 + lower;
+        if (mine) q.slot_info[(v >> kSlotBits) * q.R + (v & kSlotMask)] = same == 1 ? kSingleBit : head + before;
+        list_segments(q, b, mine && before == 0, head, same, hv, z);
+    }
+    // large sub-buckets: one warp each
+    for (uint32_t g = warp; g < nbig; g += kPartThreads / 32) {
+        const uint32_t s0 = start[big[g]], s1 = start[big[g] + 1];
+        warp_sort_keys(aw + s0, s1 - s0);
+        for (uint32_t h = s0; h < s1;) {
+            // the segment that begins at h: its end, and its source entries
+            const uint32_t hv = (uint32_t)(a[h] >> 32);
+            uint32_t e = h, z = 0, in = 0xFFFFFFFFu;
+            for (; in == 0xFFFFFFFFu && e < s1; e += 32) {
+                const uint64_t key = e + lane < s1 ? a[e + lane] : 0ull;
+                const bool same = e + lane < s1 && (uint32_t)(key >> 32) == hv;
+                in = __ballot_sync(0xFFFFFFFFu, same);
+                z += __popc(__ballot_sync(0xFFFFFFFFu, same && ((uint32_t)key & kSlotMask) == 0));
             }
-            if (threadIdx.x == 0) {
-                *sh.mcnt = 0;
-                *sh.lcnt = 0;
+            const uint32_t end = e - 32 + __popc(in), len = end - h;
+            for (uint32_t i = h + lane; i < end; i += 32) {
+                const uint32_t v = (uint32_t)a[i];
+                q.slot_info[(v >> kSlotBits) * q.R + (v & kSlotMask)] = len == 1 ? kSingleBit : pbase + i;
             }
-            __syncthreads();
-            if (lane == 0 && n_m) atomicAdd(sh.mcnt, n_m);
-            if (lane == 0 && n_l) atomicAdd(sh.lcnt, n_l);
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                *sh.mbase = *sh.mcnt ? atomicAdd(q.mcount + b, *sh.mcnt) : 0u;
-                *sh.lbase = *sh.lcnt ? atomicAdd(q.lcount + b, *sh.lcnt) : 0u;
-                *sh.mcnt = 0;
-                *sh.lcnt = 0;
-            }
-            __syncthreads();
+            list_segments(q, b, lane == 0, pbase + h, len, hv, z);
+            h = end;
         }
     }
 }
 
-__global__ void __launch_bounds__(kGroupThreads) k_group_cluster(GroupParams q, int log_parts) {
-    extern __shared__ uint64_t gkeys[];                      // kGroupCap keys
-    __shared__ uint32_t s_cnt[1 << kGroupMaxLog][kSub];      // this slice: keys per (part, sub-bucket)
-    __shared__ uint32_t s_pre[1 << kGroupMaxLog][kSub];      // keys of (part, sub) in lower ranks' slices
-    __shared__ uint32_t s_off[1 << kGroupMaxLog][kSub];      // where this slice's next key of (part, sub) goes
-    __shared__ uint32_t s_start[kSub + 1];                   // my part's sub-bucket starts
-    __shared__ uint32_t s_tot[1 << kGroupMaxLog];            // keys per part
-    __shared__ uint32_t s_big[kSub];                         // sub-buckets too large for one thread
-    __shared__ uint32_t s_nbig, s_mcnt, s_lcnt, s_mbase, s_lbase;
-    cg::cluster_group cl = cg::this_cluster();
-    const uint32_t P = 1u << log_parts, me = cl.block_rank();
-    const int b = blockIdx.y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(kPartThreads) k_group_parts(GroupParams q, int log_parts) {
+    extern __shared__ uint64_t gkeys[];  // kPartCap keys
+    __shared__ uint32_t once[1u << (kMapBits - 5)], twice[1u << (kMapBits - 5)];
+    __shared__ uint32_t cnt[kPartSub];        // keys per sub-bucket, then the next key's place
+    __shared__ uint32_t start[kPartSub + 1];  // sub-bucket starts
+    __shared__ uint32_t wtot[32];
+    __shared__ uint16_t big[kPartSub];
+    __shared__ uint32_t nbig, pbase;
+    constexpr int U = 8;  // record entries per thread loaded at once
+    const uint32_t me = blockIdx.x, tid = threadIdx.x;
+    const int b = blockIdx.y, lane = tid & 31, warp = tid >> 5;
     uint64_t base;
     uint32_t n;
     batch_range(q, b, &base, &n);
-    for (uint32_t i = threadIdx.x; i < P * kSub; i += blockDim.x) (&s_cnt[0][0])[i] = 0;
-    if (threadIdx.x == 0) s_nbig = 0;
+    const int32_t* rec = q.rec + base;
+    const uint32_t s_base = (uint32_t)((int64_t)b * q.batch);
+    for (uint32_t i = tid; i < 1u << (kMapBits - 5); i += kPartThreads) once[i] = twice[i] = 0u;
+    cnt[tid] = 0;
+    if (tid == 0) nbig = 0;
     __syncthreads();
-    const uint32_t per = (n + P - 1) / P;
-    const uint32_t lo = min(n, me * per), hi = min(n, lo + per);
-    const int sub_shift = 24 - log_parts;
-    // pass 1: counts of this slice
-    for (uint32_t r = lo; r < hi; r += kGroupThreads * kGroupPerThread) {
-        uint64_t it[kGroupPerThread];
+    // f(entry index, sample within the batch, slot, hrow) for each of the part's entries
+    auto each = [&](auto&& f) {
+        for (uint32_t r = tid; r < n; r += kPartThreads * U) {
+            int32_t row[U];
 #pragma unroll
-        for (int k = 0; k < kGroupPerThread; ++k) {
-            const uint32_t i = r + k * kGroupThreads + threadIdx.x;
-            it[k] = i < hi ? q.items[base + i] : 0ull;
-        }
+            for (int k = 0; k < U; ++k) {
+                const uint32_t i = r + k * kPartThreads;
+                row[k] = i < n ? __ldg(rec + i) : 0;
+            }
 #pragma unroll
-        for (int k = 0; k < kGroupPerThread; ++k) {
-            const uint32_t i = r + k * kGroupThreads + threadIdx.x;
-            if (i < hi) {
-                const uint32_t hv = hrow((uint32_t)(it[k] >> 32));
-                const uint32_t pt = log_parts ? hv >> (32 - log_parts) : 0u;
-                atomicAdd(&s_cnt[pt][(hv >> sub_shift) & (kSub - 1)], 1u);
-                if (q.depmap) {
-                    const uint32_t db = hv >> (32 - kDepLog);
-                    atomicOr(q.depmap + (size_t)b * kDepWords + (db >> 5), 1u << (db & 31u));
-                }
+            for (int k = 0; k < U; ++k) {
+                const uint32_t i = r + k * kPartThreads;
+                const uint32_t smp = __umulhi(i, q.R_magic), slot = i - smp * q.R;
+                const uint32_t hv = hrow((uint32_t)row[k] + (slot ? q.ctx_off : 0u));
+                if (i < n && (log_parts == 0 || hv >> (32 - log_parts) == me)) f(i, smp, slot, hv);
             }
         }
-    }
-    cl.sync();
-    // every (part, sub-bucket): total over the cluster, and the keys of lower
-    // ranks (which go first); then per part the sub-bucket starts
-    for (uint32_t e = threadIdx.x; e < P * kSub; e += blockDim.x) {
-        uint32_t c[1 << kGroupMaxLog];
-#pragma unroll
-        for (uint32_t rk = 0; rk < (1u << kGroupMaxLog); ++rk)  // all loads in flight at once
-            c[rk] = rk < P ? cl.map_shared_rank(&s_cnt[0][0], rk)[e] : 0u;
-        uint32_t tot = 0, before = 0;
-#pragma unroll
-        for (uint32_t rk = 0; rk < (1u << kGroupMaxLog); ++rk) {
-            if (rk < me) before += c[rk];
-            tot += c[rk];
+    };
+    each([&](uint32_t, uint32_t, uint32_t, uint32_t hv) {
+        const uint32_t h = (hv << log_parts) >> (32 - kMapBits), bit = 1u << (h & 31u);
+        if (atomicOr(&once[h >> 5], bit) & bit) atomicOr(&twice[h >> 5], bit);
+        if (q.depmap) {
+            const uint32_t db = hv >> (32 - kDepLog);
+            atomicOr(q.depmap + (size_t)b * kDepWords + (db >> 5), 1u << (db & 31u));
         }
-        (&s_off[0][0])[e] = tot;  // totals for now
-        (&s_pre[0][0])[e] = before;
-    }
+    });
     __syncthreads();
-    if (warp < (int)P) {
-        // exclusive scan of part `warp`'s sub-bucket totals: lane l owns 8
-        uint32_t v[kSub / 32], own = 0;
-#pragma unroll
-        for (int k = 0; k < kSub / 32; ++k) own += (v[k] = s_off[warp][lane * (kSub / 32) + k]);
-        uint32_t incl = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += x;
-        }
-        uint32_t run = incl - own;
-#pragma unroll
-        for (int k = 0; k < kSub / 32; ++k) {
-            const int sb = lane * (kSub / 32) + k;
-            if (warp == (int)me) s_start[sb] = run;
-            s_off[warp][sb] = run + s_pre[warp][sb];
-            run += v[k];
-        }
-        if (lane == 31) {
-            s_tot[warp] = run;
-            if (warp == (int)me) s_start[kSub] = run;
-        }
-    }
+    each([&](uint32_t i, uint32_t, uint32_t, uint32_t hv) {
+        const uint32_t h = (hv << log_parts) >> (32 - kMapBits);
+        if (twice[h >> 5] >> (h & 31u) & 1u) atomicAdd(&cnt[(hv << log_parts) >> (32 - 10)], 1u);
+        else q.slot_info[base + i] = kSingleBit;
+    });
     __syncthreads();
-    uint32_t qbase = 0, pbase[1 << kGroupMaxLog];
-    bool fits[1 << kGroupMaxLog];
-    for (uint32_t p2 = 0, run = 0; p2 < P; ++p2) {
-        pbase[p2] = run;
-        if (p2 == me) qbase = run;
-        fits[p2] = s_tot[p2] <= kGroupCap;
-        run += s_tot[p2];
-    }
-    const uint32_t nq = s_tot[me];
-    // pass 2: send every key to its place (a part too large for shared memory
-    // - a very skewed draw - uses its own range of the scratch array)
-    for (uint32_t r = lo; r < hi; r += kGroupThreads * kGroupPerThread) {
-        uint64_t it[kGroupPerThread];
+    // exclusive scan of the 1,024 counts
+    const uint32_t own = cnt[tid];
+    uint32_t incl = own;
 #pragma unroll
-        for (int k = 0; k < kGroupPerThread; ++k) {
-            const uint32_t i = r + k * kGroupThreads + threadIdx.x;
-            it[k] = i < hi ? q.items[base + i] : 0ull;
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) wtot[warp] = incl;
+    __syncthreads();
+    uint32_t wsum = lane < warp ? wtot[lane] : 0u;
 #pragma unroll
-        for (int k = 0; k < kGroupPerThread; ++k) {
-            const uint32_t i = r + k * kGroupThreads + threadIdx.x;
-            if (i < hi) {
-                const uint32_t hv = hrow((uint32_t)(it[k] >> 32));
-                const uint32_t pt = log_parts ? hv >> (32 - log_parts) : 0u;
-                const uint32_t at = atomicAdd(&s_off[pt][(hv >> sub_shift) & (kSub - 1)], 1u);
-                uint64_t* dst = fits[pt] ? cl.map_shared_rank(gkeys, pt) : q.bucketed + base + pbase[pt];
-                dst[at] = ((uint64_t)hv << 32) | (uint32_t)it[k];
-            }
+    for (int o = 16; o >= 1; o >>= 1) wsum += __shfl_xor_sync(0xFFFFFFFFu, wsum, o);
+    start[tid] = cnt[tid] = wsum + incl - own;
+    if (tid == kPartThreads - 1) {
+        start[kPartSub] = wsum + incl;
+        pbase = atomicAdd(q.pcount + b, wsum + incl);
+    }
+    if (own > kRankMax) big[atomicAdd(&nbig, 1u)] = (uint16_t)tid;
+    __syncthreads();
+    const uint32_t nc = start[kPartSub];
+    const bool fits = nc <= kPartCap;
+    uint64_t* far = q.bucketed + base + pbase;  // a part too large for shared memory (a very skewed draw)
+    each([&](uint32_t, uint32_t smp, uint32_t slot, uint32_t hv) {
+        const uint32_t h = (hv << log_parts) >> (32 - kMapBits);
+        if (twice[h >> 5] >> (h & 31u) & 1u) {
+            const uint32_t at = atomicAdd(&cnt[(hv << log_parts) >> (32 - 10)], 1u);
+            const uint64_t key = ((uint64_t)hv << 32) | ((s_base + smp) << kSlotBits | slot);
+            if (fits) gkeys[at] = key;
+            else far[at] = key;
         }
-    }
-    cl.sync();
-    const GroupShared sh{s_start, s_big, &s_nbig, &s_mcnt, &s_lcnt, &s_mbase, &s_lbase};
-    if (fits[me]) group_tail(q, gkeys, nq, n, qbase, b, me, P, log_parts, sh);
-    else group_tail(q, q.bucketed + base + qbase, nq, n, qbase, b, me, P, log_parts, sh);
-}
-
-// eta[b] = lr0 (schedule 0) or lr0 * max(1 - t0/T, floor) (schedule 1) for
-// the batch starting at global sample t0 = t_chunk + b * batch, in FP32:
-// 1 - t0/T as (T - t0) / T from the exact integer difference.
-__global__ void k_batch_eta(int n_batches, uint64_t t_chunk, int64_t batch, float lr0, int schedule, float floor_frac,
-                            uint64_t total, float* __restrict__ eta) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= n_batches) return;
-    float f = 1.0f;
-    if (schedule == 1) {
-        const uint64_t t0 = t_chunk + (uint64_t)b * (uint64_t)batch;
-        f = t0 >= total ? 0.0f : (float)(total - t0) / (float)total;
-        if (f < floor_frac) f = floor_frac;
-    }
-    eta[b] = lr0 * f;
+    });
+    __syncthreads();
+    if (fits) group_segments(q, gkeys, gkeys, nc, start, log_parts, pbase, b, big, nbig);
+    else group_segments(q, far, far, nc, start, log_parts, pbase, b, big, nbig);
 }
 
 // ---------------------------------------------------------------------------
@@ -1695,7 +1628,7 @@ struct ChunkSet {
 };
 
 struct TrainWorkspace {
-    Buf items0, items1, gcnt, boff, counters, slab, gbar;
+    Buf items0, items1, gcnt, boff, pcount, counters, slab, gbar;
     ChunkSet set[2];
     cudaStream_t prep = nullptr;    // pre-pass stream
     cudaStream_t cap = nullptr;     // stream the data-phase graphs are captured on
@@ -1799,6 +1732,7 @@ static cudaError_t launch_data_batched(const DataParams& p, int warps_per_block,
     size_t smem = 0;
     // 4 warps per block: at ~70 registers a 4096-sample batch is one wave
     const int wpb = gather_warps<D, DT>(p, warps_per_block, kGatherWarps, &smem, kGatherWarps);
+    if (G::E <= 4 && p.K < 8) smem = 0;  // the register body stages nothing
     static std::atomic<uint64_t> attr_set{0};
     once_per_device(attr_set, [] {
         cudaFuncSetAttribute(k_gather<D, DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
@@ -1917,12 +1851,12 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     const int64_t max_chunk = nb * a.batch;
     const int64_t max_items = max_chunk * R;
     const uint32_t parts = (uint32_t)((a.batch * R + kPartItems - 1) / kPartItems);
-    // batches of up to 8 parts of ~3.5K items are grouped by one cluster in
-    // distributed shared memory; larger ones are bucketed through global
-    // memory first
+    // batches of up to 16 parts of 16,384 items are grouped part by part in
+    // shared memory (every part scans the whole batch); larger ones are
+    // bucketed through global memory first
     int log_parts = 0;
-    while (a.batch * R > ((int64_t)3584 << log_parts)) ++log_parts;
-    const bool direct = log_parts <= kGroupMaxLog;
+    while (a.batch * R > ((int64_t)kPartItems2 << log_parts)) ++log_parts;
+    const bool direct = log_parts <= kPartMaxLog;
     // the persistent schedule needs all its CTAs resident at once, which a
     // second cooperative launch on the other order's stream could prevent:
     // concurrent orders run the batched schedule
@@ -1951,14 +1885,17 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
                 if (!f(cs.rec, sizeof(int32_t) * max_items) || !f(cs.tchunk, 256)) return false;
             return true;
         }
-        if (!f(ws->items0, sizeof(uint64_t) * max_items) || !f(ws->items1, sizeof(uint64_t) * max_items) ||
-            !f(ws->gcnt, sizeof(uint32_t) * (size_t)nb * parts * kBuckets) ||
-            !f(ws->boff, sizeof(uint32_t) * (size_t)nb * (kBuckets + 1)) || !f(ws->counters, 256) ||
+        if (!f(ws->items1, sizeof(uint64_t) * max_items) || !f(ws->counters, 256) ||
+            !f(ws->pcount, sizeof(uint32_t) * (nb + 1)) ||
             !f(ws->slab, sizeof(float) * (size_t)std::min<int64_t>(max_items, a.batch * R) * a.dim))
+            return false;
+        if (!direct && (!f(ws->items0, sizeof(uint64_t) * max_items) ||
+                        !f(ws->gcnt, sizeof(uint32_t) * (size_t)nb * parts * kBuckets) ||
+                        !f(ws->boff, sizeof(uint32_t) * (size_t)nb * (kBuckets + 1))))
             return false;
         for (auto& cs : ws->set) {
             if (!f(cs.rec, sizeof(int32_t) * max_items) || !f(cs.eta, sizeof(float) * (nb + 1)) ||
-                !f(cs.slot_info, sizeof(uint2) * max_items) || !f(cs.mdesc, sizeof(uint4) * (size_t)nb * mcap) ||
+                !f(cs.slot_info, sizeof(uint32_t) * max_items) || !f(cs.mdesc, sizeof(uint4) * (size_t)nb * mcap) ||
                 !f(cs.mcount, sizeof(uint32_t) * (nb + 1)) || !f(cs.ldesc, sizeof(uint4) * (size_t)nb * lcap) ||
                 !f(cs.lcount, sizeof(uint32_t) * (nb + 1)) || !f(cs.tchunk, 256))
                 return false;
@@ -1987,10 +1924,10 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
         return cudaErrorInvalidValue;
     }
     const size_t sort_smem = (size_t)kSortBucketsPerCta * 2 * kWarpSortCap * sizeof(uint64_t);
-    const size_t group_smem = (size_t)kGroupCap * sizeof(uint64_t);
+    const size_t group_smem = (size_t)kPartCap * sizeof(uint64_t);
     if ((e = cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem)) !=
             cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_group_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)group_smem)) !=
+        (e = cudaFuncSetAttribute(k_group_parts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)group_smem)) !=
             cudaSuccess)
         return e;
     cudaStream_t ps = ws->prep;
@@ -2010,7 +1947,11 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     pp.K = a.K;
     pp.order = a.order;
     pp.walk = a.walk_len > 0;
-    pp.items = hogwild ? nullptr : (uint64_t*)ws->items0.p;
+    pp.lr0 = (float)a.lr0;
+    pp.lr_floor = (float)a.lr_floor;
+    pp.lr_schedule = a.lr_schedule;
+    pp.lr_total = a.lr_total;
+    pp.pcount = (uint32_t*)ws->pcount.p;
 
     WalkParams wp{};
     if (a.walk_len > 0) {
@@ -2026,9 +1967,6 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
         wp.P = (uint64_t)a.walk_len * a.window - (uint64_t)a.window * (a.window - 1) / 2;
         wp.reuse = (uint32_t)a.walk_reuse;
         wp.R = (uint64_t)R;
-        wp.items = hogwild ? nullptr : (uint64_t*)ws->items0.p;
-        wp.ctx_off = a.order == 2 ? (uint32_t)a.n_nodes : 0u;
-        wp.slot_bits = kSlotBits;
     }
 
     GroupParams gq{};
@@ -2037,9 +1975,11 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     gq.K = (uint32_t)a.K;
     gq.parts = parts;
     gq.row_bits = row_bits;
-    gq.items = (const uint64_t*)ws->items0.p;
+    gq.R_magic = (uint32_t)(((uint64_t)1 << 32) / (uint32_t)R) + 1u;
+    gq.ctx_off = a.order == 2 ? (uint32_t)a.n_nodes : 0u;
     gq.bucketed = (uint64_t*)ws->items1.p;
-    gq.tmp = (uint64_t*)ws->items0.p;  // the draws are consumed by the bucketing before the sort
+    gq.tmp = (uint64_t*)ws->items0.p;
+    gq.pcount = (uint32_t*)ws->pcount.p;
     gq.gcnt = (uint32_t*)ws->gcnt.p;
     gq.boff = (uint32_t*)ws->boff.p;
     gq.mcap = mcap;
@@ -2091,6 +2031,12 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
         pp.chunk_samples = cs;
         pp.rec = (int32_t*)cset.rec.p;
         pp.t_out = (uint64_t*)cset.tchunk.p;
+        if (!hogwild) {
+            pp.n_batches = cb;
+            pp.eta = (float*)cset.eta.p;
+            pp.mcount = (uint32_t*)cset.mcount.p;
+            pp.lcount = (uint32_t*)cset.lcount.p;
+        }
         {
             const int64_t work = cs * (a.K + 1);
             const unsigned g = (unsigned)std::min<int64_t>((work + 255) / 256, 152 * 64);
@@ -2102,45 +2048,28 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
                 if ((e = walk_pairs(wp, ps)) != cudaSuccess) return e;
                 ++launches;
             }
-            if (!hogwild)
-                k_batch_eta<<<(unsigned)((cb + 127) / 128), 128, 0, ps>>>(cb, t, a.batch, (float)a.lr0, a.lr_schedule,
-                                                                          (float)a.lr_floor, a.lr_total,
-                                                                          (float*)cset.eta.p);
         }
         if (!hogwild) {
             gq.n_batches = cb;
             gq.chunk_samples = cs;
-            gq.slot_info = (uint2*)cset.slot_info.p;
+            gq.rec = (const int32_t*)cset.rec.p;
+            gq.slot_info = (uint32_t*)cset.slot_info.p;
             gq.mdesc = (uint4*)cset.mdesc.p;
             gq.mcount = (uint32_t*)cset.mcount.p;
             gq.ldesc = (uint4*)cset.ldesc.p;
             gq.lcount = (uint32_t*)cset.lcount.p;
             gq.depmap = persistent ? (uint32_t*)cset.depmap.p : nullptr;
-            if ((e = cudaMemsetAsync(cset.mcount.p, 0, sizeof(uint32_t) * (cb + 1), ps)) != cudaSuccess) return e;
-            if ((e = cudaMemsetAsync(cset.lcount.p, 0, sizeof(uint32_t) * (cb + 1), ps)) != cudaSuccess) return e;
             if (persistent &&
                 (e = cudaMemsetAsync(cset.depmap.p, 0, sizeof(uint32_t) * (size_t)cb * kDepWords, ps)) != cudaSuccess)
                 return e;
             if (direct) {
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(1u << log_parts, cb);
-                cfg.blockDim = dim3(kGroupThreads);
-                cfg.dynamicSmemBytes = group_smem;
-                cfg.stream = ps;
-                cudaLaunchAttribute attr[1];
-                attr[0].id = cudaLaunchAttributeClusterDimension;
-                attr[0].val.clusterDim.x = 1u << log_parts;
-                attr[0].val.clusterDim.y = 1;
-                attr[0].val.clusterDim.z = 1;
-                cfg.attrs = attr;
-                cfg.numAttrs = 1;
-                if ((e = cudaLaunchKernelEx(&cfg, k_group_cluster, gq, log_parts)) != cudaSuccess) return e;
-                launches += 3;
+                k_group_parts<<<dim3(1u << log_parts, cb), kPartThreads, group_smem, ps>>>(gq, log_parts);
+                launches += 2;
             } else {
                 k_bucket_count<<<dim3(parts, cb), kBucketThreads, 0, ps>>>(gq);
                 k_bucket_scatter<<<dim3(parts, cb), kBucketThreads, 0, ps>>>(gq);
                 k_bucket_sort<<<dim3(kBuckets / kSortBucketsPerCta, cb), kSortThreads, sort_smem, ps>>>(gq);
-                launches += 5;
+                launches += 4;
             }
         } else {
             launches += 1;  // the draws alone
@@ -2179,7 +2108,7 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
             if ((e = hogwild_chunk(hp, a.dim, a.dtype, a.hogwild_workers, s)) != cudaSuccess) return e;
         } else {
             dp.rec = (const int32_t*)cset.rec.p;
-            dp.slot_info = (const uint2*)cset.slot_info.p;
+            dp.slot_info = (const uint32_t*)cset.slot_info.p;
             dp.mdesc = (const uint4*)cset.mdesc.p;
             dp.mcount = (const uint32_t*)cset.mcount.p;
             dp.ldesc = (const uint4*)cset.ldesc.p;

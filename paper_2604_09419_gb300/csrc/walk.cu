@@ -150,11 +150,6 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_walk_pairs(WalkParams p) {
             const uint64_t s = t - p.t0;
             p.rec[s * p.R] = u;
             p.rec[s * p.R + 1] = v;
-            if (p.items) {
-                const uint64_t lowbits = (uint32_t)s << p.slot_bits;  // s < 2^26 within a chunk
-                p.items[s * p.R] = ((uint64_t)(uint32_t)u << 32) | lowbits;
-                p.items[s * p.R + 1] = ((uint64_t)((uint32_t)v + p.ctx_off) << 32) | lowbits | 1u;
-            }
         }
         __syncwarp();  // the nodes are rewritten by the warp's next walk
     }
