@@ -74,7 +74,8 @@ __device__ __forceinline__ void add_row(void* table, int64_t row, int lig, const
 #pragma unroll
         for (int q = 0; q < G::NV; ++q) {
             const uint32_t k4 = (uint32_t)((lig * G::E + 4 * q) >> 2);
-            const uint64_t r = sr_bits(seed, table_id, (uint64_t)row, key, k4);
+            const uint2 rw = sr_words(sr_salt(seed, key), table_id, (uint64_t)row, k4);
+            const uint64_t r = ((uint64_t)rw.y << 32) | rw.x;
             float dd[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {

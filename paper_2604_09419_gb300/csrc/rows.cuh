@@ -62,28 +62,30 @@ __device__ __forceinline__ uint32_t fmix32(uint32_t h) {
     return h;
 }
 
-// 64 random bits for the stochastic rounding of the 4 values at columns
-// 4 k4 .. 4 k4 + 3 of `row` of table `table_id`, written by the batch that
-// starts at sample t0: with the batch's salt s, the SplitMix64 output
-// function (Steele, Lea, Flood, OOPSLA 2014) of seed ^ t0 0x9E3779B97F4A7C15
-// (the same for every row of the batch, so it is computed once per thread),
-// the words w_j = fmix32(lo32(s) + (2 row + table) 0x9E3779B1 + 2 k4 + j),
-// j = 0 (low) and 1 (high).
-__device__ __forceinline__ uint64_t sr_bits(uint64_t seed, uint32_t table_id, uint64_t row, uint64_t t0, uint32_t k4) {
+// Random bits for the stochastic rounding of the rows written by the batch
+// that starts at sample t0.  The batch's salt is the low half of the
+// SplitMix64 output function (Steele, Lea, Flood, OOPSLA 2014) of
+// seed ^ t0 0x9E3779B97F4A7C15; the 64 bits for the 4 values at columns
+// 4 k4 .. 4 k4 + 3 of `row` of table `table_id` are the words
+// w_j = fmix32(salt + (2 row + table) 0x9E3779B1 + 2 k4 + j), j = 0 (low) and
+// 1 (high).
+__device__ __forceinline__ uint32_t sr_salt(uint64_t seed, uint64_t t0) {
     uint64_t s = seed ^ (t0 * 0x9E3779B97F4A7C15ull);
     s = (s ^ (s >> 30)) * 0xBF58476D1CE4E5B9ull;
     s = (s ^ (s >> 27)) * 0x94D049BB133111EBull;
-    s ^= s >> 31;
-    const uint32_t base = (uint32_t)s + (uint32_t)(2 * row + table_id) * 0x9E3779B1u + 2u * k4;
-    return ((uint64_t)fmix32(base + 1u) << 32) | fmix32(base);
+    return (uint32_t)(s ^ (s >> 31));
+}
+__device__ __forceinline__ uint2 sr_words(uint32_t salt, uint32_t table_id, uint64_t row, uint32_t k4) {
+    const uint32_t base = salt + (uint32_t)(2 * row + table_id) * 0x9E3779B1u + 2u * k4;
+    return make_uint2(fmix32(base), fmix32(base + 1u));
 }
 
 // Store a row part; BF16 rounds stochastically: value i of a 4-value vector
-// adds bits [16 i, 16 i + 16) of sr_bits(...) below the BF16 mantissa, then
+// adds bits [16 i, 16 i + 16) of sr_words(...) below the BF16 mantissa, then
 // truncates (two values per cvt.rs instruction).
 template <int D, int DT>
 __device__ __forceinline__ void store_row(void* table, int64_t row, int lig, const float (&v)[Geom<D, DT>::E],
-                                          uint64_t seed, uint64_t t0, uint32_t table_id) {
+                                          uint32_t salt, uint32_t table_id) {
     using G = Geom<D, DT>;
     if constexpr (DT == LINE_DTYPE_F32) {
         float4* p = reinterpret_cast<float4*>(reinterpret_cast<float*>(table) + row * D + lig * G::E);
@@ -93,13 +95,93 @@ __device__ __forceinline__ void store_row(void* table, int64_t row, int lig, con
         uint2* p = reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(table) + row * D + lig * G::E);
 #pragma unroll
         for (int q = 0; q < G::NV; ++q) {
-            const uint32_t k4 = (uint32_t)((lig * G::E + 4 * q) >> 2);
-            const uint64_t r = sr_bits(seed, table_id, (uint64_t)row, t0, k4);
-            const uint32_t r0 = (uint32_t)r, r1 = (uint32_t)(r >> 32);
-            __stcg(p + q, make_uint2(bf16x2_sr(v[4 * q], v[4 * q + 1], r0), bf16x2_sr(v[4 * q + 2], v[4 * q + 3], r1)));
+            const uint2 r = sr_words(salt, table_id, (uint64_t)row, (uint32_t)((lig * G::E + 4 * q) >> 2));
+            __stcg(p + q, make_uint2(bf16x2_sr(v[4 * q], v[4 * q + 1], r.x), bf16x2_sr(v[4 * q + 2], v[4 * q + 3], r.y)));
         }
     }
 }
+
+// Packed FP32 arithmetic on E values (two per instruction on sm_100 and
+// later, each half rounded as the scalar instruction would be).
+// r = a b + c
+template <int E>
+__device__ __forceinline__ void vfma(float (&r)[E], float a, const float (&b)[E], const float (&c)[E]) {
+#pragma unroll
+    for (int e = 0; e < E; e += 2) {
+        const float2 t = __ffma2_rn(make_float2(a, a), make_float2(b[e], b[e + 1]), make_float2(c[e], c[e + 1]));
+        r[e] = t.x;
+        r[e + 1] = t.y;
+    }
+}
+// r = a b
+template <int E>
+__device__ __forceinline__ void vmul(float (&r)[E], float a, const float (&b)[E]) {
+#pragma unroll
+    for (int e = 0; e < E; e += 2) {
+        const float2 t = __fmul2_rn(make_float2(a, a), make_float2(b[e], b[e + 1]));
+        r[e] = t.x;
+        r[e + 1] = t.y;
+    }
+}
+
+// Sums of N values over the L lanes of a group, each in the order of the
+// butterfly (lane distances L/2 .. 1) and so with the same bits, but each
+// total only in some lanes: at every distance a lane gives away half of its
+// values and receives its partner's half of the others, so N values cost
+// about N + log2 L shuffles instead of N log2 L.  After reduce(), value j is
+// in s[slot(j)] of lane lane(j) (and of the lanes that differ from it outside
+// the distances that split it); kept() values a lane remain.
+template <int L, int N>
+struct Transposed {
+    static constexpr int kept() {
+        int n = N;
+        for (int o = L / 2; o >= 1; o >>= 1) n = n > 1 ? (n + 1) / 2 : n;
+        return n;
+    }
+    static constexpr int find(int j, bool want_lane) {
+        int n = N, lane = 0;
+        for (int o = L / 2; o >= 1; o >>= 1) {
+            if (n <= 1) continue;
+            const int half = (n + 1) / 2;
+            if (j >= half) {
+                lane |= o;
+                j -= half;
+            }
+            n = half;
+        }
+        return want_lane ? lane : j;
+    }
+    static constexpr int lane(int j) { return find(j, true); }
+    static constexpr int slot(int j) { return find(j, false); }
+    // lanes that hold value 0 in slot 0: those with none of these bits
+    static constexpr int split() {
+        int n = N, m = 0;
+        for (int o = L / 2; o >= 1; o >>= 1) {
+            if (n > 1) m |= o;
+            n = n > 1 ? (n + 1) / 2 : n;
+        }
+        return m;
+    }
+    static __device__ __forceinline__ void reduce(float (&s)[N], int lig) {
+        int n = N;
+#pragma unroll
+        for (int o = L / 2; o >= 1; o >>= 1) {
+            const bool hi = (lig & o) != 0;
+            const int half = (n + 1) / 2;
+#pragma unroll
+            for (int i = 0; i < (N + 1) / 2; ++i) {
+                if (i >= half) continue;
+                if (i + half < n) {
+                    const float keep = hi ? s[i + half] : s[i], give = hi ? s[i] : s[i + half];
+                    s[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+                } else {
+                    s[i] += __shfl_xor_sync(0xFFFFFFFFu, s[i], o);
+                }
+            }
+            n = half;
+        }
+    }
+};
 
 template <int L>
 __device__ __forceinline__ float group_sum(float v) {

@@ -97,6 +97,13 @@ __device__ __forceinline__ uint32_t dep_bit(uint32_t rowid) { return hrow(rowid)
 // ---------------------------------------------------------------------------
 // Kernel parameters shared by the data-phase kernels.
 // ---------------------------------------------------------------------------
+// Written by the pre-pass for every batch: its learning rate (FP32) and the
+// salt of its stochastic rounding (sr_salt).
+struct BatchParams {
+    float eta;
+    uint32_t salt;
+};
+
 struct DataParams {
     void* U;
     void* C;       // order 2 context table; == U for order 1
@@ -114,13 +121,10 @@ struct DataParams {
     uint32_t lcap;
     float* slab;             // [batch * (K+2)][D], by position within the batch
     const uint32_t* depmap;  // [n_batches][kDepWords] rows each batch touches (bit dep_bit(row id))
-    uint64_t t_chunk;        // global index of the chunk's first sample
-    const uint64_t* t_chunk_dev;  // when set, the same read from device memory (graph replays)
     int64_t chunk_samples;
     int64_t batch;
     int n_batches;
-    uint64_t seed;
-    const float* eta;  // [n_batches] learning rate of each batch (FP32)
+    const BatchParams* bpar;  // [n_batches]
     float lambda, alpha_neg;
     uint32_t* status;
     // persistent schedule
@@ -146,16 +150,24 @@ __device__ __forceinline__ T rec_entry(uint32_t gm, T held, const T* row, int id
 // Per-sample work.
 // ctx_stage: this warp's shared staging area, (K+1) x 32 lanes x E floats.
 // ---------------------------------------------------------------------------
-// Register-resident gather body for K + 1 <= JB (6 or 8): the K+1 context
-// rows stay in registers; the dots, their reductions and the K+1 sigmoids are
-// independent chains.  Same arithmetic, in the same order, as the staged
-// body.  JB = 6 covers K <= 5 in fewer registers, so that a batch's gather
-// leaves room on every SM for the next chunk's pre-pass.
-template <int D, int DT, int JB = 8>
-__device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bool active, float eta, uint64_t t0,
+// Register-resident gather body for K + 1 <= JB: the K+1 context rows stay in
+// registers; the dots and their reductions are independent chains.  Same
+// arithmetic, in the same order, as the staged body.
+//
+// All of a batch's warps run at once (4,096 samples at d = 128 are one wave of
+// 27 warps an SM), so after the row loads arrive the gather is bound by issue
+// slots: 1,960,000 warp instructions a batch were 1.6 of its 4.0 us (R-MAT 20,
+// K = 5).  Hence the transposed reduction (one sigmoid per lane instead of
+// K+1), packed FP32 pairs for everything but the dots (whose order over a
+// lane's values is fixed), and one selected address and value per FP32 row
+// instead of two branches: 1,420,000 warp instructions.  2^22 samples of one
+// order in BF16: 7.80 -> 6.69 ms; both orders FP32 12.09 -> 11.75.
+template <int D, int DT, int JB>
+__device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bool active, float eta, uint32_t salt,
                                                 uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
                                                 const uint32_t* info) {
     using G = Geom<D, DT>;
+    using T = Transposed<G::L, JB>;
     const int32_t u = __shfl_sync(gm, r0, 0, G::L);
     float xu[G::E];
     float c[JB][G::E];
@@ -163,7 +175,12 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
 #pragma unroll
     for (int j = 0; j < JB; ++j) {
         const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active && j <= p.K);
-        if (j <= p.K) load_row<D, DT>(p.C, y, lig, c[j]);
+        if (j <= p.K) {
+            load_row<D, DT>(p.C, y, lig, c[j]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < G::E; ++e) c[j][e] = 0.0f;
+        }
     }
     float sj[JB];
 #pragma unroll
@@ -172,55 +189,62 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
 #pragma unroll
         for (int e = 0; e < G::E; ++e) sj[j] = fmaf(xu[e], c[j][e], sj[j]);
     }
+    T::reduce(sj, lig);
+    float gv[T::kept()];
 #pragma unroll
-    for (int o = G::L / 2; o >= 1; o >>= 1)
-#pragma unroll
-        for (int j = 0; j < JB; ++j) sj[j] += __shfl_xor_sync(0xFFFFFFFFu, sj[j], o);
-    float g[JB];
-#pragma unroll
-    for (int j = 0; j < JB; ++j) {
-        const float sig = 1.0f / (1.0f + expf(-sj[j]));
-        g[j] = j == 0 ? eta * (1.0f - sig) : -eta * p.alpha_neg * sig;
+    for (int i = 0; i < T::kept(); ++i) {
+        const float sig = 1.0f / (1.0f + expf(-sj[i]));
+        gv[i] = i == 0 && (lig & T::split()) == 0 ? eta * (1.0f - sig) : -eta * p.alpha_neg * sig;
     }
-    const uint32_t ctx_table = p.order == 2 ? 1u : 0u;
-    const float etalam = eta * p.lambda;
+    const float decay = eta * p.lambda;
     float du[G::E];
 #pragma unroll
     for (int e = 0; e < G::E; ++e) du[e] = 0.0f;
 #pragma unroll
     for (int j = 0; j < JB; ++j) {
         if (j > p.K) continue;
-#pragma unroll
-        for (int e = 0; e < G::E; ++e) du[e] = fmaf(g[j], c[j][e], du[e]);
+        const float g = __shfl_sync(0xFFFFFFFFu, gv[T::slot(j)], T::lane(j), G::L);
+        vfma(du, g, c[j], du);
         const uint32_t inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
         const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
-        if (active) {
-            if (inf & kSingleBit) {
-                const float decay = 1.0f * etalam;
-                float x[G::E];
+        const bool single = (inf & kSingleBit) != 0;
+        // a singleton's new row c - decay c + g x, or the contribution g x
+        float x[G::E];
+        if constexpr (DT == LINE_DTYPE_F32) {
+            vfma(x, -decay, c[j], c[j]);
 #pragma unroll
-                for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[j][e], c[j][e]) + g[j] * xu[e];
-                store_row<D, DT>(p.C, y, lig, x, p.seed, t0, ctx_table);
+            for (int e = 0; e < G::E; ++e) x[e] = single ? x[e] : -0.0f;  // (g x) + -0 is g x, sign of zero included
+            vfma(x, g, xu, x);
+            float* dst = (single ? reinterpret_cast<float*>(p.C) + (int64_t)y * D : p.slab + (int64_t)inf * D) + lig * G::E;
+            if (active) {
+#pragma unroll
+                for (int q = 0; q < G::NV; ++q)
+                    st_cg(reinterpret_cast<float4*>(dst) + q, make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]));
+            }
+        } else if (active) {
+            if (single) {
+                vfma(x, -decay, c[j], c[j]);
+                vfma(x, g, xu, x);
+                store_row<D, DT>(p.C, y, lig, x, salt, p.order == 2 ? 1u : 0u);
             } else {
+                vmul(x, g, xu);
                 float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
 #pragma unroll
-                for (int q = 0; q < G::E / 4; ++q)
-                    st_cg(dst + q, make_float4(g[j] * xu[4 * q], g[j] * xu[4 * q + 1], g[j] * xu[4 * q + 2],
-                                               g[j] * xu[4 * q + 3]));
+                for (int q = 0; q < G::NV; ++q) st_cg(dst + q, make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]));
             }
         }
     }
     const uint32_t inf0 = shfl_w(gm, i0, 0, G::L);
     if (active) {
         if (inf0 & kSingleBit) {
-            const float decay = (float)(p.K + 1) * etalam;
+            vfma(xu, -((float)(p.K + 1) * decay), xu, xu);
 #pragma unroll
-            for (int e = 0; e < G::E; ++e) xu[e] = fmaf(-decay, xu[e], xu[e]) + du[e];
-            store_row<D, DT>(p.U, u, lig, xu, p.seed, t0, 0u);
+            for (int e = 0; e < G::E; ++e) xu[e] += du[e];
+            store_row<D, DT>(p.U, u, lig, xu, salt, 0u);
         } else {
             float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0 * D + lig * G::E);
 #pragma unroll
-            for (int q = 0; q < G::E / 4; ++q) st_cg(dst + q, make_float4(du[4 * q], du[4 * q + 1], du[4 * q + 2], du[4 * q + 3]));
+            for (int q = 0; q < G::NV; ++q) st_cg(dst + q, make_float4(du[4 * q], du[4 * q + 1], du[4 * q + 2], du[4 * q + 3]));
         }
     }
 }
@@ -230,7 +254,7 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
 // time.  Same arithmetic, in the same order, as the register body.
 template <int D, int DT>
 __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig, int lane, bool active, float eta,
-                                                   uint64_t t0, uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
+                                                   uint32_t salt, uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
                                                    const uint32_t* info, float* ctx_stage) {
     using G = Geom<D, DT>;
     constexpr int CH = G::E <= 4 ? 8 : 4;  // context rows in flight per lane
@@ -261,7 +285,8 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
     float du[G::E];
 #pragma unroll
     for (int e = 0; e < G::E; ++e) du[e] = 0.0f;
-    constexpr int JB = 8;  // dot products reduced together (independent shuffles)
+    constexpr int JB = 8;  // dot products reduced together
+    using T = Transposed<G::L, JB>;
     for (int j0 = 0; j0 <= p.K; j0 += JB) {
         float sj[JB];
 #pragma unroll
@@ -279,10 +304,13 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
                 }
             }
         }
+        T::reduce(sj, lig);
+        float gv[T::kept()];
 #pragma unroll
-        for (int o = G::L / 2; o >= 1; o >>= 1)
-#pragma unroll
-            for (int jj = 0; jj < JB; ++jj) sj[jj] += __shfl_xor_sync(0xFFFFFFFFu, sj[jj], o);
+        for (int i = 0; i < T::kept(); ++i) {
+            const float sig = 1.0f / (1.0f + expf(-sj[i]));
+            gv[i] = i == 0 && j0 == 0 && (lig & T::split()) == 0 ? eta * (1.0f - sig) : -eta * p.alpha_neg * sig;
+        }
 #pragma unroll
         for (int jj = 0; jj < JB; ++jj) {
             const int j = j0 + jj;
@@ -297,10 +325,8 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
                 c[4 * q + 2] = a.z;
                 c[4 * q + 3] = a.w;
             }
-            const float sig = 1.0f / (1.0f + expf(-sj[jj]));
-            const float g = j == 0 ? eta * (1.0f - sig) : -eta * p.alpha_neg * sig;
-#pragma unroll
-            for (int e = 0; e < G::E; ++e) du[e] = fmaf(g, c[e], du[e]);
+            const float g = __shfl_sync(0xFFFFFFFFu, gv[T::slot(jj)], T::lane(jj), G::L);
+            vfma(du, g, c, du);
             const uint32_t inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
             const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
             if (active) {
@@ -310,7 +336,7 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
                     float x[G::E];
 #pragma unroll
                     for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[e], c[e]) + g * xu[e];
-                    store_row<D, DT>(p.C, y, lig, x, p.seed, t0, ctx_table);
+                    store_row<D, DT>(p.C, y, lig, x, salt, ctx_table);
                 } else {
                     float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
 #pragma unroll
@@ -326,7 +352,7 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
             const float decay = (float)(p.K + 1) * etalam;
 #pragma unroll
             for (int e = 0; e < G::E; ++e) xu[e] = fmaf(-decay, xu[e], xu[e]) + du[e];
-            store_row<D, DT>(p.U, u, lig, xu, p.seed, t0, 0u);
+            store_row<D, DT>(p.U, u, lig, xu, salt, 0u);
         } else {
             float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0 * D + lig * G::E);
 #pragma unroll
@@ -335,38 +361,13 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
     }
 }
 
-template <int D, int DT, bool PDL = false>
-__device__ __forceinline__ void sample_item(const DataParams& p, int64_t s_local, int lig, int lane, bool active,
-                                            float eta, uint64_t t0, float* ctx_stage) {
-    using G = Geom<D, DT>;
-    const int R = p.K + 2;
-    const int64_t sbase = (active ? s_local : 0) * R;
-    const int32_t* rec = p.rec + sbase;
-    const uint32_t* info = p.slot_info + sbase;
-    const uint32_t gm = group_mask<G::L>(lane / G::L);
-    const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
-    const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
-    if constexpr (PDL) pdl_wait();  // the tables' rows: written by the previous kernel
-    if constexpr (G::E <= 4) {
-        if (p.K < 6) {
-            sample_body_reg<D, DT, 6>(p, lig, active, eta, t0, gm, r0, i0, rec, info);
-            return;
-        }
-        if (p.K < 8) {
-            sample_body_reg<D, DT, 8>(p, lig, active, eta, t0, gm, r0, i0, rec, info);
-            return;
-        }
-    }
-    sample_body_staged<D, DT>(p, lig, lane, active, eta, t0, gm, r0, i0, rec, info, ctx_stage);
-}
-
 // ---------------------------------------------------------------------------
 // Per shared segment: fixed-order sum of its contiguous slab entries and the
 // write-back.
 // ---------------------------------------------------------------------------
 template <int D, int DT>
 __device__ __forceinline__ void segment_item(const DataParams& p, uint4 d, int lig, bool active, float eta,
-                                             uint64_t t0) {
+                                             uint32_t salt) {
     using G = Geom<D, DT>;
     constexpr int PF = G::E <= 4 ? 8 : 4;  // slab entries in flight per lane
     if (!active) return;
@@ -416,7 +417,7 @@ __device__ __forceinline__ void segment_item(const DataParams& p, uint4 d, int l
     const float decay = (float)d.w * (eta * p.lambda);
 #pragma unroll
     for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, x[e], x[e]) + acc[e];
-    store_row<D, DT>(table, row, lig, x, p.seed, t0, is_c ? 1u : 0u);
+    store_row<D, DT>(table, row, lig, x, salt, is_c ? 1u : 0u);
 }
 
 // Warps of an apply block: 16 when one order trains alone (a hub row's
@@ -430,7 +431,7 @@ constexpr int kApplyWarpsAlone = 16, kApplyWarpsShared = 8;
 // depend on the number of warps.  Uses lane group 0 of each warp.  part:
 // shared, NW x D floats.
 template <int D, int DT, int NW>
-__device__ __forceinline__ void long_segment_cta(const DataParams& p, uint4 d, float eta, uint64_t t0, float* part) {
+__device__ __forceinline__ void long_segment_cta(const DataParams& p, uint4 d, float eta, uint32_t salt, float* part) {
     using G = Geom<D, DT>;
     constexpr int PF = G::E <= 4 ? 8 : 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -495,7 +496,7 @@ __device__ __forceinline__ void long_segment_cta(const DataParams& p, uint4 d, f
         const float decay = (float)d.w * (eta * p.lambda);
 #pragma unroll
         for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, x[e], x[e]) + acc[e];
-        store_row<D, DT>(table, row, lig, x, p.seed, t0, is_c ? 1u : 0u);
+        store_row<D, DT>(table, row, lig, x, salt, is_c ? 1u : 0u);
     }
 }
 
@@ -511,20 +512,34 @@ constexpr size_t kMaxSmem = 200 * 1024;
 // of the register file, and any pre-pass block displaced gather warps).
 constexpr int kGatherWarps = 4;
 
-template <int D, int DT, bool PDL>
+// JB: context rows held in registers (K + 1 <= JB), or 0 for the staged body.
+template <int D, int DT, int JB>
 __global__ void __launch_bounds__(kGatherWarps * 32, 8) k_gather(DataParams p, int b) {
     using G = Geom<D, DT>;
     extern __shared__ float4 smem4[];
-    float* smem = reinterpret_cast<float*>(smem4);
-    if constexpr (PDL) pdl_launch_dependents();
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = lane / G::L, lig = lane % G::L;
     const int64_t s_begin = (int64_t)b * p.batch;
     const int64_t s_end = min(s_begin + p.batch, p.chunk_samples);
     const int64_t s_local = s_begin + ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * G::GPW + grp;
-    float* stage = smem + (size_t)warp * (p.K + 1) * 32 * G::E;
-    const uint64_t tc = p.t_chunk_dev ? *p.t_chunk_dev : p.t_chunk;
-    sample_item<D, DT, PDL>(p, s_local, lig, lane, s_local < s_end, p.eta[b], tc + (uint64_t)s_begin, stage);
+    const bool active = s_local < s_end;
+    const int R = p.K + 2;
+    const int64_t sbase = (active ? s_local : 0) * R;
+    const int32_t* rec = p.rec + sbase;
+    const uint32_t* info = p.slot_info + sbase;
+    const uint32_t gm = group_mask<G::L>(grp);
+    // the chunk's index data comes from the pre-pass: read before the wait
+    const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
+    const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
+    const BatchParams bp = p.bpar[b];
+    pdl_wait();  // the tables' rows: written by the previous kernel (no effect without a programmatic launch)
+    if constexpr (JB > 0) {
+        sample_body_reg<D, DT, JB>(p, lig, active, bp.eta, bp.salt, gm, r0, i0, rec, info);
+    } else {
+        float* stage = reinterpret_cast<float*>(smem4) + (size_t)warp * (p.K + 1) * 32 * G::E;
+        sample_body_staged<D, DT>(p, lig, lane, active, bp.eta, bp.salt, gm, r0, i0, rec, info, stage);
+    }
 }
 
 // Blocks [0, g_long) take the batch's long shared segments, one per CTA; the
@@ -540,15 +555,15 @@ __global__ void __launch_bounds__(NW * 32) k_apply(DataParams p, int b, int g_lo
     const uint32_t n_m = p.mcount[b];
     const uint32_t n_long = p.lcount[b];
     const uint4* md = p.mdesc + (size_t)b * p.mcap;
-    const uint64_t t0 = (p.t_chunk_dev ? *p.t_chunk_dev : p.t_chunk) + (uint64_t)b * (uint64_t)p.batch;
-    const float eta = p.eta[b];
+    const float eta = p.bpar[b].eta;
+    const uint32_t salt = p.bpar[b].salt;
     if ((int)blockIdx.x < g_long) {
         // descriptors come from the pre-pass: read before the wait
         uint4 d = blockIdx.x < n_long ? p.ldesc[(size_t)b * p.lcap + blockIdx.x] : make_uint4(0u, 0u, 0u, 0u);
         pdl_wait();  // the slab and the rows: written by the gather
         for (uint32_t l = blockIdx.x; l < n_long; l += (uint32_t)g_long) {
             if (l != blockIdx.x) d = p.ldesc[(size_t)b * p.lcap + l];
-            long_segment_cta<D, DT, NW>(p, d, eta, t0, part);
+            long_segment_cta<D, DT, NW>(p, d, eta, salt, part);
         }
         return;
     }
@@ -559,7 +574,7 @@ __global__ void __launch_bounds__(NW * 32) k_apply(DataParams p, int b, int g_lo
     for (int64_t m = m0; m < n_m; m += groups) {
         if (m != m0) d = md[m];
         if (d.y & kLongBit) continue;
-        segment_item<D, DT>(p, d, lig, true, eta, t0);
+        segment_item<D, DT>(p, d, lig, true, eta, salt);
     }
 }
 
@@ -654,7 +669,7 @@ __device__ __forceinline__ void slot_row(const unsigned char* set, int j, int li
 }
 
 template <int D, int DT>
-__device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, bool active, float eta, uint64_t t0,
+__device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, bool active, float eta, uint32_t salt,
                                                  uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
                                                  const uint32_t* info, const unsigned char* set) {
     using G = Geom<D, DT>;
@@ -701,7 +716,7 @@ __device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, b
                     float x[G::E];
 #pragma unroll
                     for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[e], c[e]) + g * xu[e];
-                    store_row<D, DT>(p.C, y, lig, x, p.seed, t0, ctx_table);
+                    store_row<D, DT>(p.C, y, lig, x, salt, ctx_table);
                 } else {
                     float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
 #pragma unroll
@@ -717,7 +732,7 @@ __device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, b
             const float decay = (float)(p.K + 1) * etalam;
 #pragma unroll
             for (int e = 0; e < G::E; ++e) xu[e] = fmaf(-decay, xu[e], xu[e]) + du[e];
-            store_row<D, DT>(p.U, u, lig, xu, p.seed, t0, 0u);
+            store_row<D, DT>(p.U, u, lig, xu, salt, 0u);
         } else {
             float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf0 * D + lig * G::E);
 #pragma unroll
@@ -756,7 +771,7 @@ __device__ __forceinline__ void issue_rows(const DataParams& p, const int32_t* r
 // sums chunks w, w+W, ... (entry order within a chunk); warp 0 adds the
 // chunk partials in chunk order, as segment_item does.  part: W x D floats.
 template <int D, int DT>
-__device__ __forceinline__ void long_segment_rt(const DataParams& p, uint4 d, float eta, uint64_t t0, float* part, int W) {
+__device__ __forceinline__ void long_segment_rt(const DataParams& p, uint4 d, float eta, uint32_t salt, float* part, int W) {
     using G = Geom<D, DT>;
     constexpr int PF = G::E <= 4 ? 8 : 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -817,7 +832,7 @@ __device__ __forceinline__ void long_segment_rt(const DataParams& p, uint4 d, fl
         const float decay = (float)d.w * (eta * p.lambda);
 #pragma unroll
         for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, x[e], x[e]) + acc[e];
-        store_row<D, DT>(table, row, lig, x, p.seed, t0, is_c ? 1u : 0u);
+        store_row<D, DT>(table, row, lig, x, salt, is_c ? 1u : 0u);
     }
 }
 
@@ -867,8 +882,8 @@ __global__ void __launch_bounds__(kPersistMaxWarps * 32, 1) k_persistent(DataPar
         const int64_t s_begin = (int64_t)b * p.batch;
         const int64_t nb = min((int64_t)p.batch, p.chunk_samples - s_begin);
         const int64_t units = (nb + G::GPW - 1) / G::GPW;
-        const uint64_t t0 = p.t_chunk + (uint64_t)s_begin;
-        const float eta = p.eta[b];
+        const float eta = p.bpar[b].eta;
+        const uint32_t salt = p.bpar[b].salt;
         const int64_t n_mine = uwarp < units ? (units - 1 - uwarp) / NW + 1 : 0;
         // ---- gather of batch b
         // copies of the first two units (unit 0's prefetched rows are in flight)
@@ -914,7 +929,7 @@ __global__ void __launch_bounds__(kPersistMaxWarps * 32, 1) k_persistent(DataPar
             const uint32_t* info = p.slot_info + sbase;
             const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
             const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
-            sample_body_slot<D, DT>(p, lig, active, eta, t0, gm, r0, i0, rec, info, set);
+            sample_body_slot<D, DT>(p, lig, active, eta, salt, gm, r0, i0, rec, info, set);
             // the slot's rows are read: it may be refilled by bulk copies
             fence_proxy_async_smem();
             __syncwarp();
@@ -966,14 +981,14 @@ __global__ void __launch_bounds__(kPersistMaxWarps * 32, 1) k_persistent(DataPar
             // long shared segments: one CTA each
             const uint32_t n_long = p.lcount[b];
             for (uint32_t l = blockIdx.x; l < n_long; l += gridDim.x)
-                long_segment_rt<D, DT>(p, p.ldesc[(size_t)b * p.lcap + l], eta, t0, part, W);
+                long_segment_rt<D, DT>(p, p.ldesc[(size_t)b * p.lcap + l], eta, salt, part, W);
             // short ones: one lane group each
             const uint32_t n_m = p.mcount[b];
             const uint4* md = p.mdesc + (size_t)b * p.mcap;
             for (int64_t m = uwarp * G::GPW + grp; m < n_m; m += NW * G::GPW) {
                 const uint4 d = md[m];
                 if (d.y & kLongBit) continue;
-                segment_item<D, DT>(p, d, lig, true, eta, t0);
+                segment_item<D, DT>(p, d, lig, true, eta, salt);
             }
         }
         if (!grid_barrier(p, round++, &s_flag)) {
@@ -1009,14 +1024,13 @@ struct PrepassParams {
     int K, order;
     int walk;  // 1: slots 0 and 1 come from the walk sampler (no arc draw here)
     int32_t* rec;
-    uint64_t* t_out;  // receives t_chunk (read by graph replays of the data phase)
-    // per batch of the chunk (minibatch schedules): the learning rate, and
-    // the counters of the grouping, zeroed here
+    // per batch of the chunk (minibatch schedules): its parameters, and the
+    // counters of the grouping, zeroed here
     int n_batches;
     float lr0, lr_floor;
     int lr_schedule;
     uint64_t lr_total;
-    float* eta;  // null: no per-batch outputs (Hogwild schedule)
+    BatchParams* bpar;  // null: no per-batch outputs (Hogwild schedule)
     uint32_t* mcount;
     uint32_t* lcount;
     uint32_t* pcount;
@@ -1040,10 +1054,10 @@ __device__ __forceinline__ float batch_eta(const PrepassParams& p, uint64_t t0) 
 
 __global__ void k_chunk_draws(PrepassParams p) {
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-    if (tid == 0 && p.t_out) *p.t_out = p.t_chunk;
-    if (p.eta)
+    if (p.bpar)
         for (uint32_t b = tid; b < (uint32_t)p.n_batches; b += stride) {
-            p.eta[b] = batch_eta(p, p.t_chunk + (uint64_t)b * (uint64_t)p.batch);
+            const uint64_t t0 = p.t_chunk + (uint64_t)b * (uint64_t)p.batch;
+            p.bpar[b] = BatchParams{batch_eta(p, t0), sr_salt(p.seed, t0)};
             p.mcount[b] = p.lcount[b] = p.pcount[b] = 0u;
         }
     const uint32_t C1 = (uint32_t)p.K + 1u, R = (uint32_t)p.K + 2u;
@@ -1613,7 +1627,7 @@ struct Buf {
 // pre-pass of chunk c+1 (on its own low-priority stream) fills one while the
 // data phase of chunk c reads the other.
 struct ChunkSet {
-    Buf rec, slot_info, depmap, mdesc, mcount, ldesc, lcount, eta, tchunk;
+    Buf rec, slot_info, depmap, mdesc, mcount, ldesc, lcount, bpar;
     // captured data phase of a full chunk of this set, and what it was
     // captured for: the parameters, the warps per block and the kernels (the
     // launcher of one row width and table type: tables of another type can
@@ -1698,16 +1712,16 @@ static void once_per_device(std::atomic<uint64_t>& done, F f) {
     done.fetch_or(bit, std::memory_order_acq_rel);
 }
 
+// Warps of a staged gather block (at most kGatherWarps, fewer when the stages
+// exceed the shared memory) and its shared memory.
 template <int D, int DT>
-static int gather_warps(const DataParams& p, int requested, int cap, size_t* smem_out, int dflt = 8) {
-    using G = Geom<D, DT>;
+static int staged_warps(int K, int requested, size_t* smem_out) {
     // staging: (K+1) context rows x 32 lanes x E floats per warp
-    const size_t per_warp = (size_t)(p.K + 1) * 32 * G::E * sizeof(float);
-    int wpb = requested > 0 ? requested : dflt;
-    wpb = std::min<int>(wpb, cap);
-    wpb = std::max<int>(1, std::min<int>(wpb, (int)(kMaxSmem / per_warp)));
-    *smem_out = (size_t)wpb * per_warp;
-    return wpb;
+    const size_t per_warp = (size_t)(K + 1) * 32 * Geom<D, DT>::E * sizeof(float);
+    const int wpb = requested > 0 ? std::min(requested, kGatherWarps) : kGatherWarps;
+    const int fit = std::max(1, std::min(wpb, (int)(kMaxSmem / per_warp)));
+    *smem_out = (size_t)fit * per_warp;
+    return fit;
 }
 
 template <typename... Args, typename... Vals>
@@ -1729,15 +1743,24 @@ static cudaError_t launch_pdl(void (*kern)(Args...), unsigned grid, unsigned blo
 template <int D, int DT>
 static cudaError_t launch_data_batched(const DataParams& p, int warps_per_block, cudaStream_t s) {
     using G = Geom<D, DT>;
+    // 4 warps per block: at 64 registers a 4096-sample batch is one wave.
+    // Rows of up to 128 values and K <= 7: the context rows in registers, in
+    // the smallest body that holds them (K + 1 <= 2, 4, 6 or 8)
     size_t smem = 0;
-    // 4 warps per block: at ~70 registers a 4096-sample batch is one wave
-    const int wpb = gather_warps<D, DT>(p, warps_per_block, kGatherWarps, &smem, kGatherWarps);
-    if (G::E <= 4 && p.K < 8) smem = 0;  // the register body stages nothing
-    static std::atomic<uint64_t> attr_set{0};
-    once_per_device(attr_set, [] {
-        cudaFuncSetAttribute(k_gather<D, DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-        cudaFuncSetAttribute(k_gather<D, DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-    });
+    int wpb = warps_per_block > 0 ? std::min(warps_per_block, kGatherWarps) : kGatherWarps;
+    void (*gather)(DataParams, int) = nullptr;
+    if constexpr (G::E <= 4) {
+        if (p.K < 8)
+            gather = p.K < 2 ? k_gather<D, DT, 2> : p.K < 4 ? k_gather<D, DT, 4> : p.K < 6 ? k_gather<D, DT, 6> : k_gather<D, DT, 8>;
+    }
+    if (!gather) {
+        gather = k_gather<D, DT, 0>;
+        wpb = staged_warps<D, DT>(p.K, warps_per_block, &smem);
+        static std::atomic<uint64_t> attr_set{0};
+        once_per_device(attr_set, [] {
+            cudaFuncSetAttribute(k_gather<D, DT, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+        });
+    }
     const int64_t per_block = (int64_t)wpb * G::GPW;
     const int aw = p.apply_warps == kApplyWarpsAlone ? kApplyWarpsAlone : kApplyWarpsShared;
     const int64_t apply_per_block = (int64_t)aw * G::GPW;
@@ -1750,8 +1773,7 @@ static cudaError_t launch_data_batched(const DataParams& p, int warps_per_block,
         const unsigned g1 = (unsigned)((nb + per_block - 1) / per_block);
         // the chunk's first gather follows the pre-pass with a full dependency;
         // later launches overlap their start with the previous kernel's tail
-        if (b == 0) e = launch_pdl(k_gather<D, DT, false>, g1, wpb * 32, smem, s, false, p, b);
-        else e = launch_pdl(k_gather<D, DT, true>, g1, wpb * 32, smem, s, true, p, b);
+        e = launch_pdl(gather, g1, wpb * 32, smem, s, b > 0, p, b);
         if (e != cudaSuccess) break;
         // a shared segment has two or more of the batch's nb * (K+2) entries
         const int64_t max_m = nb * (p.K + 2) / 2 + 1;
@@ -1882,7 +1904,7 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     auto each = [&](auto&& f) -> bool {
         if (hogwild) {
             for (auto& cs : ws->set)
-                if (!f(cs.rec, sizeof(int32_t) * max_items) || !f(cs.tchunk, 256)) return false;
+                if (!f(cs.rec, sizeof(int32_t) * max_items)) return false;
             return true;
         }
         if (!f(ws->items1, sizeof(uint64_t) * max_items) || !f(ws->counters, 256) ||
@@ -1894,10 +1916,10 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
                         !f(ws->boff, sizeof(uint32_t) * (size_t)nb * (kBuckets + 1))))
             return false;
         for (auto& cs : ws->set) {
-            if (!f(cs.rec, sizeof(int32_t) * max_items) || !f(cs.eta, sizeof(float) * (nb + 1)) ||
+            if (!f(cs.rec, sizeof(int32_t) * max_items) || !f(cs.bpar, sizeof(BatchParams) * (nb + 1)) ||
                 !f(cs.slot_info, sizeof(uint32_t) * max_items) || !f(cs.mdesc, sizeof(uint4) * (size_t)nb * mcap) ||
                 !f(cs.mcount, sizeof(uint32_t) * (nb + 1)) || !f(cs.ldesc, sizeof(uint4) * (size_t)nb * lcap) ||
-                !f(cs.lcount, sizeof(uint32_t) * (nb + 1)) || !f(cs.tchunk, 256))
+                !f(cs.lcount, sizeof(uint32_t) * (nb + 1)))
                 return false;
             if (persistent && !f(cs.depmap, sizeof(uint32_t) * (size_t)nb * kDepWords)) return false;
         }
@@ -1998,7 +2020,6 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     dp.lcap = lcap;
     dp.slab = (float*)ws->slab.p;
     dp.batch = a.batch;
-    dp.seed = a.seed;
     dp.lambda = (float)a.lambda;
     dp.alpha_neg = (float)a.alpha_neg;
     dp.status = status;
@@ -2030,10 +2051,9 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
         pp.t_chunk = t;
         pp.chunk_samples = cs;
         pp.rec = (int32_t*)cset.rec.p;
-        pp.t_out = (uint64_t*)cset.tchunk.p;
         if (!hogwild) {
             pp.n_batches = cb;
-            pp.eta = (float*)cset.eta.p;
+            pp.bpar = (BatchParams*)cset.bpar.p;
             pp.mcount = (uint32_t*)cset.mcount.p;
             pp.lcount = (uint32_t*)cset.lcount.p;
         }
@@ -2113,18 +2133,15 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
             dp.mcount = (const uint32_t*)cset.mcount.p;
             dp.ldesc = (const uint4*)cset.ldesc.p;
             dp.lcount = (const uint32_t*)cset.lcount.p;
-            dp.eta = (const float*)cset.eta.p;
+            dp.bpar = (const BatchParams*)cset.bpar.p;
             dp.depmap = (const uint32_t*)cset.depmap.p;
-            dp.t_chunk = t;
             dp.chunk_samples = cs;
             dp.n_batches = cb;
             if (persistent && (e = cudaMemsetAsync(abort_word, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
             if (!persistent && a.graph && !ws->graph_failed && cs == max_chunk && c > 0) {
-                // a full chunk: replay this set's captured data phase (the chunk's
-                // first sample index comes from the set's device copy)
-                dp.t_chunk_dev = (const uint64_t*)cset.tchunk.p;
+                // a full chunk: replay this set's captured data phase (what
+                // differs from chunk to chunk is in the set's buffers)
                 DataParams key = dp;
-                key.t_chunk = 0;
                 if (!cset.graph || cset.graph_wpb != a.warps_per_block || cset.graph_fn != data ||
                     memcmp(&key, &cset.graph_key, sizeof key) != 0) {
                     if (cset.graph) cudaGraphExecDestroy(cset.graph);
@@ -2151,11 +2168,9 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
                 if (cset.graph) {
                     if ((e = cudaGraphLaunch(cset.graph, s)) != cudaSuccess) return e;
                 } else {
-                    dp.t_chunk_dev = nullptr;
                     if ((e = data(dp, a.warps_per_block, s)) != cudaSuccess) return e;
                 }
             } else {
-                dp.t_chunk_dev = nullptr;
                 if ((e = data(dp, a.warps_per_block, s)) != cudaSuccess) return e;
             }
         }
