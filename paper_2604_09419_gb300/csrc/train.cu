@@ -64,10 +64,32 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // A shared segment's entries are summed in chunks of kChunk: partial sums in
-// entry order, then the partials in chunk order.  Segments longer than one
-// chunk (the hub rows) are summed by a whole CTA in the batched schedule.
+// entry order, then the partials in chunk order.  Segments are listed by the
+// number of their chunks: class 0 has one, classes 1, 2 and 3 up to 2, 4 and
+// 8, class 4 more (the hub rows).
 constexpr uint32_t kChunk = 8;
-constexpr uint32_t kLongBit = 1u << 31;  // in mdesc.y: summed by a CTA
+constexpr int kClasses = 5;
+constexpr int kLong = kClasses;  // one more list: all of classes 1 .. 4, as they come
+constexpr int kCounts = 8;       // counters of a batch: one per list, padded
+
+__host__ __device__ inline int seg_class(uint32_t len) {
+    const uint32_t c = (len + kChunk - 1) / kChunk;
+    return c <= 1 ? 0 : c <= 2 ? 1 : c <= 4 ? 2 : c <= 8 ? 3 : 4;
+}
+
+// Where a batch's classes begin in its list, for at most n entries a batch.
+struct SegLayout {
+    uint32_t off[kClasses + 1];
+    uint32_t cap;
+    __host__ void set(int64_t n) {
+        const uint32_t least[kClasses + 1] = {2, kChunk + 1, 2 * kChunk + 1, 4 * kChunk + 1, 8 * kChunk + 1, kChunk + 1};
+        cap = 0;
+        for (int c = 0; c <= kClasses; ++c) {
+            off[c] = cap;
+            cap += (uint32_t)(n / least[c]) + 1;
+        }
+    }
+};
 
 // Sort item value: (sample within the chunk) << kSlotBits | slot.
 constexpr uint32_t kSlotBits = 6;
@@ -113,12 +135,9 @@ struct DataParams {
     uint32_t row_bits;
     const int32_t* rec;      // [chunk samples][K+2]
     const uint32_t* slot_info;  // [chunk samples][K+2]: position, or the singleton bit
-    const uint4* mdesc;      // [n_batches][mcap] shared segments: {first position, length | long bit, row, pair count}
-    const uint32_t* mcount;  // [n_batches]
-    uint32_t mcap;
-    const uint4* ldesc;      // [n_batches][lcap] long shared segments (also in mdesc, flagged)
-    const uint32_t* lcount;  // [n_batches]
-    uint32_t lcap;
+    const uint4* seg;        // [n_batches][sl.cap] shared segments by class: {first position, length, row, pair count}
+    const uint32_t* scount;  // [n_batches][kCounts] segments of each list
+    SegLayout sl;
     float* slab;             // [batch * (K+2)][D], by position within the batch
     const uint32_t* depmap;  // [n_batches][kDepWords] rows each batch touches (bit dep_bit(row id))
     int64_t chunk_samples;
@@ -371,8 +390,8 @@ __device__ __forceinline__ void segment_item(const DataParams& p, uint4 d, int l
     using G = Geom<D, DT>;
     constexpr int PF = G::E <= 4 ? 8 : 4;  // slab entries in flight per lane
     if (!active) return;
-    // d = {first position, length | long bit, row, pair count}
-    const uint32_t len = d.y & ~kLongBit;
+    // d = {first position, length, row, pair count}
+    const uint32_t len = d.y;
     const uint32_t rowid = d.z & ((1u << p.row_bits) - 1u);
     const bool is_c = p.order == 2 && rowid >= (uint32_t)p.n_nodes;
     void* table = is_c ? p.C : p.U;
@@ -420,56 +439,48 @@ __device__ __forceinline__ void segment_item(const DataParams& p, uint4 d, int l
     store_row<D, DT>(table, row, lig, x, salt, is_c ? 1u : 0u);
 }
 
-// Warps of an apply block: 16 when one order trains alone (a hub row's
-// chunks are summed in fewer rounds), 8 when two orders train concurrently
-// (smaller blocks interleave better with the other order's kernels).
-constexpr int kApplyWarpsAlone = 16, kApplyWarpsShared = 8;
-
-// A long shared segment summed by the NW warps of a CTA: warp w sums chunks
-// w, w+NW, ... (entry order within a chunk); warp 0 adds the chunk partials
-// in chunk order - the same order as segment_item, so the result does not
-// depend on the number of warps.  Uses lane group 0 of each warp.  part:
-// shared, NW x D floats.
-template <int D, int DT, int NW>
-__device__ __forceinline__ void long_segment_cta(const DataParams& p, uint4 d, float eta, uint32_t salt, float* part) {
+// A shared segment of more than one chunk, summed by a team of `ts` lane
+// groups of the CTA (this one is group g, member g % ts): member w
+// sums chunks w, w + ts, ... (entry order within a chunk); the first member
+// adds the partials in chunk order - the same order as segment_item, so the
+// result does not depend on the team.  Called by all threads of the CTA, with
+// the same number of rounds.  part: shared, one row of D floats per group.
+template <int D, int DT>
+__device__ __forceinline__ void segment_team(const DataParams& p, uint4 d, uint32_t ts, uint32_t g, int lig, float eta,
+                                             uint32_t salt, float* part) {
     using G = Geom<D, DT>;
     constexpr int PF = G::E <= 4 ? 8 : 4;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool mine = lane < G::L;  // group 0 of the warp
-    const int lig = lane;
-    const uint32_t len = d.y & ~kLongBit;
-    const uint32_t n_chunks = (len + kChunk - 1) / kChunk;
+    const uint32_t tg = g % ts;
+    const bool first = d.y && tg == 0;
     const uint32_t rowid = d.z & ((1u << p.row_bits) - 1u);
     const bool is_c = p.order == 2 && rowid >= (uint32_t)p.n_nodes;
-    void* table = is_c ? p.C : p.U;
-    const int64_t row = is_c ? (int64_t)rowid - p.n_nodes : (int64_t)rowid;
-    float x[G::E];
-    if (warp == 0 && mine) load_row<D, DT>(table, row, lig, x);  // in flight during the sums
     float acc[G::E];
 #pragma unroll
     for (int e = 0; e < G::E; ++e) acc[e] = 0.0f;
-    const float* base = p.slab + (int64_t)d.x * D + (mine ? lig : 0) * G::E;
-    for (uint32_t r0 = 0; r0 < n_chunks; r0 += NW) {
-        const uint32_t c = r0 + (uint32_t)warp;
-        if (mine && c < n_chunks) {
+    const float* src = p.slab + ((int64_t)d.x + tg * kChunk) * D + lig * G::E;
+    float* mine = part + g * D + lig * G::E;
+    const uint32_t rounds = max(1u, (d.y + kChunk * ts - 1) / (kChunk * ts));
+    // left: entries of the segment from this member's chunk on
+    int left = (int)d.y - (int)(tg * kChunk);
+    for (uint32_t r = 0; r < rounds; ++r) {
+        if (left > 0) {
             float pt[G::E];
 #pragma unroll
             for (int e = 0; e < G::E; ++e) pt[e] = 0.0f;
-            const uint32_t c0 = c * kChunk;
 #pragma unroll
-            for (uint32_t k0 = 0; k0 < kChunk; k0 += PF) {
+            for (int k0 = 0; k0 < (int)kChunk; k0 += PF) {
                 float4 buf[PF][G::E / 4];
 #pragma unroll
                 for (int kk = 0; kk < PF; ++kk) {
-                    if (c0 + k0 + kk < len) {
-                        const float4* src = reinterpret_cast<const float4*>(base + (int64_t)(c0 + k0 + kk) * D);
+                    if (k0 + kk < left) {
 #pragma unroll
-                        for (int q = 0; q < G::E / 4; ++q) buf[kk][q] = ld_cg(src + q);
+                        for (int q = 0; q < G::E / 4; ++q)
+                            buf[kk][q] = ld_cg(reinterpret_cast<const float4*>(src + (k0 + kk) * D) + q);
                     }
                 }
 #pragma unroll
                 for (int kk = 0; kk < PF; ++kk) {
-                    if (c0 + k0 + kk < len) {
+                    if (k0 + kk < left) {
 #pragma unroll
                         for (int q = 0; q < G::E / 4; ++q) {
                             pt[4 * q] += buf[kk][q].x;
@@ -480,25 +491,46 @@ __device__ __forceinline__ void long_segment_cta(const DataParams& p, uint4 d, f
                     }
                 }
             }
+            float4* dst = reinterpret_cast<float4*>(mine);
 #pragma unroll
-            for (int e = 0; e < G::E; ++e) part[warp * D + lig * G::E + e] = pt[e];
+            for (int q = 0; q < G::E / 4; ++q) dst[q] = make_float4(pt[4 * q], pt[4 * q + 1], pt[4 * q + 2], pt[4 * q + 3]);
         }
         __syncthreads();
-        if (warp == 0 && mine) {
-            const uint32_t nr = min((uint32_t)NW, n_chunks - r0);
-            for (uint32_t w = 0; w < nr; ++w)
+        if (first) {
+            const int nr = min((int)ts, (left + (int)kChunk - 1) / (int)kChunk);
+#pragma unroll 4
+            for (int w = 0; w < nr; ++w) {
+                const float4* v4 = reinterpret_cast<const float4*>(mine + w * D);
 #pragma unroll
-                for (int e = 0; e < G::E; ++e) acc[e] += part[w * D + lig * G::E + e];
+                for (int q = 0; q < G::E / 4; ++q) {
+                    const float4 v = v4[q];
+                    acc[4 * q] += v.x;
+                    acc[4 * q + 1] += v.y;
+                    acc[4 * q + 2] += v.z;
+                    acc[4 * q + 3] += v.w;
+                }
+            }
         }
-        __syncthreads();
+        if (r + 1 < rounds) __syncthreads();
+        left -= (int)(ts * kChunk);
+        src += (int64_t)ts * kChunk * D;
     }
-    if (warp == 0 && mine) {
+    if (first) {
+        void* table = is_c ? p.C : p.U;
+        const int64_t row = is_c ? (int64_t)rowid - p.n_nodes : (int64_t)rowid;
+        float x[G::E];
+        load_row<D, DT>(table, row, lig, x);
         const float decay = (float)d.w * (eta * p.lambda);
 #pragma unroll
         for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, x[e], x[e]) + acc[e];
         store_row<D, DT>(table, row, lig, x, salt, is_c ? 1u : 0u);
     }
 }
+
+// Warps of an apply block: 16 when one order trains alone (a hub row's
+// chunks are summed in fewer rounds), 8 when two orders train concurrently
+// (smaller blocks interleave better with the other order's kernels).
+constexpr int kApplyWarpsAlone = 16, kApplyWarpsShared = 8;
 
 // ---------------------------------------------------------------------------
 // Batched schedule: one launch per phase per batch.
@@ -511,6 +543,7 @@ constexpr size_t kMaxSmem = 200 * 1024;
 // pre-pass kernels of the next chunk (one batch at 72 registers filled 95%
 // of the register file, and any pre-pass block displaced gather warps).
 constexpr int kGatherWarps = 4;
+
 
 // JB: context rows held in registers (K + 1 <= JB), or 0 for the staged body.
 template <int D, int DT, int JB>
@@ -542,39 +575,90 @@ __global__ void __launch_bounds__(kGatherWarps * 32, 8) k_gather(DataParams p, i
     }
 }
 
-// Blocks [0, g_long) take the batch's long shared segments, one per CTA; the
-// other blocks take the short ones, one per lane group.
-
+// The first long_blocks() blocks take the batch's segments of several chunks,
+// those after them the short ones, one per lane group; blocks that the short
+// ones leave free help with the long ones, and return at once where there is
+// nothing to help with (a waiting block holds registers that the next
+// gather's blocks could start in: 4% of one order's time).  A block of NG
+// lane groups takes one long segment, or up to NG/2, NG/4 or NG/8 of classes
+// 1, 2 and 3 (a team per segment, a lane group per chunk, one round).
+// Bound: latency - a slab read from L2, a sum through shared memory and the
+// row's write.  On small or skewed graphs most segments are long (R-MAT 16,
+// B = 4096: 320 of 5,000 a batch, 814 chunks): with one block per long
+// segment, 64 of them, 2^22 samples took 12.1 ms (one order) and 17.0 (both);
+// with teams 8.6 and 12.8.  R-MAT 14 at d = 64: 17.2 and 7.6; 1,024 nodes at
+// d = 32: 22.2 and 8.7.  R-MAT 20: 7.33 and 7.51 (FP32), 6.54 and 6.51 (BF16),
+// both orders 11.66 and 11.30.
+template <int NW>
+constexpr uint32_t long_blocks() {
+    return 1024 / NW;
+}
 template <int D, int DT, int NW>
-__global__ void __launch_bounds__(NW * 32) k_apply(DataParams p, int b, int g_long) {
+__global__ void __launch_bounds__(NW * 32, D <= 128 ? 32 / NW : 1) k_apply(DataParams p, int b) {
     using G = Geom<D, DT>;
-    __shared__ float part[NW * D];
+    constexpr uint32_t kLongBlocks = long_blocks<NW>();
+    constexpr uint32_t NG = NW * G::GPW, kLogNG = NG == 8 ? 3 : NG == 16 ? 4 : NG == 32 ? 5 : NG == 64 ? 6 : 7;
+    static_assert(NG == 1u << kLogNG, "a block's lane groups");
+    __shared__ __align__(16) float part[NG * D];
     pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = lane / G::L, lig = lane % G::L;
-    const uint32_t n_m = p.mcount[b];
-    const uint32_t n_long = p.lcount[b];
-    const uint4* md = p.mdesc + (size_t)b * p.mcap;
+    const uint32_t g = (uint32_t)(warp * G::GPW + grp);
+    // The lists come from the pre-pass and are read before the wait, the short
+    // segment without waiting for the counts: little of this prologue overlaps
+    // the gather, whose blocks hold the register file.
+    const uint32_t* cnt = p.scount + (size_t)b * kCounts;
+    const uint4* seg = p.seg + (size_t)b * p.sl.cap;
+    const uint32_t n0 = cnt[0], nl = cnt[kLong], most = p.sl.off[1];  // class 0 begins at 0
     const float eta = p.bpar[b].eta;
     const uint32_t salt = p.bpar[b].salt;
-    if ((int)blockIdx.x < g_long) {
-        // descriptors come from the pre-pass: read before the wait
-        uint4 d = blockIdx.x < n_long ? p.ldesc[(size_t)b * p.lcap + blockIdx.x] : make_uint4(0u, 0u, 0u, 0u);
+    uint32_t m = blockIdx.x >= kLongBlocks ? (blockIdx.x - kLongBlocks) * NG + g : most;
+    const uint32_t first = m < most ? m : p.sl.off[kLong] + blockIdx.x;
+    uint4 d = first < p.sl.cap ? seg[first] : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t nsb = min(gridDim.x - kLongBlocks, (n0 + NG - 1) / NG);  // blocks with short segments
+    if (blockIdx.x - kLongBlocks < nsb) {
         pdl_wait();  // the slab and the rows: written by the gather
-        for (uint32_t l = blockIdx.x; l < n_long; l += (uint32_t)g_long) {
-            if (l != blockIdx.x) d = p.ldesc[(size_t)b * p.lcap + l];
-            long_segment_cta<D, DT, NW>(p, d, eta, salt, part);
+        while (m < n0) {
+            segment_item<D, DT>(p, d, lig, true, eta, salt);
+            m += nsb * NG;
+            if (m < n0) d = seg[m];
         }
         return;
     }
-    const int64_t groups = (int64_t)(gridDim.x - g_long) * (blockDim.x >> 5) * G::GPW;
-    const int64_t m0 = ((int64_t)(blockIdx.x - g_long) * (blockDim.x >> 5) + warp) * G::GPW + grp;
-    uint4 d = m0 < n_m ? md[m0] : make_uint4(0u, 0u, 0u, 0u);
-    pdl_wait();  // the slab and the rows: written by the gather
-    for (int64_t m = m0; m < n_m; m += groups) {
-        if (m != m0) d = md[m];
-        if (d.y & kLongBit) continue;
-        segment_item<D, DT>(p, d, lig, true, eta, salt);
+    // few segments of several chunks: one a block (an SM reads a segment
+    // faster when it reads no other)
+    if (nl <= kLongBlocks) {
+        // the first block waits even without a segment: the next gather relies
+        // on this kernel's end coming after the gather's
+        if (blockIdx.x >= nl && blockIdx.x != 0) return;
+        if (blockIdx.x >= nl) d.y = 0u;
+        pdl_wait();
+        segment_team<D, DT>(p, d, NG, g, lig, eta, salt, part);
+        return;
+    }
+    const uint32_t helper = blockIdx.x < kLongBlocks ? blockIdx.x : blockIdx.x - nsb, helpers = gridDim.x - nsb;
+    for (uint32_t t = helper;; t += helpers) {
+        // (the counts are read again for every task: held over segment_team
+        // they would not fit 64 registers)
+        const uint4 n03 = ld_again(reinterpret_cast<const uint4*>(cnt));
+        const uint32_t n4 = ld_again(cnt + 4);
+        const uint32_t t1 = (n03.y + NG / 2 - 1) / (NG / 2), t2 = (n03.z + NG / 4 - 1) / (NG / 4),
+                       t3 = (n03.w + NG / 8 - 1) / (NG / 8);
+        if (t >= t1 + t2 + t3 + n4) return;  // (not the first block's first task)
+        // task t, the longest segments first
+        uint32_t lts = kLogNG, at = t, n = n4, off = p.sl.off[4];
+        if (at >= n4) {
+            at -= n4, lts = 3, n = n03.w, off = p.sl.off[3];
+            if (at >= t3) {
+                at -= t3, lts = 2, n = n03.z, off = p.sl.off[2];
+                if (at >= t2) at -= t2, lts = 1, n = n03.y, off = p.sl.off[1];
+            }
+        }
+        const uint32_t k = (at << (kLogNG - lts)) + (g >> lts);
+        d = k < n ? seg[off + k] : make_uint4(0u, 0u, 0u, 0u);
+        if (t == helper) pdl_wait();
+        else __syncthreads();  // `part` is read by the last task
+        segment_team<D, DT>(p, d, 1u << lts, g, lig, eta, salt, part);
     }
 }
 
@@ -777,7 +861,7 @@ __device__ __forceinline__ void long_segment_rt(const DataParams& p, uint4 d, fl
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool mine = lane < G::L;
     const int lig = lane;
-    const uint32_t len = d.y & ~kLongBit;
+    const uint32_t len = d.y;
     const uint32_t n_chunks = (len + kChunk - 1) / kChunk;
     const uint32_t rowid = d.z & ((1u << p.row_bits) - 1u);
     const bool is_c = p.order == 2 && rowid >= (uint32_t)p.n_nodes;
@@ -978,18 +1062,18 @@ __global__ void __launch_bounds__(kPersistMaxWarps * 32, 1) k_persistent(DataPar
             }
         }
         {
-            // long shared segments: one CTA each
-            const uint32_t n_long = p.lcount[b];
-            for (uint32_t l = blockIdx.x; l < n_long; l += gridDim.x)
-                long_segment_rt<D, DT>(p, p.ldesc[(size_t)b * p.lcap + l], eta, salt, part, W);
-            // short ones: one lane group each
-            const uint32_t n_m = p.mcount[b];
-            const uint4* md = p.mdesc + (size_t)b * p.mcap;
-            for (int64_t m = uwarp * G::GPW + grp; m < n_m; m += NW * G::GPW) {
-                const uint4 d = md[m];
-                if (d.y & kLongBit) continue;
-                segment_item<D, DT>(p, d, lig, true, eta, salt);
+            // segments of several chunks: one CTA each
+            const uint32_t* cnt = p.scount + (size_t)b * kCounts;
+            const uint4* seg = p.seg + (size_t)b * p.sl.cap;
+            uint32_t l = blockIdx.x;
+            for (int c = 1; c < kClasses; ++c) {
+                for (; l < cnt[c]; l += gridDim.x)
+                    long_segment_rt<D, DT>(p, seg[p.sl.off[c] + l], eta, salt, part, W);
+                l -= cnt[c];
             }
+            // short ones: one lane group each
+            for (int64_t m = uwarp * G::GPW + grp; m < cnt[0]; m += NW * G::GPW)
+                segment_item<D, DT>(p, seg[m], lig, true, eta, salt);
         }
         if (!grid_barrier(p, round++, &s_flag)) {
             ok = false;
@@ -1031,8 +1115,7 @@ struct PrepassParams {
     int lr_schedule;
     uint64_t lr_total;
     BatchParams* bpar;  // null: no per-batch outputs (Hogwild schedule)
-    uint32_t* mcount;
-    uint32_t* lcount;
+    uint32_t* scount;
     uint32_t* pcount;
 };
 
@@ -1058,7 +1141,8 @@ __global__ void k_chunk_draws(PrepassParams p) {
         for (uint32_t b = tid; b < (uint32_t)p.n_batches; b += stride) {
             const uint64_t t0 = p.t_chunk + (uint64_t)b * (uint64_t)p.batch;
             p.bpar[b] = BatchParams{batch_eta(p, t0), sr_salt(p.seed, t0)};
-            p.mcount[b] = p.lcount[b] = p.pcount[b] = 0u;
+            for (int k = 0; k < kCounts; ++k) p.scount[(size_t)b * kCounts + k] = 0u;
+            p.pcount[b] = 0u;
         }
     const uint32_t C1 = (uint32_t)p.K + 1u, R = (uint32_t)p.K + 2u;
     const uint32_t total = (uint32_t)p.chunk_samples * C1;
@@ -1105,12 +1189,9 @@ struct GroupParams {
     uint32_t* pcount;       // [n_batches] positions handed out (k_group_parts)
     // outputs
     uint32_t* slot_info;
-    uint4* mdesc;
-    uint32_t* mcount;
-    uint32_t mcap;
-    uint4* ldesc;
-    uint32_t* lcount;
-    uint32_t lcap;
+    uint4* seg;
+    uint32_t* scount;
+    SegLayout sl;
     uint32_t* depmap;     // [n_batches][kDepWords] rows each batch touches (zeroed before), or null
 };
 
@@ -1350,14 +1431,11 @@ __global__ void __launch_bounds__(kSortThreads) k_bucket_sort(GroupParams q) {
             q.slot_info[(v >> kSlotBits) * q.R + slot] = len == 1 ? kSingleBit : pos;
         }
         if (len > 1) {
-            uint32_t flagged = len;
-            if (len > kChunk) {
-                const uint32_t l = atomicAdd(q.lcount + b, 1u);
-                q.ldesc[(size_t)b * q.lcap + l] = make_uint4(head, len, key, cnt);
-                flagged |= kLongBit;
-            }
-            const uint32_t m = atomicAdd(q.mcount + b, 1u);
-            q.mdesc[(size_t)b * q.mcap + m] = make_uint4(head, flagged, key, cnt);
+            const int c = seg_class(len);
+            const uint32_t m = atomicAdd(q.scount + (size_t)b * kCounts + c, 1u);
+            uint4* seg = q.seg + (size_t)b * q.sl.cap;
+            seg[q.sl.off[c] + m] = make_uint4(head, len, key, cnt);
+            if (c) seg[q.sl.off[kLong] + atomicAdd(q.scount + (size_t)b * kCounts + kLong, 1u)] = make_uint4(head, len, key, cnt);
         }
     }
 }
@@ -1441,19 +1519,28 @@ __device__ __forceinline__ void warp_sort_keys(uint64_t* a, uint32_t n) {
 __device__ __forceinline__ void list_segments(const GroupParams& q, int b, bool is_head, uint32_t head, uint32_t len,
                                               uint32_t hv, uint32_t z) {
     const int lane = threadIdx.x & 31;
-    const bool m = is_head && len > 1, l = m && len > kChunk;
-    const uint32_t mm = __ballot_sync(0xFFFFFFFFu, m), lm = __ballot_sync(0xFFFFFFFFu, l);
-    if (!mm) return;
-    uint32_t base = 0;  // lane 0: mdesc entries, lane 1: ldesc entries
-    if (lane == 0) base = atomicAdd(q.mcount + b, (uint32_t)__popc(mm));
-    else if (lane == 1 && lm) base = atomicAdd(q.lcount + b, (uint32_t)__popc(lm));
-    const uint32_t mb = __shfl_sync(0xFFFFFFFFu, base, 0), lb = __shfl_sync(0xFFFFFFFFu, base, 1);
-    const uint32_t lt = (1u << lane) - 1u;
+    const bool m = is_head && len > 1;
+    if (!__any_sync(0xFFFFFFFFu, m)) return;
+    const int cls = m ? seg_class(len) : kClasses + 1;
+    // lane c reserves the places of list c
+    const uint32_t longs = __ballot_sync(0xFFFFFFFFu, m && cls > 0);
+    uint32_t peers = 0, count = lane == kLong ? __popc(longs) : 0u, base = 0;
+#pragma unroll
+    for (int c = 0; c < kClasses; ++c) {
+        const uint32_t mk = __ballot_sync(0xFFFFFFFFu, cls == c);
+        if (cls == c) peers = mk;
+        if (lane == c) count = __popc(mk);
+    }
+    if (count) base = atomicAdd(q.scount + (size_t)b * kCounts + lane, count);
+    const uint32_t lbase = __shfl_sync(0xFFFFFFFFu, base, kLong);
+    base = __shfl_sync(0xFFFFFFFFu, base, cls);
+    // pair count: K + 1 for a source entry, 1 otherwise
     if (m) {
-        // pair count: K + 1 for a source entry, 1 otherwise
-        const uint4 d = make_uint4(head, l ? len | kLongBit : len, unhrow(hv), len + z * q.K);
-        q.mdesc[(size_t)b * q.mcap + mb + __popc(mm & lt)] = d;
-        if (l) q.ldesc[(size_t)b * q.lcap + lb + __popc(lm & lt)] = make_uint4(head, len, d.z, d.w);
+        const uint32_t lt = (1u << lane) - 1u;
+        const uint4 d = make_uint4(head, len, unhrow(hv), len + z * q.K);
+        uint4* seg = q.seg + (size_t)b * q.sl.cap;
+        seg[q.sl.off[cls] + base + __popc(peers & lt)] = d;
+        if (cls > 0) seg[q.sl.off[kLong] + lbase + __popc(longs & lt)] = d;
     }
 }
 
@@ -1627,7 +1714,7 @@ struct Buf {
 // pre-pass of chunk c+1 (on its own low-priority stream) fills one while the
 // data phase of chunk c reads the other.
 struct ChunkSet {
-    Buf rec, slot_info, depmap, mdesc, mcount, ldesc, lcount, bpar;
+    Buf rec, slot_info, depmap, seg, scount, bpar;
     // captured data phase of a full chunk of this set, and what it was
     // captured for: the parameters, the warps per block and the kernels (the
     // launcher of one row width and table type: tables of another type can
@@ -1762,11 +1849,14 @@ static cudaError_t launch_data_batched(const DataParams& p, int warps_per_block,
         });
     }
     const int64_t per_block = (int64_t)wpb * G::GPW;
-    const int aw = p.apply_warps == kApplyWarpsAlone ? kApplyWarpsAlone : kApplyWarpsShared;
+    const int aw = p.apply_warps == kApplyWarpsAlone && D <= 128 ? kApplyWarpsAlone : kApplyWarpsShared;
+    // blocks for the short segments, at most (R-MAT 20 has about 3,000 of them
+    // a batch).  2^22 samples, one order BF16 with 152, 228 and 304 blocks of
+    // 16 warps: 7.36, 6.55 and 6.50 ms; both orders FP32 with 152, 304, 456 and
+    // 608 of 8: 12.44, 11.41, 11.24 and 11.46; d = 256 with 304 of 16: 5.27 for
+    // 2^19, with 608 of 8 (which leave registers for the gather's): 4.83
+    const int64_t short_blocks = aw == kApplyWarpsAlone ? 304 : D <= 128 ? 456 : 608;
     const int64_t apply_per_block = (int64_t)aw * G::GPW;
-    // long shared segments (more than kChunk entries, ~34 per batch on R-MAT 20)
-    // each get a CTA of their own
-    const int g_long = 64;
     cudaError_t e = cudaSuccess;
     for (int b = 0; b < p.n_batches && e == cudaSuccess; ++b) {
         const int64_t nb = std::min<int64_t>(p.batch, p.chunk_samples - (int64_t)b * p.batch);
@@ -1777,15 +1867,9 @@ static cudaError_t launch_data_batched(const DataParams& p, int warps_per_block,
         if (e != cudaSuccess) break;
         // a shared segment has two or more of the batch's nb * (K+2) entries
         const int64_t max_m = nb * (p.K + 2) / 2 + 1;
-        // short shared segments run about 10% of the batch's entries (R-MAT
-        // 20: ~2.9K of 28.7K); 2 blocks per SM leave room for the next kernel
-        const unsigned g2 = (unsigned)std::min<int64_t>((max_m + apply_per_block - 1) / apply_per_block, 152 * 2);
-        if (aw == kApplyWarpsAlone)
-            e = launch_pdl(k_apply<D, DT, kApplyWarpsAlone>, (unsigned)g_long + g2, kApplyWarpsAlone * 32, 0, s, true, p,
-                           b, g_long);
-        else
-            e = launch_pdl(k_apply<D, DT, kApplyWarpsShared>, (unsigned)g_long + g2, kApplyWarpsShared * 32, 0, s, true,
-                           p, b, g_long);
+        const unsigned g2 = 1024 / aw + (unsigned)std::min<int64_t>((max_m + apply_per_block - 1) / apply_per_block, short_blocks);
+        if (aw == kApplyWarpsAlone) e = launch_pdl(k_apply<D, DT, kApplyWarpsAlone>, g2, kApplyWarpsAlone * 32, 0, s, true, p, b);
+        else e = launch_pdl(k_apply<D, DT, kApplyWarpsShared>, g2, kApplyWarpsShared * 32, 0, s, true, p, b);
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -1884,10 +1968,8 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     // concurrent orders run the batched schedule
     const bool persistent = a.mode == LINE_MODE_PERSISTENT && !a.concurrent;
     const bool hogwild = a.mode == LINE_MODE_HOGWILD;  // records only: no grouping, slab or apply
-    // shared segments (two or more entries) and long ones (more than kChunk)
-    // per batch, at most
-    const uint32_t mcap = (uint32_t)(a.batch * R / 2 + 1);
-    const uint32_t lcap = (uint32_t)(a.batch * R / (kChunk + 1) + 1);
+    SegLayout sl;
+    sl.set(a.batch * R);
 
     cudaError_t e;
     auto ensure = [&](Buf& b, size_t bytes) -> bool {
@@ -1917,9 +1999,8 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
             return false;
         for (auto& cs : ws->set) {
             if (!f(cs.rec, sizeof(int32_t) * max_items) || !f(cs.bpar, sizeof(BatchParams) * (nb + 1)) ||
-                !f(cs.slot_info, sizeof(uint32_t) * max_items) || !f(cs.mdesc, sizeof(uint4) * (size_t)nb * mcap) ||
-                !f(cs.mcount, sizeof(uint32_t) * (nb + 1)) || !f(cs.ldesc, sizeof(uint4) * (size_t)nb * lcap) ||
-                !f(cs.lcount, sizeof(uint32_t) * (nb + 1)))
+                !f(cs.slot_info, sizeof(uint32_t) * max_items) || !f(cs.seg, sizeof(uint4) * (size_t)nb * sl.cap) ||
+                !f(cs.scount, sizeof(uint32_t) * (size_t)nb * kCounts))
                 return false;
             if (persistent && !f(cs.depmap, sizeof(uint32_t) * (size_t)nb * kDepWords)) return false;
         }
@@ -2004,8 +2085,7 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     gq.pcount = (uint32_t*)ws->pcount.p;
     gq.gcnt = (uint32_t*)ws->gcnt.p;
     gq.boff = (uint32_t*)ws->boff.p;
-    gq.mcap = mcap;
-    gq.lcap = lcap;
+    gq.sl = sl;
 
     uint32_t* abort_word = (uint32_t*)ws->counters.p + 16;
 
@@ -2016,8 +2096,7 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     dp.K = a.K;
     dp.n_nodes = a.n_nodes;
     dp.row_bits = row_bits;
-    dp.mcap = mcap;
-    dp.lcap = lcap;
+    dp.sl = sl;
     dp.slab = (float*)ws->slab.p;
     dp.batch = a.batch;
     dp.lambda = (float)a.lambda;
@@ -2054,8 +2133,7 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
         if (!hogwild) {
             pp.n_batches = cb;
             pp.bpar = (BatchParams*)cset.bpar.p;
-            pp.mcount = (uint32_t*)cset.mcount.p;
-            pp.lcount = (uint32_t*)cset.lcount.p;
+            pp.scount = (uint32_t*)cset.scount.p;
         }
         {
             const int64_t work = cs * (a.K + 1);
@@ -2074,10 +2152,8 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
             gq.chunk_samples = cs;
             gq.rec = (const int32_t*)cset.rec.p;
             gq.slot_info = (uint32_t*)cset.slot_info.p;
-            gq.mdesc = (uint4*)cset.mdesc.p;
-            gq.mcount = (uint32_t*)cset.mcount.p;
-            gq.ldesc = (uint4*)cset.ldesc.p;
-            gq.lcount = (uint32_t*)cset.lcount.p;
+            gq.seg = (uint4*)cset.seg.p;
+            gq.scount = (uint32_t*)cset.scount.p;
             gq.depmap = persistent ? (uint32_t*)cset.depmap.p : nullptr;
             if (persistent &&
                 (e = cudaMemsetAsync(cset.depmap.p, 0, sizeof(uint32_t) * (size_t)cb * kDepWords, ps)) != cudaSuccess)
@@ -2129,10 +2205,8 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
         } else {
             dp.rec = (const int32_t*)cset.rec.p;
             dp.slot_info = (const uint32_t*)cset.slot_info.p;
-            dp.mdesc = (const uint4*)cset.mdesc.p;
-            dp.mcount = (const uint32_t*)cset.mcount.p;
-            dp.ldesc = (const uint4*)cset.ldesc.p;
-            dp.lcount = (const uint32_t*)cset.lcount.p;
+            dp.seg = (const uint4*)cset.seg.p;
+            dp.scount = (const uint32_t*)cset.scount.p;
             dp.bpar = (const BatchParams*)cset.bpar.p;
             dp.depmap = (const uint32_t*)cset.depmap.p;
             dp.chunk_samples = cs;
