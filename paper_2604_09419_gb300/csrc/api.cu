@@ -68,6 +68,36 @@ cudaError_t grow(T** p, size_t* cap, size_t bytes) {
     return e;
 }
 
+// Scratch for one synchronous call: up to kKeptScratch bytes from the
+// context's buffer (grown, kept for later calls, freed by line_destroy: a
+// cudaMalloc and cudaFree per call cost 100-200 us), more from an allocation
+// of the call's own.
+constexpr size_t kKeptScratch = (size_t)256 << 20;
+struct Scratch {
+    void* p = nullptr;
+    bool own = false;
+    cudaError_t take(line_ctx* c, size_t bytes) {
+        own = bytes > kKeptScratch;
+        if (own) return cudaMalloc(&p, bytes);
+        cudaError_t e = grow(&c->scratch, &c->scratch_cap, bytes);
+        p = c->scratch;
+        return e;
+    }
+    ~Scratch() {
+        if (own && p) cudaFree(p);
+    }
+};
+inline size_t round256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+// Whether p is memory of the context's device (its kernels write there).
+bool on_device(const line_ctx* c, const void* p) {
+    cudaPointerAttributes attr;
+    const bool dev = cudaPointerGetAttributes(&attr, p) == cudaSuccess && attr.type == cudaMemoryTypeDevice &&
+                     attr.device == c->device;
+    cudaGetLastError();
+    return dev;
+}
+
 line_status ensure_row_ptr(line_ctx* c) {
     if (c->row_ptr_ok) return LINE_OK;
     cudaError_t e = grow(&c->row_ptr, &c->row_ptr_cap, sizeof(int64_t) * (size_t)(c->n_nodes + 1));
@@ -209,6 +239,7 @@ void line_destroy(line_ctx* c) {
     if (c->side) cudaStreamDestroy(c->side);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
+    if (c->scratch) cudaFree(c->scratch);
     if (c->status) cudaFree(c->status);
     if (c->dscratch) cudaFree(c->dscratch);
     if (c->ev0) cudaEventDestroy(c->ev0);
@@ -302,13 +333,18 @@ line_status line_get_alias(line_ctx* c, int table, uint32_t* thr, uint32_t* alia
         return fail(c, LINE_ERR_ARG, "line_get_alias: bad arguments");
     const int64_t n = table == LINE_TABLE_EDGE ? c->n_arcs : c->n_nodes;
     const uint2* tab = table == LINE_TABLE_EDGE ? c->edge_tab : c->neg_tab;
-    uint32_t* buf = nullptr;
-    CK(cudaMalloc(&buf, sizeof(uint32_t) * 2 * n), "alias export scratch");
+    if (on_device(c, thr) && on_device(c, alias) && !(((uintptr_t)thr | (uintptr_t)alias) & 3)) {
+        CK(export_alias(tab, n, thr, alias, c->stream), "line_get_alias");
+        CK(cudaStreamSynchronize(c->stream), "line_get_alias");
+        return LINE_OK;
+    }
+    Scratch sc;
+    CK(sc.take(c, sizeof(uint32_t) * 2 * n), "alias export scratch");
+    uint32_t* buf = (uint32_t*)sc.p;
     cudaError_t e = export_alias(tab, n, buf, buf + n, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(thr, buf, sizeof(uint32_t) * n, cudaMemcpyDefault, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(alias, buf + n, sizeof(uint32_t) * n, cudaMemcpyDefault, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(buf);
     if (e != cudaSuccess) return cuda_fail(c, e, "line_get_alias");
     return LINE_OK;
 }
@@ -655,18 +691,17 @@ line_status line_eval_loss(line_ctx* c, int order, int K, uint64_t seed, int64_t
         *out_host = 0.0;
         return LINE_OK;
     }
-    double* terms = nullptr;
-    void* tmp = nullptr;
-    cudaError_t e = cudaMalloc(&terms, sizeof(double) * m);
-    if (e == cudaSuccess) e = cudaMalloc(&tmp, fixed_sum_tmp_bytes(m));
+    Scratch sc;
+    const size_t term_bytes = round256(sizeof(double) * m);
+    cudaError_t e = sc.take(c, term_bytes + fixed_sum_tmp_bytes(m));
+    double* terms = (double*)sc.p;
+    void* tmp = (char*)sc.p + term_bytes;
     if (e == cudaSuccess)
         e = eval_loss_terms(t.U, order == 2 ? t.C : t.U, t.dtype, t.dim, K, c->src, c->dst, c->edge_tab, c->n_arcs,
                             c->neg_tab, c->n_nodes, seed, m, terms, c->stream);
     if (e == cudaSuccess) e = fixed_sum_f64(terms, m, (double*)tmp, c->dscratch, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out_host, c->dscratch, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (terms) cudaFree(terms);
-    if (tmp) cudaFree(tmp);
     if (e != cudaSuccess) return cuda_fail(c, e, "line_eval_loss");
     return LINE_OK;
 }
@@ -691,14 +726,14 @@ line_status line_eval_auc(line_ctx* c, int orders, int score, const int32_t* pos
         ++t.n;
     }
     const int64_t n = n_pos + n_neg;
-    int32_t* pairs = nullptr;
-    float* scores = nullptr;
-    void* tmp = nullptr;
     unsigned long long counts[2] = {0, 0};
     cudaStream_t s = c->stream;
-    cudaError_t e = cudaMalloc(&pairs, sizeof(int32_t) * 2 * n);
-    if (e == cudaSuccess) e = cudaMalloc(&scores, sizeof(float) * n);
-    if (e == cudaSuccess) e = cudaMalloc(&tmp, auc_tmp_bytes(n_pos, n_neg));
+    Scratch sc;
+    const size_t pair_bytes = round256(sizeof(int32_t) * 2 * n), score_bytes = round256(sizeof(float) * n);
+    cudaError_t e = sc.take(c, pair_bytes + score_bytes + auc_tmp_bytes(n_pos, n_neg));
+    int32_t* pairs = (int32_t*)sc.p;
+    float* scores = (float*)((char*)sc.p + pair_bytes);
+    void* tmp = (char*)sc.p + pair_bytes + score_bytes;
     int32_t* src = pairs;
     int32_t* dst = pairs + n;
     if (e == cudaSuccess) e = cudaMemcpyAsync(src, pos_src, sizeof(int32_t) * n_pos, cudaMemcpyDefault, s);
@@ -710,9 +745,6 @@ line_status line_eval_auc(line_ctx* c, int orders, int score, const int32_t* pos
         e = cudaMemcpyAsync(scores_out, scores, sizeof(float) * n, cudaMemcpyDefault, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(counts, tmp, sizeof counts, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (pairs) cudaFree(pairs);
-    if (scores) cudaFree(scores);
-    if (tmp) cudaFree(tmp);
     if (e != cudaSuccess) return cuda_fail(c, e, "line_eval_auc");
     if ((st = check_status(c, "line_eval_auc"))) return st;
     if (counts_out) {

@@ -55,6 +55,9 @@ struct line_ctx {
     void* alias_tmp = nullptr;
     // tables by order (index 1 and 2)
     line::Tables tab[3];
+    // scratch of the synchronous evaluation calls (take_scratch)
+    void* scratch = nullptr;
+    size_t scratch_cap = 0;
     // device status word and small scratch
     uint32_t* status = nullptr;
     uint32_t* flag = nullptr;

@@ -162,7 +162,8 @@ struct Transposed {
         }
         return m;
     }
-    static __device__ __forceinline__ void reduce(float (&s)[N], int lig) {
+    template <typename V>
+    static __device__ __forceinline__ void reduce(V (&s)[N], int lig) {
         int n = N;
 #pragma unroll
         for (int o = L / 2; o >= 1; o >>= 1) {
@@ -172,7 +173,7 @@ struct Transposed {
             for (int i = 0; i < (N + 1) / 2; ++i) {
                 if (i >= half) continue;
                 if (i + half < n) {
-                    const float keep = hi ? s[i + half] : s[i], give = hi ? s[i] : s[i + half];
+                    const V keep = hi ? s[i + half] : s[i], give = hi ? s[i] : s[i + half];
                     s[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
                 } else {
                     s[i] += __shfl_xor_sync(0xFFFFFFFFu, s[i], o);
