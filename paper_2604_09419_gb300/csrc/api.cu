@@ -98,19 +98,8 @@ bool on_device(const line_ctx* c, const void* p) {
     return dev;
 }
 
-line_status ensure_row_ptr(line_ctx* c) {
-    if (c->row_ptr_ok) return LINE_OK;
-    cudaError_t e = grow(&c->row_ptr, &c->row_ptr_cap, sizeof(int64_t) * (size_t)(c->n_nodes + 1));
-    if (e == cudaSuccess) e = row_offsets(c->n_nodes, c->n_arcs, c->src, c->row_ptr, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "row offsets");
-    c->row_ptr_ok = true;
-    return LINE_OK;
-}
-
 line_status ensure_walk_tables(line_ctx* c) {
     if (c->cw_ok) return LINE_OK;
-    line_status st = ensure_row_ptr(c);
-    if (st) return st;
     cudaError_t e = grow(&c->cw, &c->cw_cap, sizeof(double) * (size_t)std::max<int64_t>(1, c->n_arcs));
     if (e == cudaSuccess) e = walk_cumw(c->n_nodes, c->row_ptr, c->w, c->cw, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "walk sampler tables");
@@ -133,7 +122,7 @@ void free_tables(Tables& t) {
 // are built again for the next graph on first use); the graph, alias and
 // walk buffers stay allocated for the next build (release_graph frees them).
 void free_graph(line_ctx* c, bool keep_tables = false) {
-    c->row_ptr_ok = c->cw_ok = false;
+    c->cw_ok = false;
     c->w = nullptr;
     c->has_graph = false;
     if (keep_tables) return;
@@ -284,22 +273,31 @@ line_status line_build_alias(line_ctx* c, const line_graph_desc* g) {
                 break;
             }
         }
-        if ((e = validate_graph(n, m, c->src, c->dst, w, c->status, s)) != cudaSuccess) { result = cuda_fail(c, e, "validate"); break; }
-        if ((result = check_status(c, "line_build_alias"))) break;
+        // one pass over the arcs: validation, the row offsets (kept for the
+        // walk sampler and the MLP inputs), and the weights' integer sums
         const int64_t big = n > m ? n : m;
-        if ((e = grow(&c->alias_x, &c->x_cap, sizeof(double) * big)) != cudaSuccess) { result = cuda_fail(c, e, "alias scratch"); break; }
+        if ((e = grow(&c->row_ptr, &c->row_ptr_cap, sizeof(int64_t) * (size_t)(n + 1))) != cudaSuccess) { result = cuda_fail(c, e, "row offsets"); break; }
+        if ((e = grow(&c->alias_x, &c->x_cap, sizeof(double) * 2 * n)) != cudaSuccess) { result = cuda_fail(c, e, "alias scratch"); break; }
         if ((e = grow(&c->alias_tmp, &c->tmp_cap, alias_build_tmp_bytes(big))) != cudaSuccess) { result = cuda_fail(c, e, "alias scratch"); break; }
         double* x = c->alias_x;
+        unsigned long long* degi = reinterpret_cast<unsigned long long*>(x + n);
         void* tmp = c->alias_tmp;
+        GraphScan found{};
+        if ((e = scan_graph(n, m, c->src, c->dst, w, c->row_ptr, degi, (GraphScan*)tmp, c->status, s)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(&found, tmp, sizeof found, cudaMemcpyDeviceToHost, s)) != cudaSuccess) {
+            result = cuda_fail(c, e, "graph scan");
+            break;
+        }
+        if ((result = check_status(c, "line_build_alias"))) break;
+        // integer weights whose sum is below 2^53: every FP64 sum of them is
+        // exact, in any order
+        const bool whole = !found.frac && found.sum < (1ull << 53);
+        const double total_w = (double)found.sum;
         // edge table: arc weights (Algorithm 3)
-        if ((e = edge_weights(m, w, x, s)) != cudaSuccess) { result = cuda_fail(c, e, "edge weights"); break; }
-        if ((e = alias_build(x, m, c->edge_tab, tmp, c->status, s)) != cudaSuccess) { result = cuda_fail(c, e, "edge alias"); break; }
+        if ((e = alias_build_arcs(w, m, whole ? &total_w : nullptr, whole, c->edge_tab, tmp, c->status, s)) != cudaSuccess) { result = cuda_fail(c, e, "edge alias"); break; }
         if ((result = check_status(c, "line_build_alias (edges)"))) break;
-        // negative table: d(v)^0.75 (Eq. 1), each node's arcs found by the
-        // row offsets (kept for the walk sampler and the MLP inputs)
-        if ((e = grow(&c->row_ptr, &c->row_ptr_cap, sizeof(int64_t) * (size_t)(n + 1))) != cudaSuccess) { result = cuda_fail(c, e, "row offsets"); break; }
-        if ((e = row_offsets(n, m, c->src, c->row_ptr, s)) != cudaSuccess) { result = cuda_fail(c, e, "row offsets"); break; }
-        if ((e = neg_weights(n, m, c->row_ptr, w, x, c->deg, c->flag + 1, s)) != cudaSuccess) { result = cuda_fail(c, e, "degree weights"); break; }
+        // negative table: d(v)^0.75 (Eq. 1)
+        if ((e = neg_weights(n, c->row_ptr, w, degi, whole, x, c->deg, s)) != cudaSuccess) { result = cuda_fail(c, e, "degree weights"); break; }
         if ((e = alias_build(x, n, c->neg_tab, tmp, c->status, s)) != cudaSuccess) { result = cuda_fail(c, e, "negative alias"); break; }
         if ((result = check_status(c, "line_build_alias (negatives)"))) break;
     } while (false);
@@ -312,7 +310,6 @@ line_status line_build_alias(line_ctx* c, const line_graph_desc* g) {
     c->n_nodes = n;
     c->n_arcs = m;
     c->has_graph = true;
-    c->row_ptr_ok = true;
     return LINE_OK;
 }
 

@@ -38,12 +38,12 @@ struct line_ctx {
     int32_t* dst = nullptr;
     float* deg = nullptr;  // weighted out-degree of each node (FP64 sum, stored FP32)
     float* w = nullptr;    // arc weights (null: all 1)
-    // built on first use for the current graph (the *_ok flags): the first
-    // arc of each node (walks, MLP inputs) and the running FP64 weight sums
-    // per node (walks); their allocations outlive the graph, like src..deg
+    // the first arc of each node (walks, MLP inputs), and the running FP64
+    // weight sums per node (walks), built on first use for the current graph
+    // (cw_ok); their allocations outlive the graph, like src..deg
     int64_t* row_ptr = nullptr;
     double* cw = nullptr;
-    bool row_ptr_ok = false, cw_ok = false;
+    bool cw_ok = false;
     size_t row_ptr_cap = 0, cw_cap = 0;
     uint2* edge_tab = nullptr;
     uint2* neg_tab = nullptr;
@@ -85,9 +85,7 @@ line_status cuda_fail(line_ctx* c, cudaError_t e, const char* what);
 line_status enter(line_ctx* c);
 // Reads and clears the device status word (synchronises the stream).
 line_status check_status(line_ctx* c, const char* what, bool timeout_sticky = true);
-// Builds row_ptr if it is missing.
-line_status ensure_row_ptr(line_ctx* c);
-// Builds the walk sampler tables (row_ptr, cw) if they are missing.
+// Builds the walk sampler's table (cw) if it is missing.
 line_status ensure_walk_tables(line_ctx* c);
 
 // An NVTX range over an entry point's host scope (no cost unless a profiler

@@ -145,16 +145,25 @@ struct DeviceScratch {
 constexpr int kSumBlock = 1024;
 cudaError_t fixed_sum_f64(const double* x, int64_t n, double* tmp, double* out, cudaStream_t s);
 size_t fixed_sum_tmp_bytes(int64_t n);
-cudaError_t validate_graph(int64_t n_nodes, int64_t n_arcs, const int32_t* src, const int32_t* dst,
-                           const float* w, uint32_t* status, cudaStream_t s);
-cudaError_t edge_weights(int64_t n_arcs, const float* w, double* x, cudaStream_t s);
-// x[v] = d(v)^0.75; deg (nullable): d(v) rounded to FP32.  row_ptr: the
-// first arc of each node (row_offsets).  flag: one word of device scratch.
-cudaError_t neg_weights(int64_t n_nodes, int64_t n_arcs, const int64_t* row_ptr, const float* w, double* x, float* deg,
-                        uint32_t* flag, cudaStream_t s);
+// What one pass over the arcs finds besides errors (status) and the row offsets.
+struct GraphScan {
+    unsigned long long sum;  // of the weights, where all are integers in [1, 2^24]
+    uint32_t frac;           // 1: some weight is not
+    uint32_t pad;
+};
+cudaError_t scan_graph(int64_t n_nodes, int64_t n_arcs, const int32_t* src, const int32_t* dst, const float* w,
+                       int64_t* row_ptr, unsigned long long* degi, GraphScan* out, uint32_t* status, cudaStream_t s);
+// x[v] = d(v)^0.75; deg (nullable): d(v) rounded to FP32.  whole: d(v) = degi
+// (of scan_graph), else the sum of v's weights in arc order.
+cudaError_t neg_weights(int64_t n_nodes, const int64_t* row_ptr, const float* w, const unsigned long long* degi, bool whole,
+                        double* x, float* deg, cudaStream_t s);
 size_t alias_build_tmp_bytes(int64_t n);
 // Builds tab[n] = {thr, alias} from weights x[n] (FP64).  tmp: alias_build_tmp_bytes(n).
 cudaError_t alias_build(const double* x, int64_t n, uint2* tab, void* tmp, uint32_t* status, cudaStream_t s);
+// The same from positive FP32 arc weights (null: all 1).  total_w (nullable,
+// host): their fixed-order FP64 sum; whole: all are integers.
+cudaError_t alias_build_arcs(const float* w, int64_t n, const double* total_w, bool whole, uint2* tab, void* tmp,
+                             uint32_t* status, cudaStream_t s);
 
 // sample.cu
 cudaError_t sample_records(const int32_t* src, const int32_t* dst, const uint2* edge_tab, int64_t n_arcs,
@@ -187,8 +196,6 @@ struct WalkParams {
     int32_t* rec;            // rec[s R], rec[s R + 1] = the pair of sample t0 + s
 };
 size_t walk_smem_bytes(int L);
-// row_ptr[n+1]: first arc of each node, from the sorted src.
-cudaError_t row_offsets(int64_t n_nodes, int64_t n_arcs, const int32_t* src, int64_t* row_ptr, cudaStream_t s);
 // cw[m]: running FP64 sums of each node's arc weights (w nullable: weight 1).
 cudaError_t walk_cumw(int64_t n_nodes, const int64_t* row_ptr, const float* w, double* cw, cudaStream_t s);
 cudaError_t walk_pairs(const WalkParams& p, cudaStream_t s);

@@ -1425,7 +1425,6 @@ static line_status mlp_features_impl(line_ctx* c, const char* what, const uint8_
     MlpState& s = *c->mlp;
     if (rows && n_rows == 0) return LINE_OK;
     const Tables& t = c->tab[s.order];
-    if ((st = ensure_row_ptr(c))) return st;
     // scratch kept in the MLP state (grown, never shrunk)
     const int64_t max_hubs = HubScratch(c->n_nodes, c->n_arcs).max_hubs;
     cudaError_t e = cudaSuccess;

@@ -81,31 +81,40 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t n, Gen gen
 // *grand (device pointer, may be null).
 template <typename T>
 __global__ void __launch_bounds__(1024) k_scan_tiles(int64_t ntiles, T* tile_sums, T* grand) {
-    __shared__ T part[1024];
     __shared__ T warp_tot[32];
     const int64_t per = (ntiles + 1023) / 1024;
     const int64_t lo = (int64_t)threadIdx.x * per;
     T acc = zero_of<T>();
     for (int64_t i = lo; i < lo + per && i < ntiles; ++i) acc = acc + tile_sums[i];
-    part[threadIdx.x] = acc;
+    // exclusive scan of the threads' sums: warps, then their totals
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T incl = acc;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        T o = shfl_up(incl, d);
+        if (lane >= d) incl = o + incl;
+    }
+    if (lane == 31) warp_tot[warp] = incl;
+    T run = shfl_up(incl, 1);
+    if (lane == 0) run = zero_of<T>();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        T run = zero_of<T>();
-        for (int i = 0; i < 1024; ++i) {
-            T v = part[i];
-            part[i] = run;
-            run = run + v;
+    if (warp == 0) {
+        T w = warp_tot[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            T o = shfl_up(w, d);
+            if (lane >= d) w = o + w;
         }
-        warp_tot[0] = run;
+        warp_tot[lane] = w;
     }
     __syncthreads();
-    T run = part[threadIdx.x];
+    if (warp > 0) run = warp_tot[warp - 1] + run;
     for (int64_t i = lo; i < lo + per && i < ntiles; ++i) {
         T v = tile_sums[i];
         tile_sums[i] = run;
         run = run + v;
     }
-    if (threadIdx.x == 0 && grand) *grand = warp_tot[0];
+    if (threadIdx.x == 0 && grand) *grand = warp_tot[31];
 }
 
 template <typename T, typename Gen, typename Out>

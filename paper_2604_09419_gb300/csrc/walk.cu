@@ -27,17 +27,6 @@ namespace {
 constexpr uint32_t kWalkDomain = 8u;
 constexpr int kWalkWarps = 4;
 
-// row_ptr[v] = first arc of v (src sorted), row_ptr[n] = n_arcs.  Arc e in
-// [0, m] fills the nodes between src[e-1] and src[e] (src[m] read as n).
-__global__ void k_row_ptr(const int32_t* __restrict__ src, int64_t n_arcs, int64_t n_nodes,
-                          int64_t* __restrict__ row_ptr) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e <= n_arcs; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t hi = e < n_arcs ? (int64_t)src[e] : n_nodes;
-        const int64_t lo = e > 0 ? (int64_t)src[e - 1] + 1 : 0;
-        for (int64_t v = lo; v <= hi; ++v) row_ptr[v] = e;
-    }
-}
-
 // cw[e]: running sum of the weights of src[e]'s arcs up to e, left to right
 // in FP64 (one thread per node, so the rounding order is the arc order).
 __global__ void k_cumw(const int64_t* __restrict__ row_ptr, const float* __restrict__ w, int64_t n_nodes,
@@ -158,12 +147,6 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_walk_pairs(WalkParams p) {
 }  // namespace
 
 size_t walk_smem_bytes(int L) { return sizeof(int32_t) * (size_t)kWalkWarps * (size_t)(L + 1); }
-
-cudaError_t row_offsets(int64_t n_nodes, int64_t n_arcs, const int32_t* src, int64_t* row_ptr, cudaStream_t s) {
-    const unsigned g = (unsigned)std::min<int64_t>((n_arcs + 1 + 255) / 256, 152 * 32);
-    k_row_ptr<<<g, 256, 0, s>>>(src, n_arcs, n_nodes, row_ptr);
-    return cudaGetLastError();
-}
 
 cudaError_t walk_cumw(int64_t n_nodes, const int64_t* row_ptr, const float* w, double* cw, cudaStream_t s) {
     const unsigned g = (unsigned)std::min<int64_t>((n_nodes + 127) / 128, 152 * 32);
