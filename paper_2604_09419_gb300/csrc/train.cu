@@ -169,6 +169,27 @@ __device__ __forceinline__ T rec_entry(uint32_t gm, T held, const T* row, int id
 // Per-sample work.
 // ctx_stage: this warp's shared staging area, (K+1) x 32 lanes x E floats.
 // ---------------------------------------------------------------------------
+// The K+2 <= JB+1 record entries and places of a lane group's sample, entry i
+// in lane i mod L.
+template <int L, int JB>
+struct Held {
+    static constexpr int H = (JB + L) / L;
+    int32_t r[H];
+    uint32_t i[H];
+    __device__ __forceinline__ void load(const DataParams& p, int64_t s_local, int lig, bool active) {
+        const int R = p.K + 2;
+        const int64_t at = (active ? s_local : 0) * R;
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            const bool in = active && k * L + lig < R;
+            r[k] = in ? p.rec[at + k * L + lig] : 0;
+            i[k] = in ? p.slot_info[at + k * L + lig] : 0u;
+        }
+    }
+    __device__ __forceinline__ int32_t row(uint32_t gm, int idx) const { return __shfl_sync(gm, r[idx / L], idx % L, L); }
+    __device__ __forceinline__ uint32_t place(uint32_t gm, int idx) const { return __shfl_sync(gm, i[idx / L], idx % L, L); }
+};
+
 // Register-resident gather body for K + 1 <= JB: the K+1 context rows stay in
 // registers; the dots and their reductions are independent chains.  Same
 // arithmetic, in the same order, as the staged body.
@@ -183,17 +204,16 @@ __device__ __forceinline__ T rec_entry(uint32_t gm, T held, const T* row, int id
 // order in BF16: 7.80 -> 6.69 ms; both orders FP32 12.09 -> 11.75.
 template <int D, int DT, int JB>
 __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bool active, float eta, uint32_t salt,
-                                                uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
-                                                const uint32_t* info) {
+                                                uint32_t gm, const Held<Geom<D, DT>::L, JB>& h) {
     using G = Geom<D, DT>;
     using T = Transposed<G::L, JB>;
-    const int32_t u = __shfl_sync(gm, r0, 0, G::L);
+    const int32_t u = h.row(gm, 0);
     float xu[G::E];
     float c[JB][G::E];
     load_row<D, DT>(p.U, u, lig, xu);
 #pragma unroll
     for (int j = 0; j < JB; ++j) {
-        const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active && j <= p.K);
+        const int32_t y = h.row(gm, 1 + j);
         if (j <= p.K) {
             load_row<D, DT>(p.C, y, lig, c[j]);
         } else {
@@ -224,8 +244,8 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
         if (j > p.K) continue;
         const float g = __shfl_sync(0xFFFFFFFFu, gv[T::slot(j)], T::lane(j), G::L);
         vfma(du, g, c[j], du);
-        const uint32_t inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
-        const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
+        const uint32_t inf = h.place(gm, 1 + j);
+        const int32_t y = h.row(gm, 1 + j);
         const bool single = (inf & kSingleBit) != 0;
         // a singleton's new row c - decay c + g x, or the contribution g x
         float x[G::E];
@@ -253,7 +273,7 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
             }
         }
     }
-    const uint32_t inf0 = shfl_w(gm, i0, 0, G::L);
+    const uint32_t inf0 = h.place(gm, 0);
     if (active) {
         if (inf0 & kSingleBit) {
             vfma(xu, -((float)(p.K + 1) * decay), xu, xu);
@@ -557,19 +577,23 @@ __global__ void __launch_bounds__(kGatherWarps * 32, 8) k_gather(DataParams p, i
     const int64_t s_end = min(s_begin + p.batch, p.chunk_samples);
     const int64_t s_local = s_begin + ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * G::GPW + grp;
     const bool active = s_local < s_end;
-    const int R = p.K + 2;
-    const int64_t sbase = (active ? s_local : 0) * R;
-    const int32_t* rec = p.rec + sbase;
-    const uint32_t* info = p.slot_info + sbase;
     const uint32_t gm = group_mask<G::L>(grp);
     // the chunk's index data comes from the pre-pass: read before the wait
-    const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
-    const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
+    // (which has no effect without a programmatic launch)
     const BatchParams bp = p.bpar[b];
-    pdl_wait();  // the tables' rows: written by the previous kernel (no effect without a programmatic launch)
     if constexpr (JB > 0) {
-        sample_body_reg<D, DT, JB>(p, lig, active, bp.eta, bp.salt, gm, r0, i0, rec, info);
+        Held<G::L, JB> h;
+        h.load(p, s_local, lig, active);
+        pdl_wait();  // the tables' rows: written by the previous kernel
+        sample_body_reg<D, DT, JB>(p, lig, active, bp.eta, bp.salt, gm, h);
     } else {
+        const int R = p.K + 2;
+        const int64_t sbase = (active ? s_local : 0) * R;
+        const int32_t* rec = p.rec + sbase;
+        const uint32_t* info = p.slot_info + sbase;
+        const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
+        const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
+        pdl_wait();
         float* stage = reinterpret_cast<float*>(smem4) + (size_t)warp * (p.K + 1) * 32 * G::E;
         sample_body_staged<D, DT>(p, lig, lane, active, bp.eta, bp.salt, gm, r0, i0, rec, info, stage);
     }
@@ -1710,19 +1734,26 @@ struct Buf {
     }
 };
 
+// A data phase captured as a CUDA graph, and what it was captured for: the
+// parameters, the warps per block and the kernels (the launcher of one row
+// width and table type: tables of another type can sit at the same addresses).
+struct CapturedPhase {
+    using Fn = cudaError_t (*)(const DataParams&, int, cudaStream_t);
+    cudaGraphExec_t exec = nullptr;  // null: `key` was met, not captured yet
+    DataParams key{};
+    int wpb = -1;
+    Fn fn = nullptr;
+    bool is(const DataParams& k, int w, Fn f) const { return fn == f && wpb == w && memcmp(&k, &key, sizeof k) == 0; }
+};
+
 // Per-chunk outputs of the pre-pass, read by the data phase.  Two sets: the
 // pre-pass of chunk c+1 (on its own low-priority stream) fills one while the
 // data phase of chunk c reads the other.
 struct ChunkSet {
     Buf rec, slot_info, depmap, seg, scount, bpar;
-    // captured data phase of a full chunk of this set, and what it was
-    // captured for: the parameters, the warps per block and the kernels (the
-    // launcher of one row width and table type: tables of another type can
-    // sit at the same addresses)
-    cudaGraphExec_t graph = nullptr;
-    DataParams graph_key{};
-    int graph_wpb = -1;
-    cudaError_t (*graph_fn)(const DataParams&, int, cudaStream_t) = nullptr;
+    // captured data phases of this set: of a full chunk, and of the shorter
+    // one that ends a call
+    CapturedPhase captured[2];
     cudaEvent_t prep_done = nullptr;  // pre-pass of the set's current chunk finished
     cudaEvent_t data_done = nullptr;  // data phase of the set's previous chunk finished
     bool data_pending = false;
@@ -1771,7 +1802,8 @@ struct TrainWorkspace {
         for (auto& cs : set) {
             if (cs.prep_done) cudaEventDestroy(cs.prep_done);
             if (cs.data_done) cudaEventDestroy(cs.data_done);
-            if (cs.graph) cudaGraphExecDestroy(cs.graph);
+            for (auto& g : cs.captured)
+                if (g.exec) cudaGraphExecDestroy(g.exec);
         }
         if (start) cudaEventDestroy(start);
         if (prep_end) cudaEventDestroy(prep_end);
@@ -2212,14 +2244,19 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
             dp.chunk_samples = cs;
             dp.n_batches = cb;
             if (persistent && (e = cudaMemsetAsync(abort_word, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
-            if (!persistent && a.graph && !ws->graph_failed && cs == max_chunk && c > 0) {
-                // a full chunk: replay this set's captured data phase (what
-                // differs from chunk to chunk is in the set's buffers)
-                DataParams key = dp;
-                if (!cset.graph || cset.graph_wpb != a.warps_per_block || cset.graph_fn != data ||
-                    memcmp(&key, &cset.graph_key, sizeof key) != 0) {
-                    if (cset.graph) cudaGraphExecDestroy(cset.graph);
-                    cset.graph = nullptr;
+            // A chunk's launches are replayed from a captured graph (what differs
+            // from chunk to chunk is in the set's buffers) when it is a full chunk
+            // after the first of its call, or when the set's last chunk of its
+            // kind, full or not, was the same: a call of few chunks that is
+            // repeated.  A launch costs 2.3 us of host time, two a batch: with
+            // both orders at B = 256 the launches, not the GPU, set the pace
+            // (7.7 us a batch; 4.6 replayed).
+            CapturedPhase& cap = cset.captured[cs == max_chunk ? 0 : 1];
+            const bool known = cap.is(dp, a.warps_per_block, data);
+            if (!persistent && a.graph && !ws->graph_failed && (known || (cs == max_chunk && c > 0))) {
+                if (!known || !cap.exec) {
+                    if (cap.exec) cudaGraphExecDestroy(cap.exec);
+                    cap = CapturedPhase{};
                     cudaGraph_t g = nullptr;
                     cudaError_t ce = cudaStreamBeginCapture(ws->cap, cudaStreamCaptureModeThreadLocal);
                     if (ce == cudaSuccess) {
@@ -2227,24 +2264,25 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
                         ce = cudaStreamEndCapture(ws->cap, &g);
                         if (ce == cudaSuccess) ce = le;
                     }
-                    if (ce == cudaSuccess) ce = cudaGraphInstantiate(&cset.graph, g, 0);
+                    if (ce == cudaSuccess) ce = cudaGraphInstantiate(&cap.exec, g, 0);
                     if (g) cudaGraphDestroy(g);
                     if (ce != cudaSuccess) {
                         cudaGetLastError();
-                        cset.graph = nullptr;
+                        cap.exec = nullptr;
                         ws->graph_failed = true;
                     } else {
-                        cset.graph_key = key;
-                        cset.graph_wpb = a.warps_per_block;
-                        cset.graph_fn = data;
+                        cap.key = dp;
+                        cap.wpb = a.warps_per_block;
+                        cap.fn = data;
                     }
                 }
-                if (cset.graph) {
-                    if ((e = cudaGraphLaunch(cset.graph, s)) != cudaSuccess) return e;
-                } else {
-                    if ((e = data(dp, a.warps_per_block, s)) != cudaSuccess) return e;
-                }
+                e = cap.exec ? cudaGraphLaunch(cap.exec, s) : data(dp, a.warps_per_block, s);
+                if (e != cudaSuccess) return e;
             } else {
+                if (!persistent && !known) {
+                    if (cap.exec) cudaGraphExecDestroy(cap.exec);
+                    cap = CapturedPhase{nullptr, dp, a.warps_per_block, data};
+                }
                 if ((e = data(dp, a.warps_per_block, s)) != cudaSuccess) return e;
             }
         }
