@@ -288,37 +288,58 @@ __device__ __forceinline__ void sample_body_reg(const DataParams& p, int lig, bo
     }
 }
 
-// Staged gather body (any K): the K+1 context rows are staged in shared
-// memory (ctx_stage: (K+1) x 32 lanes x E floats), the dots reduced JB at a
-// time.  Same arithmetic, in the same order, as the register body.
+// This lane's values of row j of a set of staged rows (D values each in the
+// table's type, in shared memory).
 template <int D, int DT>
-__device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig, int lane, bool active, float eta,
-                                                   uint32_t salt, uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
-                                                   const uint32_t* info, float* ctx_stage) {
+__device__ __forceinline__ void slot_row(const unsigned char* set, int j, int lig, float (&v)[Geom<D, DT>::E]) {
     using G = Geom<D, DT>;
-    constexpr int CH = G::E <= 4 ? 8 : 4;  // context rows in flight per lane
-    const int32_t u = __shfl_sync(gm, r0, 0, G::L);
-    float xu[G::E];
-    load_row<D, DT>(p.U, u, lig, xu);
-    for (int j0 = 0; j0 <= p.K; j0 += CH) {
-        float c[CH][G::E];
+    if constexpr (DT == LINE_DTYPE_F32) {
+        const float4* q = reinterpret_cast<const float4*>(set + (size_t)j * D * 4 + (size_t)lig * G::E * 4);
 #pragma unroll
-        for (int jj = 0; jj < CH; ++jj) {
-            const int j = j0 + jj;
-            int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active && j <= p.K);
-            if (j <= p.K) load_row<D, DT>(p.C, y, lig, c[jj]);
+        for (int k = 0; k < G::NV; ++k) {
+            const float4 a = q[k];
+            v[4 * k] = a.x;
+            v[4 * k + 1] = a.y;
+            v[4 * k + 2] = a.z;
+            v[4 * k + 3] = a.w;
         }
+    } else {
+        const uint2* q = reinterpret_cast<const uint2*>(set + (size_t)j * D * 2 + (size_t)lig * G::E * 2);
 #pragma unroll
-        for (int jj = 0; jj < CH; ++jj) {
-            const int j = j0 + jj;
-            if (j <= p.K) {
-                float4* st = reinterpret_cast<float4*>(ctx_stage + (j * 32 + lane) * G::E);
-#pragma unroll
-                for (int q = 0; q < G::E / 4; ++q)
-                    st[q] = make_float4(c[jj][4 * q], c[jj][4 * q + 1], c[jj][4 * q + 2], c[jj][4 * q + 3]);
-            }
+        for (int k = 0; k < G::NV; ++k) {
+            const uint2 a = q[k];
+            v[4 * k] = __uint_as_float(a.x << 16);
+            v[4 * k + 1] = __uint_as_float(a.x & 0xFFFF0000u);
+            v[4 * k + 2] = __uint_as_float(a.y << 16);
+            v[4 * k + 3] = __uint_as_float(a.y & 0xFFFF0000u);
         }
     }
+}
+
+// Staged gather body (any K): the K+1 context rows come into shared memory by
+// asynchronous 16-byte copies past L1 (stage: (K+1) D values of the table's
+// type per lane group), all in flight at once and without registers; the dots
+// are reduced JB at a time.  Same arithmetic, in the same order, as the
+// register body.  Rows moved through registers, four or eight at a time,
+// waited for memory two or three times a sample: 2^19 samples at d = 256,
+// K = 10 took 4.62 ms, like this 3.72 (BF16 4.00 and 2.98; d = 64, K = 10, B = 4096:
+// 1.71 and 1.35).
+template <int D, int DT>
+__device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig, bool active, float eta, uint32_t salt,
+                                                   uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
+                                                   const uint32_t* info, unsigned char* stage) {
+    using G = Geom<D, DT>;
+    constexpr int kRowBytes = D * (DT == LINE_DTYPE_F32 ? 4 : 2);
+    const int32_t u = __shfl_sync(gm, r0, 0, G::L);
+    for (int j = 0; j <= p.K; ++j) {
+        const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
+        const unsigned char* from = reinterpret_cast<const unsigned char*>(p.C) + (int64_t)y * kRowBytes;
+        for (int o = lig * 16; o < kRowBytes; o += G::L * 16) cp_async16(stage + j * kRowBytes + o, from + o);
+    }
+    float xu[G::E];
+    load_row<D, DT>(p.U, u, lig, xu);
+    cp_async_wait_all();
+    __syncwarp(gm);
     const uint32_t ctx_table = p.order == 2 ? 1u : 0u;
     const float etalam = eta * p.lambda;
     float du[G::E];
@@ -332,15 +353,10 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
         for (int jj = 0; jj < JB; ++jj) {
             sj[jj] = 0.0f;
             if (j0 + jj <= p.K) {
-                const float4* ld = reinterpret_cast<const float4*>(ctx_stage + ((j0 + jj) * 32 + lane) * G::E);
+                float c[G::E];
+                slot_row<D, DT>(stage, j0 + jj, lig, c);
 #pragma unroll
-                for (int q = 0; q < G::E / 4; ++q) {
-                    const float4 a = ld[q];
-                    sj[jj] = fmaf(xu[4 * q], a.x, sj[jj]);
-                    sj[jj] = fmaf(xu[4 * q + 1], a.y, sj[jj]);
-                    sj[jj] = fmaf(xu[4 * q + 2], a.z, sj[jj]);
-                    sj[jj] = fmaf(xu[4 * q + 3], a.w, sj[jj]);
-                }
+                for (int e = 0; e < G::E; ++e) sj[jj] = fmaf(xu[e], c[e], sj[jj]);
             }
         }
         T::reduce(sj, lig);
@@ -355,15 +371,7 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
             const int j = j0 + jj;
             if (j > p.K) break;
             float c[G::E];
-            const float4* ld = reinterpret_cast<const float4*>(ctx_stage + (j * 32 + lane) * G::E);
-#pragma unroll
-            for (int q = 0; q < G::E / 4; ++q) {
-                const float4 a = ld[q];
-                c[4 * q] = a.x;
-                c[4 * q + 1] = a.y;
-                c[4 * q + 2] = a.z;
-                c[4 * q + 3] = a.w;
-            }
+            slot_row<D, DT>(stage, j, lig, c);
             const float g = __shfl_sync(0xFFFFFFFFu, gv[T::slot(jj)], T::lane(jj), G::L);
             vfma(du, g, c, du);
             const uint32_t inf = rec_entry<G::L>(gm, i0, info, 1 + j, active);
@@ -371,16 +379,14 @@ __device__ __forceinline__ void sample_body_staged(const DataParams& p, int lig,
             if (active) {
                 if (inf & kSingleBit) {
                     // the only reader of row y in this batch: write it now
-                    const float decay = 1.0f * etalam;
-                    float x[G::E];
-#pragma unroll
-                    for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[e], c[e]) + g * xu[e];
-                    store_row<D, DT>(p.C, y, lig, x, salt, ctx_table);
+                    vfma(c, -etalam, c, c);
+                    vfma(c, g, xu, c);
+                    store_row<D, DT>(p.C, y, lig, c, salt, ctx_table);
                 } else {
+                    vmul(c, g, xu);
                     float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
 #pragma unroll
-                    for (int q = 0; q < G::E / 4; ++q)
-                        st_cg(dst + q, make_float4(g * xu[4 * q], g * xu[4 * q + 1], g * xu[4 * q + 2], g * xu[4 * q + 3]));
+                    for (int q = 0; q < G::E / 4; ++q) st_cg(dst + q, make_float4(c[4 * q], c[4 * q + 1], c[4 * q + 2], c[4 * q + 3]));
                 }
             }
         }
@@ -594,8 +600,9 @@ __global__ void __launch_bounds__(kGatherWarps * 32, 8) k_gather(DataParams p, i
         const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
         const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
         pdl_wait();
-        float* stage = reinterpret_cast<float*>(smem4) + (size_t)warp * (p.K + 1) * 32 * G::E;
-        sample_body_staged<D, DT>(p, lig, lane, active, bp.eta, bp.salt, gm, r0, i0, rec, info, stage);
+        unsigned char* stage = reinterpret_cast<unsigned char*>(smem4) +
+                               (size_t)(warp * G::GPW + grp) * (p.K + 1) * D * (DT == LINE_DTYPE_F32 ? 4 : 2);
+        sample_body_staged<D, DT>(p, lig, active, bp.eta, bp.salt, gm, r0, i0, rec, info, stage);
     }
 }
 
@@ -750,32 +757,6 @@ __device__ __forceinline__ bool grid_barrier(const DataParams& p, uint32_t r, ui
 // One lane group's sample from its staged rows (slot: row 0 = U[u], rows
 // 1..K+1 = the context rows, D values each in the table's type).  The
 // arithmetic is sample_body_staged's, in the same order.
-template <int D, int DT>
-__device__ __forceinline__ void slot_row(const unsigned char* set, int j, int lig, float (&v)[Geom<D, DT>::E]) {
-    using G = Geom<D, DT>;
-    if constexpr (DT == LINE_DTYPE_F32) {
-        const float4* q = reinterpret_cast<const float4*>(set + (size_t)j * D * 4 + (size_t)lig * G::E * 4);
-#pragma unroll
-        for (int k = 0; k < G::NV; ++k) {
-            const float4 a = q[k];
-            v[4 * k] = a.x;
-            v[4 * k + 1] = a.y;
-            v[4 * k + 2] = a.z;
-            v[4 * k + 3] = a.w;
-        }
-    } else {
-        const uint2* q = reinterpret_cast<const uint2*>(set + (size_t)j * D * 2 + (size_t)lig * G::E * 2);
-#pragma unroll
-        for (int k = 0; k < G::NV; ++k) {
-            const uint2 a = q[k];
-            v[4 * k] = __uint_as_float(a.x << 16);
-            v[4 * k + 1] = __uint_as_float(a.x & 0xFFFF0000u);
-            v[4 * k + 2] = __uint_as_float(a.y << 16);
-            v[4 * k + 3] = __uint_as_float(a.y & 0xFFFF0000u);
-        }
-    }
-}
-
 template <int D, int DT>
 __device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, bool active, float eta, uint32_t salt,
                                                  uint32_t gm, int32_t r0, uint32_t i0, const int32_t* rec,
@@ -1835,9 +1816,11 @@ static void once_per_device(std::atomic<uint64_t>& done, F f) {
 // exceed the shared memory) and its shared memory.
 template <int D, int DT>
 static int staged_warps(int K, int requested, size_t* smem_out) {
-    // staging: (K+1) context rows x 32 lanes x E floats per warp
-    const size_t per_warp = (size_t)(K + 1) * 32 * Geom<D, DT>::E * sizeof(float);
-    const int wpb = requested > 0 ? std::min(requested, kGatherWarps) : kGatherWarps;
+    // staging: K+1 context rows per lane group
+    const size_t per_warp = (size_t)(K + 1) * Geom<D, DT>::GPW * D * (DT == LINE_DTYPE_F32 ? 4 : 2);
+    // (2 warps a block: 3.72 ms for 2^19 samples at d = 256, K = 10, with 4
+    // 3.99; narrower rows within 1%)
+    const int wpb = requested > 0 ? std::min(requested, kGatherWarps) : 2;
     const int fit = std::max(1, std::min(wpb, (int)(kMaxSmem / per_warp)));
     *smem_out = (size_t)fit * per_warp;
     return fit;
