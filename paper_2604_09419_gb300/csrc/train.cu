@@ -1453,11 +1453,11 @@ __global__ void __launch_bounds__(kSortThreads) k_bucket_sort(GroupParams q) {
 //      indexed by hrow, record which bits are hit and which are hit twice.
 //      On R-MAT 20 73% of a batch's items are such rows; they (but for about
 //      one in ten, which shares its bit) get the singleton mark at once.
-//   2. The other items ("candidates") are counted into 1,024 sub-buckets by
+//   2. The other items ("candidates") are counted into 4,096 sub-buckets by
 //      further hrow bits and placed there as keys (hrow(row) << 32 | sample,
 //      slot), in no particular order.
 //   3. One thread per key compares it with the keys of its sub-bucket (about
-//      five): the keys of smaller rows, of its own row, and those of its row
+//      three): the keys of smaller rows, of its own row, and those of its row
 //      that come before it give its position, its segment's head and length.
 //      Nothing is sorted.  Only a sub-bucket of more than kRankMax keys (a
 //      hub row) is sorted, by one warp.
@@ -1465,18 +1465,21 @@ __global__ void __launch_bounds__(kSortThreads) k_bucket_sort(GroupParams q) {
 // slot) order; where a part begins depends on the order in which the parts
 // arrive, which no result depends on.
 // Bound: issue slots and the latency of the three scans.  A chunk of 64
-// batches of 28,672 items (R-MAT 20, d = 128, K = 5) takes 36 us with nothing
-// beside it and 38-41 beside the data phase, on 128 CTAs; the earlier form,
-// which sorted all items of a batch in an 8-CTA cluster, 107 and 118 on 512.
-// 16 batches of 114,688 items (8 parts each): 82 us against 276 for the
-// three kernels below.  One order at B = 4096 went from 8.74 to 7.80 ms for
+// batches of 28,672 items (R-MAT 20, d = 128, K = 5) takes 31 us with nothing
+// beside it and 32 beside the data phase, on 128 CTAs (36 and 38-41 with 1,024
+// sub-buckets and a reservation of list places per warp and round); the
+// earlier form, which sorted all items of a batch in an 8-CTA cluster, 107 and
+// 118 on 512.  16 batches of 114,688 items (8 parts each): 78 us against 276
+// for the three kernels below.  One order at B = 4096 went from 8.74 to 7.80 ms for
 // 2^22 samples (BF16), both orders from 13.99 to 12.09 (FP32).  Beyond 16
 // parts every part's scan of the whole batch costs more than it saves.
 constexpr int kPartThreads = 1024;
 constexpr uint32_t kPartItems2 = 16384;  // a part's share of the items, at most
 constexpr uint32_t kPartCap = 15360;     // keys held in shared memory; more go to the scratch array
 constexpr int kPartMaxLog = 4;
-constexpr int kPartSub = 1024;           // sub-buckets of a part (one per thread)
+constexpr int kLogSub = 12;
+constexpr int kPartSub = 1 << kLogSub;   // sub-buckets of a part (four per thread)
+constexpr uint32_t kFound = 1u << (17 - 5 + 1);  // results kept in the bitmaps' place
 constexpr uint32_t kMapBits = 17;
 constexpr uint32_t kRankMax = 128;
 
@@ -1550,17 +1553,21 @@ __device__ __forceinline__ void list_segments(const GroupParams& q, int b, bool 
 }
 
 // Steps 2b and 3 for the part's nc keys, grouped by sub-bucket in a (shared
-// memory, or the scratch array; inlined for each).
+// memory, or the scratch array; inlined for each).  found: room for kFound
+// results (the bitmaps, no longer needed): with at most so many keys the
+// segments are counted first, and listed after one reservation of the part's
+// places (a reservation per warp and round costs a round trip to L2 each).
 __device__ __forceinline__ void group_segments(const GroupParams& q, const uint64_t* a, uint64_t* aw, uint32_t nc,
                                                const uint32_t* start, int log_parts, uint32_t pbase, int b,
-                                               const uint16_t* big, uint32_t nbig) {
+                                               const uint16_t* big, uint32_t nbig, uint32_t* found, uint32_t* lcnt) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool later = nc <= kFound;
     for (uint32_t i0 = warp * 32; i0 < nc; i0 += kPartThreads) {
         const uint32_t i = i0 + lane;
         bool mine = i < nc;
         const uint64_t key = mine ? a[i] : 0ull;
         const uint32_t hv = (uint32_t)(key >> 32), v = (uint32_t)key;
-        const uint32_t sub = (hv << log_parts) >> (32 - 10);
+        const uint32_t sub = (hv << log_parts) >> (32 - kLogSub);
         const uint32_t s0 = start[sub], c = start[sub + 1] - s0;
         mine = mine && c <= kRankMax;
         uint32_t lower = 0, same = 0, before = 0, z = 0;
@@ -1578,7 +1585,44 @@ __device__ __forceinline__ void group_segments(const GroupParams& q, const uint6
         }
         const uint32_t head = pbase + s0 + lower;
         if (mine) q.slot_info[(v >> kSlotBits) * q.R + (v & kSlotMask)] = same == 1 ? kSingleBit : head + before;
-        list_segments(q, b, mine && before == 0, head, same, hv, z);
+        const bool is_head = mine && before == 0;
+        if (later) {
+            // lower, same, z <= kRankMax = 2^7: 8 bits each
+            const bool m = is_head && same > 1;
+            if (i < nc) found[i] = m ? (1u << 31) | (lower << 16) | (same << 8) | z : 0u;
+            const int cls = m ? seg_class(same) : kClasses + 1;
+#pragma unroll
+            for (int cc = 0; cc < kClasses; ++cc) {
+                const uint32_t mk = __ballot_sync(0xFFFFFFFFu, cls == cc);
+                if (mk && lane == 0) atomicAdd(lcnt + cc, (uint32_t)__popc(mk));
+            }
+        } else {
+            list_segments(q, b, is_head, head, same, hv, z);
+        }
+    }
+    if (later) {
+        __syncthreads();
+        if (warp == 0) {
+            // lane c reserves the part's places of list c
+            uint32_t n = lane < kClasses ? lcnt[lane] : 0u;
+            const uint32_t longs = __reduce_add_sync(0xFFFFFFFFu, lane > 0 ? n : 0u);
+            if (lane == kLong) n = longs;
+            if (lane < kCounts) lcnt[lane] = n ? atomicAdd(q.scount + (size_t)b * kCounts + lane, n) : 0u;
+        }
+        __syncthreads();
+        uint4* seg = q.seg + (size_t)b * q.sl.cap;
+        for (uint32_t i = threadIdx.x; i < nc; i += kPartThreads) {
+            const uint32_t f = found[i];
+            if (!f) continue;
+            const uint32_t hv = (uint32_t)(a[i] >> 32), len = (f >> 8) & 0xFFu, z = f & 0xFFu;
+            const int cls = seg_class(len);
+            // pair count: K + 1 for a source entry, 1 otherwise
+            const uint4 d = make_uint4(pbase + start[(hv << log_parts) >> (32 - kLogSub)] + ((f >> 16) & 0xFFu), len,
+                                       unhrow(hv), len + z * q.K);
+            seg[q.sl.off[cls] + atomicAdd(lcnt + cls, 1u)] = d;
+            if (cls > 0) seg[q.sl.off[kLong] + atomicAdd(lcnt + kLong, 1u)] = d;
+        }
+        __syncthreads();
     }
     // large sub-buckets: one warp each
     for (uint32_t g = warp; g < nbig; g += kPartThreads / 32) {
@@ -1606,12 +1650,15 @@ __device__ __forceinline__ void group_segments(const GroupParams& q, const uint6
 }
 
 __global__ void __launch_bounds__(kPartThreads) k_group_parts(GroupParams q, int log_parts) {
-    extern __shared__ uint64_t gkeys[];  // kPartCap keys
-    __shared__ uint32_t once[1u << (kMapBits - 5)], twice[1u << (kMapBits - 5)];
-    __shared__ uint32_t cnt[kPartSub];        // keys per sub-bucket, then the next key's place
-    __shared__ uint32_t start[kPartSub + 1];  // sub-bucket starts
+    extern __shared__ uint64_t gkeys[];  // kPartCap keys, then the sub-buckets' counts and starts
+    __shared__ uint32_t maps[2u << (kMapBits - 5)];  // hit once, hit twice
+    uint32_t* const once = maps;
+    uint32_t* const twice = maps + (1u << (kMapBits - 5));
+    uint32_t* const cnt = reinterpret_cast<uint32_t*>(gkeys + kPartCap);  // keys per sub-bucket, then the next key's place
+    uint32_t* const start = cnt + kPartSub;                               // [kPartSub + 1] sub-bucket starts
+    __shared__ uint32_t lcnt[kCounts];        // segments per list, then the next one's place
     __shared__ uint32_t wtot[32];
-    __shared__ uint16_t big[kPartSub];
+    __shared__ uint16_t big[(kPartItems2 << kPartMaxLog) / kRankMax];
     __shared__ uint32_t nbig, pbase;
     constexpr int U = 8;  // record entries per thread loaded at once
     const uint32_t me = blockIdx.x, tid = threadIdx.x;
@@ -1621,8 +1668,9 @@ __global__ void __launch_bounds__(kPartThreads) k_group_parts(GroupParams q, int
     batch_range(q, b, &base, &n);
     const int32_t* rec = q.rec + base;
     const uint32_t s_base = (uint32_t)((int64_t)b * q.batch);
-    for (uint32_t i = tid; i < 1u << (kMapBits - 5); i += kPartThreads) once[i] = twice[i] = 0u;
-    cnt[tid] = 0;
+    for (uint32_t i = tid; i < 2u << (kMapBits - 5); i += kPartThreads) maps[i] = 0u;
+    for (uint32_t i = tid; i < kPartSub; i += kPartThreads) cnt[i] = 0u;
+    if (tid < kCounts) lcnt[tid] = 0u;
     if (tid == 0) nbig = 0;
     __syncthreads();
     // f(entry index, sample within the batch, slot, hrow) for each of the part's entries
@@ -1654,12 +1702,14 @@ __global__ void __launch_bounds__(kPartThreads) k_group_parts(GroupParams q, int
     __syncthreads();
     each([&](uint32_t i, uint32_t, uint32_t, uint32_t hv) {
         const uint32_t h = (hv << log_parts) >> (32 - kMapBits);
-        if (twice[h >> 5] >> (h & 31u) & 1u) atomicAdd(&cnt[(hv << log_parts) >> (32 - 10)], 1u);
+        if (twice[h >> 5] >> (h & 31u) & 1u) atomicAdd(&cnt[(hv << log_parts) >> (32 - kLogSub)], 1u);
         else q.slot_info[base + i] = kSingleBit;
     });
     __syncthreads();
-    // exclusive scan of the 1,024 counts
-    const uint32_t own = cnt[tid];
+    // exclusive scan of the counts, four a thread
+    uint4* const cnt4 = reinterpret_cast<uint4*>(cnt) + tid;
+    const uint4 c4 = *cnt4;
+    const uint32_t own = c4.x + c4.y + c4.z + c4.w;
     uint32_t incl = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1671,12 +1721,22 @@ __global__ void __launch_bounds__(kPartThreads) k_group_parts(GroupParams q, int
     uint32_t wsum = lane < warp ? wtot[lane] : 0u;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) wsum += __shfl_xor_sync(0xFFFFFFFFu, wsum, o);
-    start[tid] = cnt[tid] = wsum + incl - own;
+    uint4 st;
+    st.x = wsum + incl - own;
+    st.y = st.x + c4.x;
+    st.z = st.y + c4.y;
+    st.w = st.z + c4.z;
+    *cnt4 = st;
+    *(reinterpret_cast<uint4*>(start) + tid) = st;
     if (tid == kPartThreads - 1) {
         start[kPartSub] = wsum + incl;
         pbase = atomicAdd(q.pcount + b, wsum + incl);
     }
-    if (own > kRankMax) big[atomicAdd(&nbig, 1u)] = (uint16_t)tid;
+    // large sub-buckets (each has over kRankMax of the batch's items)
+    if (c4.x > kRankMax) big[atomicAdd(&nbig, 1u)] = (uint16_t)(4 * tid);
+    if (c4.y > kRankMax) big[atomicAdd(&nbig, 1u)] = (uint16_t)(4 * tid + 1);
+    if (c4.z > kRankMax) big[atomicAdd(&nbig, 1u)] = (uint16_t)(4 * tid + 2);
+    if (c4.w > kRankMax) big[atomicAdd(&nbig, 1u)] = (uint16_t)(4 * tid + 3);
     __syncthreads();
     const uint32_t nc = start[kPartSub];
     const bool fits = nc <= kPartCap;
@@ -1684,15 +1744,15 @@ __global__ void __launch_bounds__(kPartThreads) k_group_parts(GroupParams q, int
     each([&](uint32_t, uint32_t smp, uint32_t slot, uint32_t hv) {
         const uint32_t h = (hv << log_parts) >> (32 - kMapBits);
         if (twice[h >> 5] >> (h & 31u) & 1u) {
-            const uint32_t at = atomicAdd(&cnt[(hv << log_parts) >> (32 - 10)], 1u);
+            const uint32_t at = atomicAdd(&cnt[(hv << log_parts) >> (32 - kLogSub)], 1u);
             const uint64_t key = ((uint64_t)hv << 32) | ((s_base + smp) << kSlotBits | slot);
             if (fits) gkeys[at] = key;
             else far[at] = key;
         }
     });
     __syncthreads();
-    if (fits) group_segments(q, gkeys, gkeys, nc, start, log_parts, pbase, b, big, nbig);
-    else group_segments(q, far, far, nc, start, log_parts, pbase, b, big, nbig);
+    if (fits) group_segments(q, gkeys, gkeys, nc, start, log_parts, pbase, b, big, nbig, maps, lcnt);
+    else group_segments(q, far, far, nc, start, log_parts, pbase, b, big, nbig, maps, lcnt);
 }
 
 // ---------------------------------------------------------------------------
@@ -2042,7 +2102,7 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
         return cudaErrorInvalidValue;
     }
     const size_t sort_smem = (size_t)kSortBucketsPerCta * 2 * kWarpSortCap * sizeof(uint64_t);
-    const size_t group_smem = (size_t)kPartCap * sizeof(uint64_t);
+    const size_t group_smem = (size_t)kPartCap * sizeof(uint64_t) + sizeof(uint32_t) * (2 * (size_t)kPartSub + 4);
     if ((e = cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem)) !=
             cudaSuccess ||
         (e = cudaFuncSetAttribute(k_group_parts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)group_smem)) !=
