@@ -32,14 +32,10 @@ namespace {
 // of a lane and 16 .. 1 are shuffles.  (One CTA per block of values, in shared
 // memory with a barrier per stride, took 289 us for 31.4M values.)
 template <typename T>
-__global__ void __launch_bounds__(256) k_tree_sum(const T* __restrict__ x, int64_t n, double* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t blk = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t base = blk * kSumBlock;
-    if (base >= n) return;
+__device__ __forceinline__ double tree_sum(const T* __restrict__ x, int64_t n, int lane) {
     double v[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = base + 32 * k + lane < n ? (double)x[base + 32 * k + lane] : 0.0;
+    for (int k = 0; k < 32; ++k) v[k] = 32 * k + lane < n ? (double)x[32 * k + lane] : 0.0;
 #pragma unroll
     for (int s = 16; s >= 1; s >>= 1)
 #pragma unroll
@@ -49,7 +45,26 @@ __global__ void __launch_bounds__(256) k_tree_sum(const T* __restrict__ x, int64
         const double o = __shfl_down_sync(0xFFFFFFFFu, v[0], s);
         v[0] = __dadd_rn(v[0], o);  // lanes >= s hold no partial sum
     }
-    if (lane == 0) out[blk] = v[0];
+    return v[0];  // in lane 0
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_tree_sum(const T* __restrict__ x, int64_t n, double* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const int64_t blk = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (blk * kSumBlock >= n) return;
+    const double v = tree_sum(x + blk * kSumBlock, n - blk * kSumBlock, lane);
+    if (lane == 0) out[blk] = v;
+}
+
+// out[r] = the sum of row r's n <= 1024 values, a warp a row.
+__global__ void __launch_bounds__(256) k_tree_rows(const double* __restrict__ x, int64_t rows, int64_t n,
+                                                   double* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (r >= rows) return;
+    const double v = tree_sum(x + r * n, n, lane);
+    if (lane == 0) out[r] = v;
 }
 
 // Sum over the block's threads of v (any order: integers), in every thread.
@@ -467,6 +482,14 @@ cudaError_t fixed_sum_f64(const double* x, int64_t n, double* tmp, double* out, 
         in = dst;
         cur = nb;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t fixed_sums_f64(const double* x, int64_t rows, int64_t padded, double* tmp, double* out, cudaStream_t s) {
+    const int64_t nb = padded / kSumBlock;  // (at most kSumBlock)
+    if (padded % kSumBlock || nb > kSumBlock) return cudaErrorInvalidValue;
+    k_tree_sum<double><<<(unsigned)((rows * nb + 7) / 8), 256, 0, s>>>(x, rows * padded, tmp);
+    k_tree_rows<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(tmp, rows, nb, out);
     return cudaGetLastError();
 }
 

@@ -56,39 +56,6 @@ line_status check_status(line_ctx* c, const char* what, bool timeout_sticky) {
     return LINE_OK;
 }
 
-// *p holds at least `bytes` (a larger earlier allocation is kept).
-template <typename T>
-cudaError_t grow(T** p, size_t* cap, size_t bytes) {
-    if (*p && *cap >= bytes) return cudaSuccess;
-    if (*p) cudaFree(*p);
-    *p = nullptr;
-    *cap = 0;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
-    if (e == cudaSuccess) *cap = bytes;
-    return e;
-}
-
-// Scratch for one synchronous call: up to kKeptScratch bytes from the
-// context's buffer (grown, kept for later calls, freed by line_destroy: a
-// cudaMalloc and cudaFree per call cost 100-200 us), more from an allocation
-// of the call's own.
-constexpr size_t kKeptScratch = (size_t)256 << 20;
-struct Scratch {
-    void* p = nullptr;
-    bool own = false;
-    cudaError_t take(line_ctx* c, size_t bytes) {
-        own = bytes > kKeptScratch;
-        if (own) return cudaMalloc(&p, bytes);
-        cudaError_t e = grow(&c->scratch, &c->scratch_cap, bytes);
-        p = c->scratch;
-        return e;
-    }
-    ~Scratch() {
-        if (own && p) cudaFree(p);
-    }
-};
-inline size_t round256(size_t v) { return (v + 255) & ~(size_t)255; }
-
 // Whether p is memory of the context's device (its kernels write there).
 bool on_device(const line_ctx* c, const void* p) {
     cudaPointerAttributes attr;

@@ -145,6 +145,10 @@ struct DeviceScratch {
 constexpr int kSumBlock = 1024;
 cudaError_t fixed_sum_f64(const double* x, int64_t n, double* tmp, double* out, cudaStream_t s);
 size_t fixed_sum_tmp_bytes(int64_t n);
+// The sums of `rows` rows of `padded` values each (a multiple of kSumBlock,
+// zero beyond a row's own): out[r] as fixed_sum_f64 of row r.  tmp:
+// rows * padded / kSumBlock doubles.
+cudaError_t fixed_sums_f64(const double* x, int64_t rows, int64_t padded, double* tmp, double* out, cudaStream_t s);
 // What one pass over the arcs finds besides errors (status) and the row offsets.
 struct GraphScan {
     unsigned long long sum;  // of the weights, where all are integers in [1, 2^24]

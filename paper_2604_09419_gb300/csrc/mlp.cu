@@ -30,6 +30,7 @@
 #include "context.cuh"
 #include "mlp_fwd.cuh"
 #include "mlp_math.cuh"
+#include "pdl.cuh"
 
 namespace line {
 
@@ -52,7 +53,6 @@ struct MlpState {
     int64_t cap = 0;
     int32_t* rows = nullptr;
     void* Xb = nullptr;      // [cap][P]
-    float* Tb = nullptr;     // [cap][dim]
     float* A1 = nullptr;     // [cap][hidden] pre-activations
     void* Hb = nullptr;      // [cap][hidden] activations
     float* Yb = nullptr;     // [cap][dim] outputs, then dL/dy
@@ -62,10 +62,11 @@ struct MlpState {
     __nv_bfloat16* gY = nullptr;
     __nv_bfloat16* gA = nullptr;
     void* arena = nullptr;  // the allocation holding every batch buffer above
-    float* part = nullptr;   // split partials
-    size_t part_elems = 0;
-    double* rowloss = nullptr;  // [cap]
-    void* sum_tmp = nullptr;
+    float* part = nullptr;   // partial sums over batch slices of gW2, gW1, gb1, gb2 (Parts)
+    // each row's loss, kLossRows steps of a batch padded to kSumBlock, and
+    // the block sums
+    double* rowloss = nullptr;
+    size_t rowloss_cap = 0;
     double* losses = nullptr;   // [loss_cap] per-step losses
     int64_t loss_cap = 0;
     int32_t* nodes = nullptr;   // training node list (device copy)
@@ -92,7 +93,7 @@ void mlp_destroy(MlpState* s) {
     if (!s) return;
     // params, grads, m and v share one allocation (params first); the
     // batch buffers share s->arena
-    for (void* p : {(void*)s->params, s->X, s->arena, (void*)s->losses, (void*)s->nodes, (void*)s->kmask,
+    for (void* p : {(void*)s->params, s->X, s->arena, (void*)s->rowloss, (void*)s->losses, (void*)s->nodes, (void*)s->kmask,
                     (void*)s->hubs, (void*)s->frows, (void*)s->flag, (void*)s->wt, (void*)s->w16})
         if (p) cudaFree(p);
     delete s;
@@ -498,33 +499,42 @@ cudaError_t features_for(int D, const FeatParams& p, int64_t count, int64_t max_
     }
 }
 
-// ---- minibatch: rows[j] = nodes[mulhi64(w1:w0, n)], draw s*B + j ------------
-__global__ void k_mlp_batch(const int32_t* __restrict__ nodes, int64_t n, uint64_t seed, uint64_t t0, int64_t B,
-                            int32_t* __restrict__ rows) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < B; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint4 w = draw_words(seed, kMlpDomain, t0 + (uint64_t)j, 0u);
-        const uint64_t r = ((uint64_t)w.y << 32) | (uint64_t)w.x;
-        rows[j] = nodes[__umul64hi(r, (uint64_t)n)];
-    }
-}
-
-// Xb[j] = X[rows[j]]; Tb[j] = U[rows[j]] (FP32) when Tb is given.
+// ---- minibatch ---------------------------------------------------------------
+// Xb[j] = X[r_j], r_j = rows[j], or with `nodes` the node nodes[mulhi64(w1:w0,
+// n)] of draw t0 + j, then also kept in rows.  A warp per row, 16 bytes a lane.
+// In the step's chain of programmatic launches the first row is drawn and
+// loaded before the wait (nothing in the chain writes the inputs), and stored
+// after it (the step before may still read Xb and rows).
 template <typename TX>
-__global__ void k_mlp_gather(const int32_t* __restrict__ rows, int64_t B, int64_t n_nodes,
-                             const TX* __restrict__ X, int P, TX* __restrict__ Xb, const void* U, int udt, int D,
-                             float* __restrict__ Tb, uint32_t* status) {
+__global__ void __launch_bounds__(256) k_mlp_gather(const int32_t* __restrict__ nodes, int64_t n, uint64_t seed, uint64_t t0,
+                                                    int32_t* __restrict__ rows, int64_t B, int64_t n_nodes,
+                                                    const TX* __restrict__ X, int P, TX* __restrict__ Xb, uint32_t* status) {
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
+    const int pieces = P * (int)sizeof(TX) / 16;  // (P is a multiple of 16)
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    bool waited = false;
     for (int64_t j = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); j < B; j += warps) {
-        int64_t r = rows[j];
-        if (r < 0 || r >= n_nodes) {
-            if (lane == 0) atomicOr(status, DEV_ERR_INDEX);
-            r = 0;
+        int64_t r;
+        if (nodes) {
+            const uint4 w = draw_words(seed, kMlpDomain, t0 + (uint64_t)j, 0u);
+            r = nodes[__umul64hi(((uint64_t)w.y << 32) | (uint64_t)w.x, (uint64_t)n)];
+        } else {
+            r = rows[j];
         }
-        for (int k = lane; k < P; k += 32) Xb[j * P + k] = X[r * P + k];
-        if (Tb)
-            for (int k = lane; k < D; k += 32) Tb[j * D + k] = load_row_elem(U, udt, r * D + k);
+        const bool out = r < 0 || r >= n_nodes;
+        if (out) r = 0;
+        const uint4* from = reinterpret_cast<const uint4*>(X + r * P);
+        uint4* to = reinterpret_cast<uint4*>(Xb + j * P);
+        const uint4 piece = lane < pieces ? __ldg(from + lane) : make_uint4(0u, 0u, 0u, 0u);
+        if (!waited) pdl_wait();
+        waited = true;
+        if (out && lane == 0) atomicOr(status, DEV_ERR_INDEX);
+        if (nodes && lane == 0) rows[j] = (int32_t)r;
+        if (lane < pieces) to[lane] = piece;
+        for (int k = lane + 32; k < pieces; k += 32) to[k] = __ldg(from + k);
     }
+    if (!waited) pdl_wait();
 }
 
 // ---- the contraction -------------------------------------------------------
@@ -973,21 +983,53 @@ __device__ __forceinline__ void store_hilo(__nv_bfloat16* hl, int64_t half, int6
     hl[half + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-// Training: y = Y + b2, r = y - t, dY = 2 r / (B D), rowloss[m] = sum r^2
-// (FP32 per lane in column order, then over the lanes in butterfly order;
-// the rows' sum is FP64).  One warp per row.  hl (nullable): dY's BF16
-// hi/lo pair as well.
-__global__ void k_ep_loss(float* __restrict__ Y, const float* __restrict__ b2, const float* __restrict__ Tb, int64_t M,
-                          int D, float scale, double* __restrict__ rowloss, __nv_bfloat16* __restrict__ hl) {
+// 4 values of a table row.
+__device__ __forceinline__ float4 load_row4(const void* U, int dtype, int64_t idx) {
+    if (dtype == LINE_DTYPE_F32) return __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(U) + idx));
+    const uint2 a = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(U) + idx));
+    return make_float4(__uint_as_float(a.x << 16), __uint_as_float(a.x & 0xFFFF0000u), __uint_as_float(a.y << 16),
+                       __uint_as_float(a.y & 0xFFFF0000u));
+}
+
+// Training: y = Y + b2, r = y - U[rows[m]], dY = 2 r / (B D), rowloss[m] = sum
+// r^2 (FP32 per lane in column order, then over the lanes in butterfly order;
+// the rows' sum is FP64).  One warp per row, 4 columns a lane.  hl (nullable):
+// dY's BF16 hi/lo pair as well.  A row id out of range counts as row 0 (the
+// gather reports it).
+__global__ void __launch_bounds__(256) k_ep_loss(float* __restrict__ Y, const float* __restrict__ b2, const void* U, int udt,
+                                                 const int32_t* __restrict__ rows, int64_t n_nodes, int64_t M, int D,
+                                                 float scale, double* __restrict__ rowloss, __nv_bfloat16* __restrict__ hl) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t m = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); m < M; m += warps) {
+        int64_t row = rows[m];
+        if (row < 0 || row >= n_nodes) row = 0;
         float acc = 0.0f;
-        for (int n = lane; n < D; n += 32) {
-            const float r = (Y[m * D + n] + b2[n]) - Tb[m * D + n];
-            acc = fmaf(r, r, acc);
-            Y[m * D + n] = scale * r;
-            if (hl) store_hilo(hl, M * D, m * D + n, scale * r);
+        for (int n = 4 * lane; n < D; n += 128) {
+            float4* yp = reinterpret_cast<float4*>(Y + m * D + n);
+            const float4 y = *yp, t = load_row4(U, udt, row * D + n);
+            const float r[4] = {(y.x + b2[n]) - t.x, (y.y + b2[n + 1]) - t.y, (y.z + b2[n + 2]) - t.z, (y.w + b2[n + 3]) - t.w};
+            float v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                acc = fmaf(r[k], r[k], acc);
+                v[k] = scale * r[k];
+            }
+            *yp = make_float4(v[0], v[1], v[2], v[3]);
+            if (hl) {
+                uint32_t hi[2], lo[2];
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+                    const __nv_bfloat162 l = __floats2bfloat162_rn(v[2 * k] - __low2float(h), v[2 * k + 1] - __high2float(h));
+                    hi[k] = *reinterpret_cast<const uint32_t*>(&h);
+                    lo[k] = *reinterpret_cast<const uint32_t*>(&l);
+                }
+                *reinterpret_cast<uint2*>(hl + m * D + n) = make_uint2(hi[0], hi[1]);
+                *reinterpret_cast<uint2*>(hl + M * D + m * D + n) = make_uint2(lo[0], lo[1]);
+            }
         }
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
@@ -1020,24 +1062,21 @@ __global__ void k_ep_dact(float* __restrict__ dH, const float* __restrict__ A1, 
     }
 }
 
-// out[i] = sum_z part[z][i], z ascending.
-__global__ void k_sum_slices(const float* __restrict__ part, int S, int64_t count, float* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        float s = 0.0f;
-#pragma unroll 8
-        for (int z = 0; z < S; ++z) s += part[(size_t)z * count + i];
-        out[i] = s;
-    }
-}
-
-// part[z][n] = sum of X[m][n] over the rows m of slice z: the slice's rows
-// split into kColGroups consecutive groups, each summed in row order by one
-// thread of a 32-column block, then the groups added in group order.
+// Bias gradients: part[z][n] = sum of X[m][n] over the rows m of slice z, the
+// slice's rows split into kColGroups consecutive groups, each summed in row
+// order by one thread of a 32-column block, then the groups added in group
+// order.  Blocks [0, nh) take dL/da (H columns), the others dL/dy (D columns).
 constexpr int kColGroups = 8;
-__global__ void __launch_bounds__(32 * kColGroups) k_colsum_slices(const float* __restrict__ X, int64_t M, int N,
-                                                                   int64_t rows_per, float* __restrict__ part) {
+__global__ void __launch_bounds__(32 * kColGroups) k_colsum_slices(const float* __restrict__ dA, int H, float* __restrict__ pb1,
+                                                                   const float* __restrict__ dY, int D,
+                                                                   float* __restrict__ pb2, int nh, int64_t M,
+                                                                   int64_t rows_per) {
+    pdl_launch_dependents();
+    pdl_wait();
     __shared__ float acc[kColGroups][32];
-    const int n = blockIdx.x * 32 + threadIdx.x;
+    const bool hidden = (int)blockIdx.x < nh;
+    const float* X = hidden ? dA : dY;
+    const int N = hidden ? H : D, n = ((int)blockIdx.x - (hidden ? 0 : nh)) * 32 + threadIdx.x;
     const int64_t m0 = (int64_t)blockIdx.y * rows_per, m1 = min(M, m0 + rows_per);
     const int64_t per = (rows_per + kColGroups - 1) / kColGroups;
     const int64_t a = m0 + threadIdx.y * per, b = min(m1, a + per);
@@ -1052,19 +1091,59 @@ __global__ void __launch_bounds__(32 * kColGroups) k_colsum_slices(const float* 
         float t = 0.0f;
 #pragma unroll
         for (int y = 0; y < kColGroups; ++y) t += acc[y][threadIdx.x];
-        part[(size_t)blockIdx.y * N + n] = t;
+        (hidden ? pb1 : pb2)[(size_t)blockIdx.y * N + n] = t;
     }
 }
 
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, int64_t n, float lr, float c1, float c2) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = 0.9f * m[i] + 0.1f * gi;
-        const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + 1e-8f);
+// The end of a step in one kernel: every parameter's gradient, its slices
+// summed in order, then (Adam) the parameter's update and its place in the
+// tensor-core tiles of the next forward pass.  As a kernel each - four sums,
+// Adam, three tilings - they took 26 us a step and eight launches, this
+// 5 us and one (18 MB of partial sums from L2).
+struct UpdateArgs {
+    const float *w2, *w1, *b1, *b2;  // partial sums
+    int SW, SB;                      // their slices: weights, biases
+    int H, P, D;
+    float *p, *g, *m, *v;  // g null: Adam, else the gradients only
+    float lr, c1, c2;
+    __nv_bfloat16* w16;    // nullable: tiles of W1, W2, W2^T
+};
+
+__global__ void __launch_bounds__(256) k_mlp_update(UpdateArgs a) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int64_t n1 = (int64_t)a.H * a.P, n2 = (int64_t)a.D * a.H, total = n1 + a.H + n2 + a.D;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const float* part;
+        int64_t count;
+        int S = a.SW;
+        if (i < n1) part = a.w1 + i, count = n1;
+        else if (i < n1 + a.H) part = a.b1 + (i - n1), count = a.H, S = a.SB;
+        else if (i < n1 + a.H + n2) part = a.w2 + (i - n1 - a.H), count = n2;
+        else part = a.b2 + (i - n1 - a.H - n2), count = a.D, S = a.SB;
+        float gi = 0.0f;
+#pragma unroll 16
+        for (int z = 0; z < S; ++z) gi += part[(size_t)z * count];
+        if (a.g) {
+            a.g[i] = gi;
+            continue;
+        }
+        const float mi = 0.9f * a.m[i] + 0.1f * gi;
+        const float vi = 0.999f * a.v[i] + 0.001f * gi * gi;
+        a.m[i] = mi;
+        a.v[i] = vi;
+        const float p = a.p[i] - a.lr * (mi * a.c1) / (sqrtf(vi * a.c2) + 1e-8f);
+        a.p[i] = p;
+        if (!a.w16) continue;
+        if (i < n1) {
+            put_tile(a.w16, a.H, a.P, (int)(i / a.P), (int)(i % a.P), p);
+        } else if (i >= n1 + a.H && i < n1 + a.H + n2) {
+            const int64_t q = i - n1 - a.H;
+            const int d = (int)(q / a.H), h = (int)(q % a.H);
+            __nv_bfloat16* w2 = a.w16 + 2 * n1;
+            put_tile(w2, a.D, a.H, d, h, p);
+            put_tile(w2 + 2 * n2, a.H, a.D, h, d, p);
+        }
     }
 }
 
@@ -1082,6 +1161,19 @@ struct Layout {
         W2 = b1 + s.hidden;
         b2 = W2 + (int64_t)s.dim * s.hidden;
         n = b2 + s.dim;
+    }
+};
+
+// The partial sums of a step's gradients, in s.part.
+struct Parts {
+    static constexpr int kSlices = 64, kBiasSlices = 32;
+    int64_t w2 = 0, w1, b1, b2, n;
+    explicit Parts(const MlpState& s) {
+        static_assert(kSlices >= kWgradMaxSlices, "slices of the weight gradients");
+        w1 = w2 + kSlices * (int64_t)s.dim * s.hidden;
+        b1 = w1 + kSlices * (int64_t)s.hidden * s.P;
+        b2 = b1 + kBiasSlices * (int64_t)s.hidden;
+        n = b2 + kBiasSlices * (int64_t)s.dim;
     }
 };
 
@@ -1122,26 +1214,20 @@ cudaError_t ensure_cap(MlpState& s, int64_t rows) {
     if (s.arena) cudaFree(s.arena);
     s.arena = nullptr;
     s.rows = nullptr;
-    s.Xb = s.Hb = s.sum_tmp = nullptr;
-    s.Tb = s.A1 = s.Yb = s.dH = s.part = nullptr;
-    s.rowloss = nullptr;
+    s.Xb = s.Hb = nullptr;
+    s.A1 = s.Yb = s.dH = s.part = nullptr;
     s.gY = s.gA = nullptr;
     s.cap = 0;
     const size_t act = s.act == LINE_DTYPE_F32 ? 4 : 2;
-    const int S = std::max(32, kWgradMaxSlices);
-    s.part_elems = (size_t)S * std::max<int64_t>((int64_t)s.hidden * s.P, (int64_t)s.dim * s.hidden);
     // every batch buffer in one allocation, each at a 256-byte boundary
     const bool hilo = s.act == LINE_DTYPE_BF16;
     const size_t sizes[] = {sizeof(int32_t) * cap,
                             act * cap * s.P,
-                            sizeof(float) * cap * s.dim,
                             sizeof(float) * cap * s.hidden,
                             act * cap * s.hidden,
                             sizeof(float) * cap * s.dim,
                             sizeof(float) * cap * s.hidden,
-                            sizeof(float) * s.part_elems,
-                            sizeof(double) * cap,
-                            fixed_sum_tmp_bytes(cap),
+                            sizeof(float) * Parts(s).n,
                             hilo ? sizeof(__nv_bfloat16) * 2 * cap * s.dim : 0,
                             hilo ? sizeof(__nv_bfloat16) * 2 * cap * s.hidden : 0};
     constexpr int kBufs = sizeof(sizes) / sizeof(sizes[0]);
@@ -1157,23 +1243,43 @@ cudaError_t ensure_cap(MlpState& s, int64_t rows) {
     s.arena = arena;
     s.rows = reinterpret_cast<int32_t*>(b + off[0]);
     s.Xb = b + off[1];
-    s.Tb = reinterpret_cast<float*>(b + off[2]);
-    s.A1 = reinterpret_cast<float*>(b + off[3]);
-    s.Hb = b + off[4];
-    s.Yb = reinterpret_cast<float*>(b + off[5]);
-    s.dH = reinterpret_cast<float*>(b + off[6]);
-    s.part = reinterpret_cast<float*>(b + off[7]);
-    s.rowloss = reinterpret_cast<double*>(b + off[8]);
-    s.sum_tmp = b + off[9];
-    s.gY = hilo ? reinterpret_cast<__nv_bfloat16*>(b + off[10]) : nullptr;
-    s.gA = hilo ? reinterpret_cast<__nv_bfloat16*>(b + off[11]) : nullptr;
+    s.A1 = reinterpret_cast<float*>(b + off[2]);
+    s.Hb = b + off[3];
+    s.Yb = reinterpret_cast<float*>(b + off[4]);
+    s.dH = reinterpret_cast<float*>(b + off[5]);
+    s.part = reinterpret_cast<float*>(b + off[6]);
+    s.gY = hilo ? reinterpret_cast<__nv_bfloat16*>(b + off[7]) : nullptr;
+    s.gA = hilo ? reinterpret_cast<__nv_bfloat16*>(b + off[8]) : nullptr;
     s.cap = cap;
     return cudaSuccess;
 }
 
-// Forward pass of rows s.rows[0..B): Xb, A1, Hb, Yb (= W2 h, before b2).
+// The rows of a pass: given (rows), or drawn from a node list (then kept in rows).
+struct Batch {
+    int32_t* rows;
+    const int32_t* nodes = nullptr;
+    int64_t n = 0;
+    uint64_t seed = 0, t0 = 0;
+};
+
+// The tensor-core tiles of the weights as they are (BF16 activations, shapes
+// that mlp_fwd.cu takes); Adam's steps keep them up to date.
+cudaError_t tile_weights(MlpState& s, cudaStream_t st) {
+    if (!fwd_fast(s)) return cudaSuccess;
+    const Layout L(s);
+    cudaError_t e = ensure_w16(s);
+    __nv_bfloat16* w2 = s.w16 + fwd_w16_elems(s.hidden, s.P);
+    if (e == cudaSuccess) e = fwd_tile_weights(s.params + L.W1, s.hidden, s.P, s.w16, st);
+    if (e == cudaSuccess) e = fwd_tile_weights(s.params + L.W2, s.dim, s.hidden, w2, st);
+    if (e == cudaSuccess)
+        e = fwd_tile_weights_t(s.params + L.W2, s.hidden, s.dim, w2 + fwd_w16_elems(s.dim, s.hidden), st);
+    return e;
+}
+
+// Forward pass of the B rows of `in`: Xb, Hb, Yb (= W2 h, before b2), and A1
+// for training.  The tiles of the weights are made by the caller.
 template <typename TX>
-cudaError_t forward(MlpState& s, int64_t B, const Tables& t, bool targets, uint32_t* status, int64_t n_nodes,
+cudaError_t forward(MlpState& s, int64_t B, const Batch& in, bool training, uint32_t* status, int64_t n_nodes,
                     cudaStream_t st) {
     const Layout L(s);
     const float* W1 = s.params + L.W1;
@@ -1181,22 +1287,19 @@ cudaError_t forward(MlpState& s, int64_t B, const Tables& t, bool targets, uint3
     const float* W2 = s.params + L.W2;
     TX* Xb = reinterpret_cast<TX*>(s.Xb);
     TX* Hb = reinterpret_cast<TX*>(s.Hb);
-    k_mlp_gather<TX><<<grid_of(B * 32, 256), 256, 0, st>>>(s.rows, B, n_nodes, reinterpret_cast<const TX*>(s.X), s.P,
-                                                            Xb, t.U, t.dtype, s.dim, targets ? s.Tb : nullptr, status);
-    cudaError_t e;
+    cudaError_t e = launch_pdl(k_mlp_gather<TX>, dim3(grid_of(B * 32, 256)), dim3(256), 0, st, true, in.nodes, in.n, in.seed,
+                               in.t0, in.rows, B, n_nodes, reinterpret_cast<const TX*>(s.X), s.P, Xb, status);
+    if (e != cudaSuccess) return e;
     if constexpr (std::is_same<TX, __nv_bfloat16>::value) {
         if (fwd_fast(s)) {
             // H = GELU(X W1^T + b1) (and A1 = X W1^T + b1 when training),
             // then Y = H W2^T, both on the tensor cores with the weights as
             // BF16 hi/lo pairs
-            if ((e = ensure_w16(s)) != cudaSuccess) return e;
-            const size_t e1 = fwd_w16_elems(s.hidden, s.P);
-            if ((e = fwd_tile_weights(W1, s.hidden, s.P, s.w16, st)) != cudaSuccess) return e;
-            if ((e = fwd_tile_weights(W2, s.dim, s.hidden, s.w16 + e1, st)) != cudaSuccess) return e;
-            if ((e = fwd_tc((int)B, s.hidden, s.P, Xb, s.w16, b1, targets ? s.A1 : nullptr, Hb, nullptr, status,
+            if ((e = fwd_tc((int)B, s.hidden, s.P, Xb, s.w16, b1, training ? s.A1 : nullptr, Hb, nullptr, status,
                             st)) != cudaSuccess)
                 return e;
-            return fwd_tc((int)B, s.dim, s.hidden, Hb, s.w16 + e1, nullptr, nullptr, nullptr, s.Yb, status, st);
+            return fwd_tc((int)B, s.dim, s.hidden, Hb, s.w16 + fwd_w16_elems(s.hidden, s.P), nullptr, nullptr, nullptr,
+                          s.Yb, status, st);
         }
     }
     const bool tc = s.act == LINE_DTYPE_BF16;
@@ -1232,14 +1335,15 @@ cudaError_t forward(MlpState& s, int64_t B, const Tables& t, bool targets, uint3
                                        W2t);
 }
 
-// Loss and gradients of the batch s.rows[0..B) into s.grads; the batch loss
-// (fixed-order FP64 sum / (B D)) into *loss_dev.
+// Loss rows (rowloss[0..B)) and the partial sums of the gradients of a batch
+// (s.part); *SW, *SB: their slices.
 template <typename TX>
-cudaError_t loss_grad(MlpState& s, int64_t B, const Tables& t, uint32_t* status, int64_t n_nodes, double* loss_dev,
-                      cudaStream_t st) {
+cudaError_t loss_grad(MlpState& s, int64_t B, const Batch& in, const Tables& t, uint32_t* status, int64_t n_nodes,
+                      double* rowloss, int* SW, int* SB, cudaStream_t st) {
     const Layout L(s);
+    const Parts parts(s);
     cudaError_t e;
-    if ((e = forward<TX>(s, B, t, true, status, n_nodes, st)) != cudaSuccess) return e;
+    if ((e = forward<TX>(s, B, in, true, status, n_nodes, st)) != cudaSuccess) return e;
     const float* W2 = s.params + L.W2;
     const float* b2 = s.params + L.b2;
     const float scale = (float)(2.0 / ((double)B * s.dim));
@@ -1248,13 +1352,14 @@ cudaError_t loss_grad(MlpState& s, int64_t B, const Tables& t, uint32_t* status,
     const bool tc = s.act == LINE_DTYPE_BF16;
     const bool wtc = tc && s.gY && s.gA && wgrad_tc_supported(s.dim, s.hidden) && wgrad_tc_supported(s.hidden, s.P) &&
                      B <= INT32_MAX;
-    k_ep_loss<<<grid_of(B * 32, 256), 256, 0, st>>>(s.Yb, b2, s.Tb, B, s.dim, scale, s.rowloss, wtc ? s.gY : nullptr);
+    if ((e = launch_pdl(k_ep_loss, dim3(grid_of(B * 32, 256)), dim3(256), 0, st, true, s.Yb, b2, (const void*)t.U, t.dtype,
+                        (const int32_t*)in.rows, n_nodes, B, s.dim, scale, rowloss, wtc ? s.gY : nullptr)) != cudaSuccess)
+        return e;
     // dH = dY W2, then dA = dH GELU'(a): with the tensor-core weight
     // gradients, one pass on the forward kernel (dY as its hi/lo pair, W2^T as
     // hi/lo tiles) that writes dA and its hi/lo pair
     if (wtc && fwd_fast(s) && s.w16 && dact_tc_supported(s.hidden, s.dim)) {
-        __nv_bfloat16* w2t = s.w16 + fwd_w16_elems(s.hidden, s.P) + fwd_w16_elems(s.dim, s.hidden);
-        if ((e = fwd_tile_weights_t(W2, s.hidden, s.dim, w2t, st)) != cudaSuccess) return e;
+        const __nv_bfloat16* w2t = s.w16 + fwd_w16_elems(s.hidden, s.P) + fwd_w16_elems(s.dim, s.hidden);
         if ((e = dact_tc((int)B, s.hidden, s.dim, s.gY, s.gY + B * s.dim, w2t, s.A1, s.dH, s.gA, status, st)) !=
             cudaSuccess)
             return e;
@@ -1274,44 +1379,84 @@ cudaError_t loss_grad(MlpState& s, int64_t B, const Tables& t, uint32_t* status,
     }
     const TX* Xb = reinterpret_cast<const TX*>(s.Xb);
     const TX* Hb = reinterpret_cast<const TX*>(s.Hb);
+    float* pw2 = s.part + parts.w2;
+    float* pw1 = s.part + parts.w1;
     const int S = slices_for(B);
+    *SW = *SB = S;
+    // gW2 = dY^T H and gW1 = dA^T X, split over the batch
     if constexpr (std::is_same<TX, __nv_bfloat16>::value) {
         if (wtc) {
-            // gW2 = dY^T H and gW1 = dA^T X, split over the batch, the slices
-            // summed in order
-            const int SW = wgrad_slices((int)B);
-            const int64_t nW2 = (int64_t)s.dim * s.hidden, nW1 = (int64_t)s.hidden * s.P;
-            if ((e = wgrad_tc(s.dim, s.hidden, (int)B, s.gY, s.gY + B * s.dim, Hb, s.part, status, st)) != cudaSuccess)
+            *SW = wgrad_slices((int)B);
+            if ((e = wgrad_tc(s.dim, s.hidden, (int)B, s.gY, s.gY + B * s.dim, Hb, pw2, status, st)) != cudaSuccess ||
+                (e = wgrad_tc(s.hidden, s.P, (int)B, s.gA, s.gA + B * s.hidden, Xb, pw1, status, st)) != cudaSuccess)
                 return e;
-            k_sum_slices<<<grid_of(nW2, 256), 256, 0, st>>>(s.part, SW, nW2, s.grads + L.W2);
-            if ((e = wgrad_tc(s.hidden, s.P, (int)B, s.gA, s.gA + B * s.hidden, Xb, s.part, status, st)) !=
-                cudaSuccess)
-                return e;
-            k_sum_slices<<<grid_of(nW1, 256), 256, 0, st>>>(s.part, SW, nW1, s.grads + L.W1);
         }
     }
     if (!wtc) {
-        // gW2 = dY^T H
-        if ((e = gemm<float, TX, false, false>(tc, s.dim, s.hidden, (int)B, S, s.Yb, s.dim, Hb, s.hidden, s.part,
-                                               status, st)) != cudaSuccess)
+        if ((e = gemm<float, TX, false, false>(tc, s.dim, s.hidden, (int)B, S, s.Yb, s.dim, Hb, s.hidden, pw2, status, st)) !=
+                cudaSuccess ||
+            (e = gemm<float, TX, false, false>(tc, s.hidden, s.P, (int)B, S, s.dH, s.hidden, Xb, s.P, pw1, status, st)) !=
+                cudaSuccess)
             return e;
-        k_sum_slices<<<grid_of((int64_t)s.dim * s.hidden, 256), 256, 0, st>>>(s.part, S, (int64_t)s.dim * s.hidden,
-                                                                              s.grads + L.W2);
-        // gW1 = dA^T X
-        if ((e = gemm<float, TX, false, false>(tc, s.hidden, s.P, (int)B, S, s.dH, s.hidden, Xb, s.P, s.part,
-                                               status, st)) != cudaSuccess)
-            return e;
-        k_sum_slices<<<grid_of((int64_t)s.hidden * s.P, 256), 256, 0, st>>>(s.part, S, (int64_t)s.hidden * s.P,
-                                                                           s.grads + L.W1);
     }
-    // bias gradients: column sums in slices of rows, slices summed in order
-    const int64_t rows_per = (B + S - 1) / S;
-    k_colsum_slices<<<dim3((s.hidden + 31) / 32, S), dim3(32, kColGroups), 0, st>>>(s.dH, B, s.hidden, rows_per, s.part);
-    k_sum_slices<<<grid_of(s.hidden, 256), 256, 0, st>>>(s.part, S, s.hidden, s.grads + L.b1);
-    k_colsum_slices<<<dim3((s.dim + 31) / 32, S), dim3(32, kColGroups), 0, st>>>(s.Yb, B, s.dim, rows_per, s.part);
-    k_sum_slices<<<grid_of(s.dim, 256), 256, 0, st>>>(s.part, S, s.dim, s.grads + L.b2);
-    if ((e = fixed_sum_f64(s.rowloss, B, reinterpret_cast<double*>(s.sum_tmp), loss_dev, st)) != cudaSuccess) return e;
-    return cudaGetLastError();
+    // bias gradients: column sums in slices of rows
+    const int nh = (s.hidden + 31) / 32;
+    return launch_pdl(k_colsum_slices, dim3(nh + (s.dim + 31) / 32, S), dim3(32, kColGroups), 0, st, true,
+                      (const float*)s.dH, s.hidden, s.part + parts.b1, (const float*)s.Yb, s.dim, s.part + parts.b2, nh, B,
+                      (B + S - 1) / S);
+}
+
+// The gradients from their partial sums: into s.grads, or (Adam, step count
+// s.t) into the parameters.
+cudaError_t update(MlpState& s, int SW, int SB, bool adam, float lr, cudaStream_t st) {
+    const Parts parts(s);
+    UpdateArgs a{};
+    a.w2 = s.part + parts.w2;
+    a.w1 = s.part + parts.w1;
+    a.b1 = s.part + parts.b1;
+    a.b2 = s.part + parts.b2;
+    a.SW = SW;
+    a.SB = SB;
+    a.H = s.hidden;
+    a.P = s.P;
+    a.D = s.dim;
+    a.p = s.params;
+    a.m = s.m;
+    a.v = s.v;
+    if (adam) {
+        a.lr = lr;
+        a.c1 = (float)(1.0 / (1.0 - pow(0.9, (double)s.t)));
+        a.c2 = (float)(1.0 / (1.0 - pow(0.999, (double)s.t)));
+        a.w16 = fwd_fast(s) ? s.w16 : nullptr;
+    } else {
+        a.g = s.grads;
+    }
+    return launch_pdl(k_mlp_update, dim3(grid_of(s.n_params, 256)), dim3(256), 0, st, true, a);
+}
+
+// Row losses of kLossRows steps are summed together.
+constexpr int64_t kLossRows = 64;
+int64_t padded_rows(int64_t B) { return (B + kSumBlock - 1) / kSumBlock * kSumBlock; }
+
+// Room for `rows` steps' row losses of batches of B, all zero, then their
+// block sums.
+cudaError_t ensure_rowloss(MlpState& s, int64_t rows, int64_t B, cudaStream_t st) {
+    const size_t n = (size_t)rows * padded_rows(B), need = sizeof(double) * (n + n / kSumBlock);
+    if (s.rowloss_cap < need) {
+        if (s.rowloss) cudaFree(s.rowloss);
+        s.rowloss = nullptr;
+        s.rowloss_cap = 0;
+        const cudaError_t e = cudaMalloc(&s.rowloss, need);
+        if (e != cudaSuccess) return e;
+        s.rowloss_cap = need;
+    }
+    return cudaMemsetAsync(s.rowloss, 0, sizeof(double) * n, st);
+}
+
+// losses[0 .. rows): each step's fixed-order FP64 sum of its row losses.
+cudaError_t sum_losses(MlpState& s, int64_t rows, int64_t B, double* losses, cudaStream_t st) {
+    const int64_t padded = padded_rows(B);
+    return fixed_sums_f64(s.rowloss, rows, padded, s.rowloss + rows * padded, losses, st);
 }
 
 __global__ void k_scale_loss(double* loss, double inv) { *loss *= inv; }
@@ -1558,9 +1703,16 @@ line_status line_mlp_grad(line_ctx* c, const int32_t* rows, int64_t n_rows, floa
     const Tables& t = c->tab[s.order];
     CK(ensure_cap(s, n_rows), "line_mlp_grad");
     CK(cudaMemcpyAsync(s.rows, rows, sizeof(int32_t) * n_rows, cudaMemcpyDefault, c->stream), "line_mlp_grad");
-    cudaError_t e = s.act == LINE_DTYPE_F32
-                        ? loss_grad<float>(s, n_rows, t, c->status, c->n_nodes, c->dscratch, c->stream)
-                        : loss_grad<__nv_bfloat16>(s, n_rows, t, c->status, c->n_nodes, c->dscratch, c->stream);
+    const Batch in{s.rows};
+    int SW = 0, SB = 0;
+    cudaError_t e = tile_weights(s, c->stream);
+    if (e == cudaSuccess) e = ensure_rowloss(s, 1, n_rows, c->stream);
+    if (e == cudaSuccess)
+        e = s.act == LINE_DTYPE_F32
+                ? loss_grad<float>(s, n_rows, in, t, c->status, c->n_nodes, s.rowloss, &SW, &SB, c->stream)
+                : loss_grad<__nv_bfloat16>(s, n_rows, in, t, c->status, c->n_nodes, s.rowloss, &SW, &SB, c->stream);
+    if (e == cudaSuccess) e = update(s, SW, SB, false, 0.0f, c->stream);
+    if (e == cudaSuccess) e = sum_losses(s, 1, n_rows, c->dscratch, c->stream);
     if (e == cudaSuccess) {
         k_scale_loss<<<1, 1, 0, c->stream>>>(c->dscratch, 1.0 / ((double)n_rows * s.dim));
         e = cudaGetLastError();
@@ -1598,19 +1750,23 @@ line_status line_mlp_train(line_ctx* c, const int32_t* nodes, int64_t n_nodes, i
         s.loss_cap = steps;
     }
     // node ids out of range are reported by the gather (status word)
-    for (int64_t k = 0; k < steps; ++k) {
-        const uint64_t gstep = step_offset + (uint64_t)k;
-        k_mlp_batch<<<grid_of(batch, 256), 256, 0, str>>>(s.nodes, n_nodes, seed, gstep * (uint64_t)batch, batch,
-                                                          s.rows);
-        cudaError_t e = s.act == LINE_DTYPE_F32
-                            ? loss_grad<float>(s, batch, t, c->status, c->n_nodes, s.losses + k, str)
-                            : loss_grad<__nv_bfloat16>(s, batch, t, c->status, c->n_nodes, s.losses + k, str);
-        if (e != cudaSuccess) return cuda_fail(c, e, "line_mlp_train");
-        ++s.t;
-        const float c1 = (float)(1.0 / (1.0 - pow(0.9, (double)s.t)));
-        const float c2 = (float)(1.0 / (1.0 - pow(0.999, (double)s.t)));
-        k_adam<<<grid_of(s.n_params, 256), 256, 0, str>>>(s.params, s.grads, s.m, s.v, s.n_params, (float)lr, c1, c2);
-        CK(cudaGetLastError(), "line_mlp_train");
+    CK(tile_weights(s, str), "line_mlp_train");
+    const int64_t padded = padded_rows(batch);
+    for (int64_t k0 = 0; k0 < steps; k0 += kLossRows) {
+        const int64_t rows = std::min(kLossRows, steps - k0);
+        CK(ensure_rowloss(s, rows, batch, str), "line_mlp_train");
+        for (int64_t k = k0; k < k0 + rows; ++k) {
+            const Batch in{s.rows, s.nodes, n_nodes, seed, (step_offset + (uint64_t)k) * (uint64_t)batch};
+            double* rl = s.rowloss + (k - k0) * padded;
+            int SW = 0, SB = 0;
+            cudaError_t e = s.act == LINE_DTYPE_F32
+                                ? loss_grad<float>(s, batch, in, t, c->status, c->n_nodes, rl, &SW, &SB, str)
+                                : loss_grad<__nv_bfloat16>(s, batch, in, t, c->status, c->n_nodes, rl, &SW, &SB, str);
+            ++s.t;
+            if (e == cudaSuccess) e = update(s, SW, SB, true, (float)lr, str);
+            if (e != cudaSuccess) return cuda_fail(c, e, "line_mlp_train");
+        }
+        CK(sum_losses(s, rows, batch, s.losses + k0, str), "line_mlp_train");
     }
     if (losses_out) {
         std::vector<double> tmp(steps);
@@ -1634,8 +1790,12 @@ line_status line_mlp_predict(line_ctx* c, const int32_t* rows, int64_t n_rows, f
     cudaStream_t str = c->stream;
     const int64_t chunk = std::min<int64_t>(n_rows, kMlpMaxBatch);
     CK(ensure_cap(s, chunk), "line_mlp_predict");
-    float* ybuf = nullptr;
-    if (y_out) CK(cudaMalloc(&ybuf, sizeof(float) * n_rows * s.dim), "line_mlp_predict");
+    // outputs in device memory are written there; others go through scratch
+    const size_t y_bytes = sizeof(float) * (size_t)n_rows * s.dim;
+    const bool direct = y_out && on_device(c, y_out) && !((uintptr_t)y_out & 3);
+    Scratch sc;
+    if (y_out && !direct) CK(sc.take(c, y_bytes), "line_mlp_predict");
+    float* ybuf = direct ? y_out : (float*)sc.p;
     const Layout L(s);
     cudaError_t e = cudaSuccess;
     // all requested ids in one copy; each chunk then takes its slice on the device
@@ -1646,25 +1806,24 @@ line_status line_mlp_predict(line_ctx* c, const int32_t* rows, int64_t n_rows, f
         if ((e = cudaMalloc(&s.frows, sizeof(int32_t) * (size_t)n_rows)) == cudaSuccess) s.frows_cap = n_rows;
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.frows, rows, sizeof(int32_t) * n_rows, cudaMemcpyDefault, str);
+    if (e == cudaSuccess) e = tile_weights(s, str);
     for (int64_t r0 = 0; r0 < n_rows && e == cudaSuccess; r0 += chunk) {
         const int64_t B = std::min(chunk, n_rows - r0);
-        e = cudaMemcpyAsync(s.rows, s.frows + r0, sizeof(int32_t) * B, cudaMemcpyDeviceToDevice, str);
-        if (e == cudaSuccess)
-            e = s.act == LINE_DTYPE_F32 ? forward<float>(s, B, t, false, c->status, c->n_nodes, str)
-                                        : forward<__nv_bfloat16>(s, B, t, false, c->status, c->n_nodes, str);
+        const Batch in{s.frows + r0};
+        e = s.act == LINE_DTYPE_F32 ? forward<float>(s, B, in, false, c->status, c->n_nodes, str)
+                                    : forward<__nv_bfloat16>(s, B, in, false, c->status, c->n_nodes, str);
         if (e == cudaSuccess) {
             if (ybuf)
                 k_ep_predict<<<grid_of(B * s.dim, 256), 256, 0, str>>>(s.Yb, s.params + L.b2, B, s.dim, nullptr, 0,
                                                                        ybuf + r0 * s.dim, LINE_DTYPE_F32);
             else
-                k_ep_predict<<<grid_of(B * s.dim, 256), 256, 0, str>>>(s.Yb, s.params + L.b2, B, s.dim, s.rows,
+                k_ep_predict<<<grid_of(B * s.dim, 256), 256, 0, str>>>(s.Yb, s.params + L.b2, B, s.dim, in.rows,
                                                                        c->n_nodes, t.U, t.dtype);
             e = cudaGetLastError();
         }
     }
-    if (e == cudaSuccess && ybuf) e = cudaMemcpyAsync(y_out, ybuf, sizeof(float) * n_rows * s.dim, cudaMemcpyDefault, str);
+    if (e == cudaSuccess && ybuf && !direct) e = cudaMemcpyAsync(y_out, ybuf, y_bytes, cudaMemcpyDefault, str);
     if (e == cudaSuccess) e = cudaStreamSynchronize(str);
-    if (ybuf) cudaFree(ybuf);
     if (e != cudaSuccess) return cuda_fail(c, e, "line_mlp_predict");
     return check_status(c, "line_mlp_predict");
 }

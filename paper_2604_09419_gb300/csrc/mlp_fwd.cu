@@ -34,6 +34,7 @@
 #include <mutex>
 
 #include "bulk.cuh"
+#include "pdl.cuh"
 #include "line_internal.cuh"
 #include "mlp_fwd.cuh"
 #include "mlp_math.cuh"
@@ -189,6 +190,25 @@ __device__ __forceinline__ void fwd_drain(uint64_t* bar, uint32_t parity) {
         if (mbar_try_wait(bar, parity)) return;
 }
 
+// 32 bytes of a lane at once (32-byte aligned): a lane holds a row of its own,
+// so a 16-byte access touches half a sector.
+__device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void st_global_v8(void* p, const float* v) {
+    uint32_t w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = __float_as_uint(v[k]);
+    st_global_v8(p, w);
+}
+__device__ __forceinline__ void ld_global_v8(const float* p, float* v) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -237,6 +257,10 @@ __global__ void __launch_bounds__(kFThreads, 1) k_mlp_fwd_tc(const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base;
+    // (after the tensor memory is allocated: the next kernel's blocks, which
+    // allocate too, start when all of these have)
+    pdl_launch_dependents();
+    pdl_wait();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -326,11 +350,11 @@ __global__ void __launch_bounds__(kFThreads, 1) k_mlp_fwd_tc(const __grid_consta
             // dL/da: the pre-activations of this warp's first 16 columns are
             // loaded before the products are waited for, and those of the
             // next 16 columns while the current ones are worked on
-            float4 a1_next[4];
+            float a1_next[16];
             if (mode == kModeDact && row < a.M) {
-                const float4* ap = reinterpret_cast<const float4*>(a.A1in + (size_t)row * N + h * quarter);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) a1_next[j] = __ldg(ap + j);
+                const float* ap = a.A1in + (size_t)row * N + h * quarter;
+                ld_global_v8(ap, a1_next);
+                ld_global_v8(ap + 8, a1_next + 8);
             }
             const bool ok = fwd_wait(&tfull[acc], u & 1u, abort_flag, a.status);
             if (!__all_sync(0xFFFFFFFFu, ok)) break;
@@ -342,48 +366,33 @@ __global__ void __launch_bounds__(kFThreads, 1) k_mlp_fwd_tc(const __grid_consta
                     // dA = C GELU'(A1), FP32 and its BF16 hi/lo pair, this row's 16 columns
                     if (row < a.M) {
                         const size_t o = (size_t)row * N + c0;
-                        float4 a1_cur[4];
+                        float a1[16];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) a1_cur[j] = a1_next[j];
+                        for (int j = 0; j < 16; ++j) a1[j] = a1_next[j];
                         if (c0 + kFChunk < c_end) {
-                            const float4* ap = reinterpret_cast<const float4*>(a.A1in + o + kFChunk);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) a1_next[j] = __ldg(ap + j);
+                            ld_global_v8(a.A1in + o + kFChunk, a1_next);
+                            ld_global_v8(a.A1in + o + kFChunk + 8, a1_next + 8);
                         }
                         float v[16];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const float4 a1 = a1_cur[j];
-                            const float2 g0 = __fmul2_rn(make_float2(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1])),
-                                                         gelu_grad_fast2(make_float2(a1.x, a1.y)));
-                            const float2 g1 = __fmul2_rn(make_float2(__uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3])),
-                                                         gelu_grad_fast2(make_float2(a1.z, a1.w)));
-                            v[4 * j] = g0.x;
-                            v[4 * j + 1] = g0.y;
-                            v[4 * j + 2] = g1.x;
-                            v[4 * j + 3] = g1.y;
-                        }
-                        float4* dp = reinterpret_cast<float4*>(a.dA + o);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) dp[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                        float hi[16], lo[16];
-#pragma unroll
                         for (int j = 0; j < 16; j += 2) {
-                            hi[j] = __bfloat162float(__float2bfloat16_rn(v[j]));
-                            hi[j + 1] = __bfloat162float(__float2bfloat16_rn(v[j + 1]));
-                            const float2 l = __fadd2_rn(make_float2(v[j], v[j + 1]), make_float2(-hi[j], -hi[j + 1]));
-                            lo[j] = l.x;
-                            lo[j + 1] = l.y;
+                            const float2 g = __fmul2_rn(make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])),
+                                                        gelu_grad_fast2(make_float2(a1[j], a1[j + 1])));
+                            v[j] = g.x;
+                            v[j + 1] = g.y;
                         }
-                        uint4* hp = reinterpret_cast<uint4*>(a.dA_hl + o);
-                        uint4* lp = reinterpret_cast<uint4*>(a.dA_hl + (size_t)a.M * N + o);
+                        st_global_v8(a.dA + o, v);
+                        st_global_v8(a.dA + o + 8, v + 8);
+                        uint32_t hi[8], lo[8];
 #pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            hp[j] = make_uint4(pack_bf16x2(hi[8 * j], hi[8 * j + 1]), pack_bf16x2(hi[8 * j + 2], hi[8 * j + 3]),
-                                               pack_bf16x2(hi[8 * j + 4], hi[8 * j + 5]), pack_bf16x2(hi[8 * j + 6], hi[8 * j + 7]));
-                            lp[j] = make_uint4(pack_bf16x2(lo[8 * j], lo[8 * j + 1]), pack_bf16x2(lo[8 * j + 2], lo[8 * j + 3]),
-                                               pack_bf16x2(lo[8 * j + 4], lo[8 * j + 5]), pack_bf16x2(lo[8 * j + 6], lo[8 * j + 7]));
+                        for (int j = 0; j < 8; ++j) {
+                            hi[j] = pack_bf16x2(v[2 * j], v[2 * j + 1]);
+                            const float2 l = __fadd2_rn(make_float2(v[2 * j], v[2 * j + 1]),
+                                                        make_float2(-__uint_as_float(hi[j] << 16), -__uint_as_float(hi[j] & 0xFFFF0000u)));
+                            lo[j] = pack_bf16x2(l.x, l.y);
                         }
+                        st_global_v8(a.dA_hl + o, hi);
+                        st_global_v8(a.dA_hl + (size_t)a.M * N + o, lo);
                     }
                     continue;
                 }
@@ -406,9 +415,8 @@ __global__ void __launch_bounds__(kFThreads, 1) k_mlp_fwd_tc(const __grid_consta
                         v[4 * j + 3] = s1.y;
                     }
                     if (a.A1 && row < a.M) {
-                        float4* p = reinterpret_cast<float4*>(a.A1 + (size_t)row * N + c0);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) p[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                        st_global_v8(a.A1 + (size_t)row * N + c0, v);
+                        st_global_v8(a.A1 + (size_t)row * N + c0 + 8, v + 8);
                     }
                     // row `lane` of the block: 2 pieces of 16 bytes, piece j at
                     // j ^ ((lane >> 2) & 1) (the map's 32-byte swizzle)
@@ -527,6 +535,8 @@ __global__ void __launch_bounds__(kWThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base;
+    pdl_launch_dependents();
+    pdl_wait();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -593,11 +603,11 @@ __global__ void __launch_bounds__(kWThreads, 1)
                 uint32_t r[16];
                 tc_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
                 if (row < a.M) {
-                    float4* p = reinterpret_cast<float4*>(out + c0);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        p[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                           __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+                    // (N a multiple of 16: 64-byte blocks)
+                    const uint32_t lo8[8] = {r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7]};
+                    const uint32_t hi8[8] = {r[8], r[9], r[10], r[11], r[12], r[13], r[14], r[15]};
+                    st_global_v8(out + c0, lo8);
+                    st_global_v8(out + c0 + 8, hi8);
                 }
             }
         } else if (nst == 0 && lane == 0) {
@@ -625,11 +635,7 @@ __global__ void k_tile_w16(const float* __restrict__ W, int N, int K, __nv_bfloa
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int n = (int)(i / K), k = (int)(i % K);
         const float w = TRANS ? W[(int64_t)k * N + n] : W[i];
-        const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(w - __bfloat162float(hi));  // w - hi is exact in FP32
-        const int64_t o = (int64_t)(n >> 3) * (K * 8) + (k >> 3) * 64 + (n & 7) * 8 + (k & 7);
-        Wt[o] = hi;
-        Wt[total + o] = lo;
+        put_tile(Wt, N, K, n, k, w);
     }
 }
 
@@ -735,8 +741,7 @@ cudaError_t launch_fwd(int mode, int M, int N, int K, const __nv_bfloat16* A, co
     a.dA_hl = dA_hl;
     a.status = status;
     const int grid = std::min(a.n_tiles, sms);
-    k_mlp_fwd_tc<<<grid, kFThreads, smem, s>>>(map, map2, omap, a);
-    return cudaGetLastError();
+    return launch_pdl(k_mlp_fwd_tc, dim3(grid), dim3(kFThreads), smem, s, true, map, map2, omap, a);
 }
 
 }  // namespace
@@ -829,8 +834,8 @@ cudaError_t wgrad_tc(int M, int N, int K, const __nv_bfloat16* A_hi, const __nv_
     w.nkb = nkb;
     w.part = part;
     w.status = status;
-    k_mlp_wgrad_tc<<<dim3((unsigned)wgrad_slices(K), (unsigned)(M / kFM)), kWThreads, smem, s>>>(mah, mal, mb, w);
-    return cudaGetLastError();
+    return launch_pdl(k_mlp_wgrad_tc, dim3((unsigned)wgrad_slices(K), (unsigned)(M / kFM)), dim3(kWThreads), smem, s, true,
+                      mah, mal, mb, w);
 }
 
 }  // namespace line

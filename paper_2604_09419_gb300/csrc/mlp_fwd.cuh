@@ -23,6 +23,15 @@ bool fwd_tc_supported(int N, int K);
 // BF16 elements of the hi/lo tiles of an N x K weight matrix (2 N K).
 inline size_t fwd_w16_elems(int N, int K) { return 2 * (size_t)N * K; }
 
+// Weight w at (n, k) of an N x K matrix into its hi and lo tiles.
+__device__ __forceinline__ void put_tile(__nv_bfloat16* Wt, int N, int K, int n, int k, float w) {
+    const __nv_bfloat16 hi = __float2bfloat16_rn(w);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(w - __bfloat162float(hi));  // w - hi is exact in FP32
+    const int64_t o = (int64_t)(n >> 3) * (K * 8) + (k >> 3) * 64 + (n & 7) * 8 + (k & 7);
+    Wt[o] = hi;
+    Wt[(int64_t)N * K + o] = lo;
+}
+
 // W (N x K, row-major FP32) into Wt: W_hi then W_lo, each in the tensor
 // core's K-major core-matrix layout (8 rows x 8 values of 16 bytes per core
 // matrix, core matrices along K 128 bytes apart, groups of 8 rows 16 K bytes

@@ -53,15 +53,11 @@
 
 #include "bulk.cuh"
 #include "line_internal.cuh"
+#include "pdl.cuh"
 #include "rows.cuh"
 #include "scan.cuh"
 
 namespace line {
-
-// Programmatic dependent launch: let the next kernel of the stream start its
-// prologue, and wait until the previous kernel's writes are visible.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // A shared segment's entries are summed in chunks of kChunk: partial sums in
 // entry order, then the partials in chunk order.  Segments are listed by the
@@ -1884,22 +1880,6 @@ static int staged_warps(int K, int requested, size_t* smem_out) {
     const int fit = std::max(1, std::min(wpb, (int)(kMaxSmem / per_warp)));
     *smem_out = (size_t)fit * per_warp;
     return fit;
-}
-
-template <typename... Args, typename... Vals>
-static cudaError_t launch_pdl(void (*kern)(Args...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                              bool pdl, Vals... vals) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, vals...);
 }
 
 template <int D, int DT>
