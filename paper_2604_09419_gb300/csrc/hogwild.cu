@@ -30,8 +30,10 @@
 // of the sample's batch.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
+#include "bulk.cuh"
 #include "line_internal.cuh"
 #include "rows.cuh"
 
@@ -91,8 +93,27 @@ __device__ __forceinline__ void add_row(void* table, int64_t row, int lig, const
     }
 }
 
-template <int D, int DT>
-__global__ void __launch_bounds__(kHogWarps * 32) k_hogwild(HogwildParams p) {
+// Four consecutive values of a row as they lie in memory, and as floats.
+template <int DT>
+using Packed = std::conditional_t<DT == LINE_DTYPE_F32, float4, uint2>;
+__device__ __forceinline__ float4 unpack(float4 v) { return v; }
+__device__ __forceinline__ float4 unpack(uint2 v) {
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
+                       __uint_as_float(v.y & 0xFFFF0000u));
+}
+
+// Bound by the rows' way through L2 and device memory; the loads of a sample
+// are its one long wait, so how many are in flight decides.  STAGED copies all
+// context rows of a sample into the stage by 16-byte asynchronous copies, past
+// the registers, and waits once; without it the rows pass through registers,
+// at most CH at a time (BF16 rows must: they are widened on the way).  A
+// sample's record is loaded while the sample before is computed.  4.2 million
+// samples, K = 5, device memory tables (R-MAT 20, D = 128 FP32): 5.84 -> 4.81
+// ms, floor 4.78; BF16 7.98 -> 7.51; D = 64, K = 10, FP32 4.94 -> 4.01.  Eight
+// resident blocks (64 registers) of the STAGED form: ten (48) are 3% slower.
+template <int D, int DT, bool STAGED>
+__global__ void __launch_bounds__(kHogWarps * 32, STAGED ? 8 : 0)
+    k_hogwild(HogwildParams p) {
     using G = Geom<D, DT>;
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -112,15 +133,18 @@ __global__ void __launch_bounds__(kHogWarps * 32) k_hogwild(HogwildParams p) {
     const int64_t rounds = (n + nw - 1) / nw;
     const uint32_t ctx_tab = p.order == 2 ? 1u : 0u;
     void* ctx = p.order == 2 ? p.C : p.U;
+    // a sample's record entry of this lane (R <= L), loaded one sample ahead
+    auto entry = [&](int64_t s) { return worker < nw && s < n && lig < R ? __ldg(p.rec + s * R + lig) : 0; };
+    int32_t held = R <= G::L ? entry(worker) : 0;
     for (int64_t r = 0; r < rounds; ++r) {
         const int64_t s = r * nw + worker;
         const bool active = worker < nw && s < n;
         if (R <= G::L) {
             // one slot per lane: the first slot of the worker holding the
             // same row of the same table, by matching keys across the warp
-            int32_t row = 0;
+            int32_t row = held;
+            if (r + 1 < rounds) held = entry(s + nw);
             if (active && lig < R) {
-                row = __ldg(p.rec + s * R + lig);
                 if (row < 0 || row >= p.n_nodes) {
                     atomicOr(p.status, DEV_ERR_INDEX);
                     row = 0;
@@ -159,30 +183,52 @@ __global__ void __launch_bounds__(kHogWarps * 32) k_hogwild(HogwildParams p) {
             }
         }
         __syncwarp(gm);
-        // the U row into registers, the distinct context rows into the
-        // stage, up to CH loads in flight per lane
-        constexpr int CH = 4;
+        // the U row into registers, the distinct context rows into the stage
         float x[G::E], x0[G::E];
         if (active) {
-            for (int k0 = 0; k0 < R; k0 += CH) {
-                float v[CH][G::E];
+            // 32 bytes and more a lane: the U row is one of the first CH
+            constexpr int FIRST = DT == LINE_DTYPE_F32 && G::E > 4 ? 0 : 1;
+            if (FIRST == 1) load_row<D, DT>(p.U, srow[0], lig, x0);
+            if constexpr (STAGED) {
+                // a lane reads back only what it copied
+                for (int k = 1; k < R; ++k) {
+                    if (sid[k] != k) continue;
+                    const float* from = reinterpret_cast<const float*>(ctx) + (int64_t)srow[k] * D + lig * G::E;
+                    float* to = stage + (size_t)k * D + lig * G::E;
 #pragma unroll
-                for (int kk = 0; kk < CH; ++kk) {
-                    const int k = k0 + kk;
-                    if (k < R && sid[k] == k) load_row<D, DT>(k == 0 ? p.U : ctx, srow[k], lig, v[kk]);
+                    for (int q = 0; q < G::NV; ++q) cp_async16(to + 4 * q, from + 4 * q);
                 }
-                if (k0 == 0) {
+                cp_async_wait_all();
+            } else {
+                constexpr int CH = DT == LINE_DTYPE_BF16 ? 6 : 4;
+                for (int k0 = FIRST; k0 < R; k0 += CH) {
+                    Packed<DT> v[CH][G::NV];
 #pragma unroll
-                    for (int e = 0; e < G::E; ++e) x0[e] = v[0][e];
-                }
+                    for (int kk = 0; kk < CH; ++kk) {
+                        const int k = k0 + kk;
+                        if (k >= R || sid[k] != k) continue;
+                        const Packed<DT>* from =
+                            reinterpret_cast<const Packed<DT>*>(k == 0 ? p.U : ctx) + ((int64_t)srow[k] * D + lig * G::E) / 4;
 #pragma unroll
-                for (int kk = 0; kk < CH; ++kk) {
-                    const int k = k0 + kk;
-                    if (k > 0 && k < R && sid[k] == k) {
+                        for (int q = 0; q < G::NV; ++q) v[kk][q] = __ldcg(from + q);
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < CH; ++kk) {
+                        const int k = k0 + kk;
+                        if (k >= R || sid[k] != k) continue;
                         float4* st = reinterpret_cast<float4*>(stage + (size_t)k * D + lig * G::E);
 #pragma unroll
-                        for (int q = 0; q < G::NV; ++q)
-                            st[q] = make_float4(v[kk][4 * q], v[kk][4 * q + 1], v[kk][4 * q + 2], v[kk][4 * q + 3]);
+                        for (int q = 0; q < G::NV; ++q) {
+                            const float4 f = unpack(v[kk][q]);
+                            if (FIRST == 1 || k > 0) {
+                                st[q] = f;
+                            } else {
+                                x0[4 * q] = f.x;
+                                x0[4 * q + 1] = f.y;
+                                x0[4 * q + 2] = f.z;
+                                x0[4 * q + 3] = f.w;
+                            }
+                        }
                     }
                 }
             }
@@ -255,8 +301,8 @@ __global__ void __launch_bounds__(kHogWarps * 32) k_hogwild(HogwildParams p) {
     }
 }
 
-template <int D, int DT>
-cudaError_t launch(const HogwildParams& p, int64_t max_workers, cudaStream_t s) {
+template <int D, int DT, bool STAGED>
+cudaError_t launch_as(const HogwildParams& p, int64_t max_workers, cudaStream_t s) {
     using G = Geom<D, DT>;
     constexpr size_t kMaxSmem = 227 * 1024;
     const size_t per_warp = (size_t)G::GPW * group_bytes(D, p.K);
@@ -284,7 +330,7 @@ cudaError_t launch(const HogwildParams& p, int64_t max_workers, cudaStream_t s) 
         cap = &allowed.back().second;
     }
     if (*cap < smem) {
-        if ((e = cudaFuncSetAttribute(k_hogwild<D, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+        if ((e = cudaFuncSetAttribute(k_hogwild<D, DT, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
             cudaSuccess)
             return e;
         *cap = smem;
@@ -297,7 +343,7 @@ cudaError_t launch(const HogwildParams& p, int64_t max_workers, cudaStream_t s) 
         }
     if (per_sm < 0) {
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hogwild<D, DT>, wpb * 32, smem)) != cudaSuccess)
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hogwild<D, DT, STAGED>, wpb * 32, smem)) != cudaSuccess)
             return e;
         waves.push_back({dev, p.K, sms, per_sm});
     }
@@ -307,8 +353,25 @@ cudaError_t launch(const HogwildParams& p, int64_t max_workers, cudaStream_t s) 
     q.workers = max_workers > 0 ? std::min<int64_t>(max_workers, full) : full;
     q.workers = std::min<int64_t>(q.workers, std::max<int64_t>(p.chunk_samples, 1));
     const unsigned grid = (unsigned)((q.workers + per_block - 1) / per_block);
-    k_hogwild<D, DT><<<grid, wpb * 32, smem, s>>>(q);
+    k_hogwild<D, DT, STAGED><<<grid, wpb * 32, smem, s>>>(q);
     return cudaGetLastError();
+}
+
+// Asynchronous copies for FP32 rows of 256 and 512 bytes in tables of 32 MB
+// and more: there the sample's loads are the bound (D = 128: 2^16 nodes 5.36
+// -> 4.56 ms, 2^20 nodes 5.84 -> 4.81).  Smaller tables lie in L2 with their
+// hub rows under contention, and more loads in flight only lengthen the queue
+// at those (2^14 nodes: up to 10% slower); rows of 64 and 128 bytes gain
+// nothing (D = 32, 2^20 nodes: 1.84 ms both), and 1 KB rows have enough in
+// flight by registers (D = 256, 2^20 nodes: 3.44 and 3.45 ms, 2^16: 3.53 and
+// 3.67).
+template <int D, int DT>
+cudaError_t launch(const HogwildParams& p, int64_t max_workers, cudaStream_t s) {
+    if constexpr (DT == LINE_DTYPE_F32 && (D == 64 || D == 128)) {
+        constexpr int64_t kLarge = (int64_t)32 << 20;
+        if (p.n_nodes * (int64_t)(D * sizeof(float)) >= kLarge) return launch_as<D, DT, true>(p, max_workers, s);
+    }
+    return launch_as<D, DT, false>(p, max_workers, s);
 }
 
 }  // namespace
