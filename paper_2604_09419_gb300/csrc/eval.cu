@@ -25,34 +25,107 @@ __device__ __forceinline__ uint32_t load_bits(const void* p, int64_t idx) {
     else return (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p) + idx) << 16;
 }
 
-// The FP32 value with bits b as FP64, in integer instructions; `odd` is set
-// for subnormals, infinities and NaNs, whose result is not valid.
-__device__ __forceinline__ double widen(uint32_t b, bool& odd) {
-    const uint32_t m = b & 0x7FFFFFFFu;
-    odd |= m != 0u && (m < 0x00800000u || m >= 0x7F800000u);
-    const uint32_t hi = (b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
-    return __hiloint2double((int)hi, (int)(b << 29));
+// FP32 bits of N consecutive values, idx a multiple of N.
+template <int N, int DT>
+__device__ __forceinline__ void load_bits(const void* p, int64_t idx, uint32_t (&b)[N]) {
+    if constexpr (N == 1) {
+        b[0] = load_bits<DT>(p, idx);
+    } else {
+        constexpr int W = DT == LINE_DTYPE_F32 ? N : N / 2;  // 32-bit words
+        uint32_t w[W];
+        const uint32_t* q = reinterpret_cast<const uint32_t*>(p) + (DT == LINE_DTYPE_F32 ? idx : idx / 2);
+        if constexpr (W == 1) {
+            w[0] = __ldg(q);
+        } else if constexpr (W == 2) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2*>(q));
+            w[0] = v.x;
+            w[1] = v.y;
+        } else {
+#pragma unroll
+            for (int k = 0; k < W; k += 4) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4*>(q) + k / 4);
+                w[k] = v.x;
+                w[k + 1] = v.y;
+                w[k + 2] = v.z;
+                w[k + 3] = v.w;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < N; ++k) b[k] = DT == LINE_DTYPE_F32 ? w[k * W / N] : (k & 1) ? w[k / 2] & 0xFFFF0000u : w[k / 2] << 16;
+    }
 }
+
+// A dot of FP32 rows in integers, IT products a lane: the 48-bit products of
+// the significands, SH bits above their last one, each shifted down by its
+// exponent's distance to the largest product's and summed exactly.  What is
+// lost are bits below 2^-(46 + SH) of the largest product, fewer than FP64
+// sums lose: against the exact dot over rows of normal, positive, widely
+// spread, subnormal and trained values and of one product above all others,
+// the rms and the largest error are below the FP64 chain's, by 2 to 20 times
+// at d >= 64 for rows whose sum cancels, by 1.1 to 3 times for the others.
+template <int IT>
+struct Fixed {
+    static constexpr int LOG = IT == 1 ? 0 : IT == 2 ? 1 : IT == 4 ? 2 : 3;
+    static constexpr int SH = IT == 1 ? 14 : 15 - LOG;  // a lane's sum stays below 2^63, each factor below 2^31
+    static constexpr int CUT = 27;       // limbs of the sum over 32 lanes: 32 2^27 fits 32 bits
+
+    // This lane's part of a dot; `top`: the largest product's exponent (of all
+    // lanes; twice biased, in place); `big`: |= an infinity or a NaN was met.
+    static __device__ __forceinline__ int64_t lane_sum(const uint32_t (&a)[IT], const uint32_t (&b)[IT], uint32_t& top, bool& big) {
+        int64_t p[IT];
+        uint32_t ex[IT], m = 0, mx = 0;
+#pragma unroll
+        for (int k = 0; k < IT; ++k) {
+            const uint32_t ea = a[k] & 0x7F800000u, eb = b[k] & 0x7F800000u;
+            mx = max(mx, max(ea, eb));
+            // subnormals: no leading bit, the smallest exponent
+            const uint32_t sa = (a[k] & 0x7FFFFFu) | min(ea, 0x800000u), sb = (b[k] & 0x7FFFFFu) | min(eb, 0x800000u);
+            const int32_t sg = (int32_t)(a[k] ^ b[k]) < 0 ? -(1 << (SH - 7)) : 1 << (SH - 7);
+            p[k] = (int64_t)(int32_t)(sa << 7) * ((int32_t)sb * sg);
+            ex[k] = p[k] ? max(ea, 0x800000u) + max(eb, 0x800000u) : 0u;
+            m = max(m, ex[k]);
+        }
+        big |= mx >= 0x7F800000u;
+        top = __reduce_max_sync(0xFFFFFFFFu, m);
+        int64_t sum = 0;
+#pragma unroll
+        for (int k = 0; k < IT; ++k) {
+            const uint32_t s = min((top - ex[k]) >> 23, 63u);
+            // eight products a lane leave fewer bits below: to nearest
+            sum += (p[k] + (IT > 4 ? (int64_t)((uint64_t)1 << s >> 1) : 0)) >> s;
+        }
+        return sum;
+    }
+    // The dot from the limbs' sums over the lanes.
+    static __device__ __forceinline__ double value(int64_t h, uint32_t lo, uint32_t top) {
+        const int e = (int)(top >> 23) - 300 - SH;
+        return fma((double)h, (double)(1u << CUT), (double)lo) * __hiloint2double((1023 + e) << 20, 0);
+    }
+};
 
 // One warp for a group of samples whose K+1 scores each fill its lanes (one
 // sample where K+1 > 32, in rounds of 32 scores).  Lane q draws its score's
-// row; the dots are taken eight at a time with all lanes on one, in FP64:
-// value k of a row in lane k mod 32, products added in order, lanes by
-// butterfly distances 16 .. 1 (transposed: each total in some lanes only);
-// then every lane evaluates the log-sigmoid of its own score, and a sample's
-// are subtracted in order.
-// Bound: GB300's FP64 pipe (two lanes a clock and SM, also for conversions).
+// row; the dots are taken N at a time with all lanes on one, IT consecutive
+// values a lane, in integers (Fixed); their limbs are reduced by transposed
+// butterflies (each total in some lanes only); then every lane evaluates the
+// log-sigmoid of its own score, and a sample's are subtracted in order.  Rows
+// with infinities or NaNs take FP64 sums, value k of a row in lane k mod 32.
+// Bound: issue slots of the integer dots (about 30 instructions a product) and
+// GB300's FP64 pipe in the log-sigmoids (two lanes a clock and SM, also for
+// conversions).  N = 3 at 64 registers keeps four blocks resident (8 at 117
+// registers: 1.85 ms, 4: 1.48).
 // One warp per sample, with all lanes on the same log-sigmoid and FP64
-// conversions of every value, took 25.2 ms for 2^20 samples of K = 5, d = 128;
-// this 2.77 ms.
+// conversions of every value, took 25.2 ms for 2^20 samples of K = 5, d = 128
+// FP32; FP64 sums of values widened by integer instructions 2.77; this 1.40.
 template <int D, int DT>
-__global__ void __launch_bounds__(256) k_loss_terms(const void* __restrict__ U, const void* __restrict__ Ctx, int K,
+__global__ void __launch_bounds__(256, 4) k_loss_terms(const void* __restrict__ U, const void* __restrict__ Ctx, int K,
                                                     const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                     const uint2* __restrict__ edge_tab, int64_t n_arcs,
                                                     const uint2* __restrict__ neg_tab, int64_t n_nodes, uint64_t seed,
                                                     int64_t m, double* __restrict__ terms) {
     constexpr int IT = D >= 32 ? D / 32 : 1;
-    constexpr int N = 8;
+    constexpr int N = D > 128 ? 2 : 3;
+    using F = Fixed<IT>;
     const int lane = threadIdx.x & 31;
     const bool holds = lane < D;
     const int C1 = K + 1, S = C1 <= 32 ? 32 / C1 : 1;
@@ -79,46 +152,67 @@ __global__ void __launch_bounds__(256) k_loss_terms(const void* __restrict__ U, 
                 u = __shfl_sync(0xFFFFFFFFu, u, lane < nq ? lane - j : 0);
                 u0 = u;  // (C1 > 32: the same in every lane)
             }
-            double score = 0.0;
+            int64_t h = 0;
+            uint32_t lo = 0, top = 0;
+            bool direct = false;  // h holds the score's bits
             for (int q0 = 0; q0 < nq; q0 += N) {
-                double part[N];
-                bool odd = false;
+                int64_t part[N];
+                uint32_t low[N], tops[N];
+                uint32_t a[N][IT], c[N][IT];
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
                     const int q = min(q0 + i, nq - 1);
                     const int64_t uq = __shfl_sync(0xFFFFFFFFu, u, q), yq = __shfl_sync(0xFFFFFFFFu, y, q);
-                    part[i] = 0.0;
+                    if (holds) {
+                        load_bits<IT, DT>(U, uq * D + lane * IT, a[i]);
+                        load_bits<IT, DT>(Ctx, yq * D + lane * IT, c[i]);
+                    } else {
 #pragma unroll
-                    for (int k = 0; k < IT; ++k) {
-                        const uint32_t a = holds ? load_bits<DT>(U, uq * D + k * 32 + lane) : 0u;
-                        const uint32_t c = holds ? load_bits<DT>(Ctx, yq * D + k * 32 + lane) : 0u;
-                        part[i] = fma(widen(a, odd), widen(c, odd), part[i]);
+                        for (int k = 0; k < IT; ++k) a[i][k] = c[i][k] = 0u;
                     }
                 }
-                if (__any_sync(0xFFFFFFFFu, odd)) {  // the same with the conversion instruction
+                bool big = false;
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    const int64_t sum = F::lane_sum(a[i], c[i], tops[i], big);
+                    low[i] = (uint32_t)sum & ((1u << F::CUT) - 1u);
+                    part[i] = sum >> F::CUT;
+                }
+                if (__any_sync(0xFFFFFFFFu, big)) {
 #pragma unroll 1
                     for (int i = 0; i < N; ++i) {
                         const int q = min(q0 + i, nq - 1);
                         const int64_t uq = __shfl_sync(0xFFFFFFFFu, u, q), yq = __shfl_sync(0xFFFFFFFFu, y, q);
                         double v = 0.0;
                         for (int k = 0; k < IT; ++k) {
-                            const uint32_t a = holds ? load_bits<DT>(U, uq * D + k * 32 + lane) : 0u;
-                            const uint32_t c = holds ? load_bits<DT>(Ctx, yq * D + k * 32 + lane) : 0u;
-                            v = fma((double)__uint_as_float(a), (double)__uint_as_float(c), v);
+                            const uint32_t x = holds ? load_bits<DT>(U, uq * D + k * 32 + lane) : 0u;
+                            const uint32_t z = holds ? load_bits<DT>(Ctx, yq * D + k * 32 + lane) : 0u;
+                            v = fma((double)__uint_as_float(x), (double)__uint_as_float(z), v);
                         }
 #pragma unroll
-                        for (int k = 0; k < N; ++k)
-                            if (k == i) part[k] = v;
+                        for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+                        if (lane == q0 + i) {
+                            h = __double_as_longlong(v);
+                            direct = true;
+                        }
                     }
+                    continue;
                 }
                 using T = Transposed<32, N>;
                 T::reduce(part, lane);
+                T::reduce(low, lane);
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
-                    const double v = __shfl_sync(0xFFFFFFFFu, part[0], T::lane(i));
-                    if (lane == q0 + i) score = v;
+                    const int64_t vh = __shfl_sync(0xFFFFFFFFu, part[0], T::lane(i));
+                    const uint32_t vl = __shfl_sync(0xFFFFFFFFu, low[0], T::lane(i));
+                    if (lane == q0 + i) {
+                        h = vh;
+                        lo = vl;
+                        top = tops[i];
+                    }
                 }
             }
+            const double score = direct ? __longlong_as_double(h) : F::value(h, lo, top);
             const double ls = lane < nq ? log_sigmoid(j == 0 ? score : -score) : 0.0;
             const int per = C1 <= 32 ? C1 : nq;
             for (int k = 0; k < per; ++k) L -= __shfl_sync(0xFFFFFFFFu, ls, min(lane * C1, 31) + k & 31);
