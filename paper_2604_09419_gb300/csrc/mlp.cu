@@ -177,55 +177,59 @@ struct FGeom {
     static constexpr int LANES = D / E;
 };
 
+// A lane's values of a row as they lie in memory (one load), and the sum.
 template <int D, int UDT>
-__device__ __forceinline__ void load_vals(const void* U, int64_t row, int lane, float (&v)[FGeom<D>::E]) {
-    constexpr int E = FGeom<D>::E;
-    if constexpr (UDT == LINE_DTYPE_F32) {
-        const float* p = reinterpret_cast<const float*>(U) + row * D + lane * E;
-        if constexpr (E == 8) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-        } else if constexpr (E == 4) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-        } else if constexpr (E == 2) {
-            const float2 a = __ldg(reinterpret_cast<const float2*>(p));
-            v[0] = a.x; v[1] = a.y;
+struct RowWords {
+    static constexpr int E = FGeom<D>::E;
+    static constexpr int N = UDT == LINE_DTYPE_F32 ? E : (E + 1) / 2;  // 32-bit words
+    uint32_t w[N];
+    __device__ __forceinline__ void load(const void* U, int64_t row, int lane) {
+        const int64_t at = row * D + lane * E;
+        if constexpr (UDT == LINE_DTYPE_BF16 && E == 1) {
+            w[0] = (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(U) + at) << 16;
         } else {
-            v[0] = __ldg(p);
-        }
-    } else {
-        const __nv_bfloat16* p = reinterpret_cast<const __nv_bfloat16*>(U) + row * D + lane * E;
-        if constexpr (E == 8) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4*>(p));
-            const uint32_t w[4] = {a.x, a.y, a.z, a.w};
+            const uint32_t* p = reinterpret_cast<const uint32_t*>(U) + (UDT == LINE_DTYPE_F32 ? at : at / 2);
+            if constexpr (N == 1) {
+                w[0] = __ldg(p);
+            } else if constexpr (N == 2) {
+                const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+                w[0] = v.x;
+                w[1] = v.y;
+            } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                v[2 * i] = __uint_as_float(w[i] << 16);
-                v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+                for (int k = 0; k < N; k += 4) {
+                    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p) + k / 4);
+                    w[k] = v.x;
+                    w[k + 1] = v.y;
+                    w[k + 2] = v.z;
+                    w[k + 3] = v.w;
+                }
             }
-        } else if constexpr (E == 4) {
-            const uint2 a = __ldg(reinterpret_cast<const uint2*>(p));
-            v[0] = __uint_as_float(a.x << 16); v[1] = __uint_as_float(a.x & 0xFFFF0000u);
-            v[2] = __uint_as_float(a.y << 16); v[3] = __uint_as_float(a.y & 0xFFFF0000u);
-        } else if constexpr (E == 2) {
-            const uint32_t a = __ldg(reinterpret_cast<const unsigned int*>(p));
-            v[0] = __uint_as_float(a << 16); v[1] = __uint_as_float(a & 0xFFFF0000u);
-        } else {
-            v[0] = __bfloat162float(p[0]);
         }
     }
-}
+    __device__ __forceinline__ void add_to(float (&acc)[E]) const {
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            if constexpr (UDT == LINE_DTYPE_F32 || E == 1) acc[i] += __uint_as_float(w[i]);
+            else acc[i] += __uint_as_float((i & 1) ? w[i / 2] & 0xFFFF0000u : w[i / 2] << 16);
+        }
+    }
+};
 
 // Adds the rows U[dst[e]] of the known neighbours among arcs [lo, hi) to acc
 // in arc order (each value's sum runs over the neighbours in arc order);
-// returns their number.  Arcs are taken 32 at a time (one per lane), and up
-// to 8 known rows (4 at d = 256) are loaded at once before they are added.
+// returns their number.  Arcs are taken 32 at a time (one per lane), and
+// kGroup known rows are loaded at once, as they lie, before they are added (few:
+// the warps in flight hide more than longer groups, whose registers cost
+// warps: BF16 rows of 128, 4 rows and 4 blocks 150 us for the two kinds of
+// nodes of k_mlp_features, 8 rows and 3 blocks 191, 12 to 16 rows and 2 blocks
+// with the loads of the next nodes ahead 200).
 template <int D, int UDT>
 __device__ __forceinline__ int sum_known_rows(int64_t lo, int64_t hi, const int32_t* __restrict__ dst, const void* U,
                                              const uint8_t* __restrict__ known, float (&acc)[FGeom<D>::E]) {
     using F = FGeom<D>;
-    constexpr int kGroup = F::E <= 4 ? 8 : 4;
+    using Words = RowWords<D, UDT>;
+    constexpr int kGroup = Words::N == 1 ? 8 : Words::N == 8 ? 2 : 4;
     const int lane = threadIdx.x & 31;
     const bool holds = lane < F::LANES;
     int cnt = 0;
@@ -248,15 +252,13 @@ __device__ __forceinline__ int sum_known_rows(int64_t lo, int64_t hi, const int3
                     m = j + 1;
                 }
             }
-            float val[kGroup][F::E];
+            Words row[kGroup];
 #pragma unroll
             for (int j = 0; j < kGroup; ++j)
-                if (j < m && holds) load_vals<D, UDT>(U, rows[j], lane, val[j]);
+                if (j < m && holds) row[j].load(U, rows[j], lane);
 #pragma unroll
             for (int j = 0; j < kGroup; ++j)
-                if (j < m)
-#pragma unroll
-                    for (int i = 0; i < F::E; ++i) acc[i] += val[j][i];
+                if (j < m) row[j].add_to(acc);
         }
     }
     return cnt;
@@ -272,12 +274,6 @@ __device__ __forceinline__ void write_features(TX* x, float deg, const float (&a
         for (int i = 0; i < F::E; ++i) x[1 + lane * F::E + i] = from_f<TX>(cnt ? acc[i] / (float)cnt : 0.0f);
     }
     for (int k = D + 1 + lane; k < P; k += 32) x[k] = from_f<TX>(0.0f);
-}
-
-// flag |= 1 if a requested row id is out of range.
-__global__ void k_check_rows(const int32_t* __restrict__ rows, int64_t n_rows, int64_t n_nodes, uint32_t* flag) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_rows; i += (int64_t)gridDim.x * blockDim.x)
-        if (rows[i] < 0 || rows[i] >= n_nodes) atomicOr(flag, 1u);
 }
 
 struct FeatParams {
@@ -298,34 +294,23 @@ struct FeatParams {
     uint32_t* pcnt;    // [slots] their known-neighbour counts
     const int32_t* rows;
     int64_t n_rows;
-    const uint32_t* flag;
+    uint32_t* flag;
 };
 
-// One warp per node; nodes with more than kHubArcs arcs are listed in hubs
-// (order irrelevant) and left to k_mlp_features_hub.  Nothing is written
-// when *flag is set (a requested row id was out of range).
-template <int D, int UDT, typename TX>
-__global__ void __launch_bounds__(256, 3) k_mlp_features(FeatParams p) {
-    if (*(volatile const uint32_t*)p.flag) return;
-    using F = FGeom<D>;
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+// Lists the hubs among the nodes asked for (each once, in any order); a row
+// id out of range sets *flag, and nothing is written by what follows.
+__global__ void k_list_hubs(FeatParams p) {
     const int64_t count = p.rows ? p.n_rows : p.n_nodes;
-    for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < count; r += warps) {
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < count; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = p.rows ? (int64_t)p.rows[r] : r;
-        const int64_t lo = __ldg(p.row_ptr + v), hi = __ldg(p.row_ptr + v + 1);
-        if (hi - lo > kHubArcs) {
-            if (lane == 0) {
-                const uint32_t bit = 1u << (v & 31);
-                if (!(atomicOr(p.hub_map + (v >> 5), bit) & bit)) p.hubs[atomicAdd(p.n_hubs, 1u)] = (uint32_t)v;
-            }
+        if (v < 0 || v >= p.n_nodes) {
+            atomicOr(p.flag, 1u);
             continue;
         }
-        float acc[F::E];
-#pragma unroll
-        for (int i = 0; i < F::E; ++i) acc[i] = 0.0f;
-        const int cnt = sum_known_rows<D, UDT>(lo, hi, p.dst, p.U, p.known, acc);
-        write_features<D, TX>(reinterpret_cast<TX*>(p.X) + v * (int64_t)p.P, __ldg(p.deg + v), acc, cnt, p.P);
+        if (__ldg(p.row_ptr + v + 1) - __ldg(p.row_ptr + v) > kHubArcs) {
+            const uint32_t bit = 1u << (v & 31);
+            if (!(atomicOr(p.hub_map + (v >> 5), bit) & bit)) p.hubs[atomicAdd(p.n_hubs, 1u)] = (uint32_t)v;
+        }
     }
 }
 
@@ -392,50 +377,66 @@ __global__ void __launch_bounds__(kPlanThreads) k_hub_plan(FeatParams p) {
     }
 }
 
-// Chunk i of the hubs' arcs (hub h = the last with off[h] <= i, chunk
-// c = i - off[h] of kHubChunk arcs): warp w sums the w-th of kHubWarps
-// contiguous slices of the chunk, the warps' sums are added in warp order;
-// a one-chunk hub's inputs are written at once, the other chunks' sums go
-// to their slots for k_hub_combine.
+// The inputs' sums.  First the hubs, a chunk of kHubChunk arcs a block
+// (chunk i of the list: hub h = the last with off[h] <= i, its chunk
+// c = i - off[h]): warp w sums the w-th of kHubWarps contiguous slices, the
+// warps' sums are added in warp order; a one-chunk hub's inputs are written at
+// once, the other chunks' sums go to their slots for k_hub_combine.  Then the
+// other nodes, one warp each.
+// Bound by the chain of loads to a row (id, arcs' range, target, known mark,
+// row) and the instructions of short nodes, so four blocks are resident (three
+// for rows of 256, which hold more registers).  Chunks and nodes in one kernel
+// fill each other's tails; a chunk's hub is found by a 32-way search, and the
+// block goes on to its next chunk while warp 0 adds the warps' sums.  R-MAT
+// 20, BF16 rows of 128: a sample of 65,536 nodes 243 -> 121 us, the 104,857
+// new nodes 340 -> 180 (two kernels, a binary search, two barriers a chunk).
+template <int D>
+constexpr int kFeatureBlocks = D <= 128 ? 4 : 3;
+
 template <int D, int UDT, typename TX>
-__global__ void __launch_bounds__(kHubWarps * 32) k_mlp_features_hub(FeatParams p) {
+__global__ void __launch_bounds__(kHubWarps * 32, kFeatureBlocks<D>) k_mlp_features(FeatParams p) {
+    if (*(volatile const uint32_t*)p.flag) return;
     using F = FGeom<D>;
-    __shared__ float part[kHubWarps][D];
-    __shared__ int pcnt[kHubWarps];
+    __shared__ float part[2][kHubWarps][D];
+    __shared__ int pcnt[2][kHubWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nh = *p.n_hubs;
     const uint32_t total = p.off[nh];
-    for (uint32_t i = blockIdx.x; i < total; i += gridDim.x) {
-        uint32_t lo_h = 0, hi_h = nh;  // off[lo_h] <= i < off[hi_h]
-        while (hi_h - lo_h > 1) {
-            const uint32_t mid = (lo_h + hi_h) >> 1;
-            if (p.off[mid] <= i) lo_h = mid;
-            else hi_h = mid;
+    int b = 0;
+    for (uint32_t i = blockIdx.x; i < total; i += gridDim.x, b ^= 1) {
+        uint32_t h = 0, n = nh;  // off[h] <= i < off[h + n]
+        while (n > 1) {
+            const uint32_t step = (n + 31) / 32;
+            const uint32_t at = lane * step;
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, at < n && p.off[h + at] <= i);  // lane 0 always
+            const uint32_t k = 31 - __clz(m);
+            h += k * step;
+            n = min(step, n - k * step);
         }
-        const uint32_t h = lo_h, c = i - p.off[h];
+        const uint32_t c = i - p.off[h];
         const int64_t v = p.hubs[h];
         const int64_t vlo = p.row_ptr[v], vhi = p.row_ptr[v + 1];
         const int64_t clo = vlo + (int64_t)c * kHubChunk, chi = min(vhi, clo + kHubChunk);
         const int64_t per = (chi - clo + kHubWarps - 1) / kHubWarps;
-        const int64_t a = min(chi, clo + warp * per), b = min(chi, a + per);
+        const int64_t lo = min(chi, clo + warp * per), hi = min(chi, lo + per);
         float acc[F::E];
 #pragma unroll
         for (int k = 0; k < F::E; ++k) acc[k] = 0.0f;
-        const int cw = sum_known_rows<D, UDT>(a, b, p.dst, p.U, p.known, acc);
+        const int cw = sum_known_rows<D, UDT>(lo, hi, p.dst, p.U, p.known, acc);
         if (lane < F::LANES)
 #pragma unroll
-            for (int k = 0; k < F::E; ++k) part[warp][lane * F::E + k] = acc[k];
-        if (lane == 0) pcnt[warp] = cw;
-        __syncthreads();
+            for (int k = 0; k < F::E; ++k) part[b][warp][lane * F::E + k] = acc[k];
+        if (lane == 0) pcnt[b][warp] = cw;
+        __syncthreads();  // part[b] is rewritten two chunks on, past the next of these
         if (warp == 0) {
             int cnt = 0;
 #pragma unroll
             for (int k = 0; k < F::E; ++k) acc[k] = 0.0f;
             for (int w = 0; w < kHubWarps; ++w) {
-                cnt += pcnt[w];
+                cnt += pcnt[b][w];
                 if (lane < F::LANES)
 #pragma unroll
-                    for (int k = 0; k < F::E; ++k) acc[k] += part[w][lane * F::E + k];
+                    for (int k = 0; k < F::E; ++k) acc[k] += part[b][w][lane * F::E + k];
             }
             if (vhi - vlo <= kHubChunk) {
                 write_features<D, TX>(reinterpret_cast<TX*>(p.X) + v * (int64_t)p.P, p.deg[v], acc, cnt, p.P);
@@ -447,7 +448,18 @@ __global__ void __launch_bounds__(kHubWarps * 32) k_mlp_features_hub(FeatParams 
                 if (lane == 0) p.pcnt[slot] = (uint32_t)cnt;
             }
         }
-        __syncthreads();
+    }
+    const int64_t count = p.rows ? p.n_rows : p.n_nodes;
+    const int64_t warps = (int64_t)gridDim.x * kHubWarps;
+    for (int64_t r = blockIdx.x * (int64_t)kHubWarps + warp; r < count; r += warps) {
+        const int64_t v = p.rows ? (int64_t)p.rows[r] : r;
+        const int64_t lo = __ldg(p.row_ptr + v), hi = __ldg(p.row_ptr + v + 1);
+        if (hi - lo > kHubArcs) continue;
+        float acc[F::E];
+#pragma unroll
+        for (int i = 0; i < F::E; ++i) acc[i] = 0.0f;
+        const int cnt = sum_known_rows<D, UDT>(lo, hi, p.dst, p.U, p.known, acc);
+        write_features<D, TX>(reinterpret_cast<TX*>(p.X) + v * (int64_t)p.P, __ldg(p.deg + v), acc, cnt, p.P);
     }
 }
 
@@ -455,13 +467,14 @@ __global__ void __launch_bounds__(kHubWarps * 32) k_mlp_features_hub(FeatParams 
 // order, then its inputs written.
 template <int D, typename TX>
 __global__ void k_hub_combine(FeatParams p) {
+    if (*(volatile const uint32_t*)p.flag) return;
     using F = FGeom<D>;
     const int lane = threadIdx.x & 31;
     const uint32_t nh = *p.n_hubs;
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
     for (uint32_t h = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); h < nh; h += warps) {
         const uint32_t c0 = p.poff[h], c1 = p.poff[h + 1];
-        if (c1 == c0) continue;  // one chunk: written by k_mlp_features_hub
+        if (c1 == c0) continue;  // one chunk: written by k_mlp_features
         float acc[F::E];
 #pragma unroll
         for (int k = 0; k < F::E; ++k) acc[k] = 0.0f;
@@ -479,10 +492,9 @@ __global__ void k_hub_combine(FeatParams p) {
 
 template <int D, int UDT, typename TX>
 cudaError_t launch_features(const FeatParams& p, int64_t count, int64_t max_hubs, cudaStream_t s) {
-    const unsigned g = (unsigned)std::min<int64_t>((count + 7) / 8, 152 * 16);
-    k_mlp_features<D, UDT, TX><<<g, 256, 0, s>>>(p);
+    k_list_hubs<<<(unsigned)std::min<int64_t>((count + 255) / 256, 152 * 16), 256, 0, s>>>(p);
     k_hub_plan<<<1, kPlanThreads, 0, s>>>(p);
-    k_mlp_features_hub<D, UDT, TX><<<152 * 4, kHubWarps * 32, 0, s>>>(p);
+    k_mlp_features<D, UDT, TX><<<152 * kFeatureBlocks<D>, kHubWarps * 32, 0, s>>>(p);
     k_hub_combine<D, TX><<<(unsigned)std::min<int64_t>((max_hubs + 7) / 8, 152 * 4), 256, 0, s>>>(p);
     return cudaGetLastError();
 }
@@ -1607,9 +1619,6 @@ static line_status mlp_features_impl(line_ctx* c, const char* what, const uint8_
     if (e == cudaSuccess) e = cudaMemsetAsync(hub_map, 0, sizeof(uint32_t) * ((size_t)hs.map_words + 1), str);
     if (e == cudaSuccess) e = cudaMemsetAsync(s.flag, 0, sizeof(uint32_t), str);
     if (e == cudaSuccess) {
-        // ids out of range are refused before any work: the flag stops the
-        // input kernels
-        if (rows) k_check_rows<<<grid_of(n_rows, 256, 152 * 16), 256, 0, str>>>(rd, n_rows, c->n_nodes, s.flag);
         const int64_t count = rows ? n_rows : c->n_nodes;
         FeatParams fp{c->n_nodes, c->row_ptr, c->dst,  c->deg,   t.U,      s.kmask, s.P,    s.X,   hub_map, hubs + 1,
                       hubs,       hub_off,    hub_poff, hub_part, hub_pcnt, rd,      n_rows, s.flag};
