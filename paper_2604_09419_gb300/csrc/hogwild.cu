@@ -109,8 +109,9 @@ __device__ __forceinline__ float4 unpack(uint2 v) {
 // at most CH at a time (BF16 rows must: they are widened on the way).  A
 // sample's record is loaded while the sample before is computed.  4.2 million
 // samples, K = 5, device memory tables (R-MAT 20, D = 128 FP32): 5.84 -> 4.81
-// ms, floor 4.78; BF16 7.98 -> 7.51; D = 64, K = 10, FP32 4.94 -> 4.01.  Eight
-// resident blocks (64 registers) of the STAGED form: ten (48) are 3% slower.
+// ms, floor 4.78; BF16 7.98 -> 7.51; D = 64, K = 10, FP32 4.94 -> 4.01.  The
+// STAGED form's bound of 8 blocks (55 registers, nine resident) is 3% faster
+// than none (47, ten), a bound of 9 or 7 4% slower than it.
 template <int D, int DT, bool STAGED>
 __global__ void __launch_bounds__(kHogWarps * 32, STAGED ? 8 : 0)
     k_hogwild(HogwildParams p) {

@@ -5,17 +5,17 @@
 //   pre-pass (index work only; it does not read the tables), on its own
 //   low-priority stream so that it overlaps the previous chunk's data phase:
 //     1. draws: for every sample its arc (u, v) and K negatives, kept as a
-//        record (u, v, n_1..n_K), and K+2 items, one per row the sample
-//        touches: key = row id, value = (sample, slot).  Slot 0 is U[u];
-//        slots 1..K+1 are the context rows Ctx[v], Ctx[n_j] (Ctx = C for
-//        second order, U for first order; C rows get ids offset by n).
-//     2. per batch, a stable counting sort of the batch's items into 256
-//        buckets by a hash of the row id;
-//     3. per (batch, bucket), a stable sort by row id, then the segments: runs of equal row = the rows the batch touches,
-//        entries in (sample, slot) order.  A segment with one entry is a
-//        singleton: its row is read and written by one sample only.  Every
-//        (sample, slot) learns its position and its segment; segments with
-//        two or more entries ("shared") are listed per batch with their first
+//        record (u, v, n_1..n_K): one entry, or item, per row the sample
+//        touches.  Slot 0 is U[u]; slots 1..K+1 are the context rows Ctx[v],
+//        Ctx[n_j] (Ctx = C for second order, U for first order; C rows get
+//        ids offset by n).
+//     2. per batch, the grouping of its items by row (k_group_parts; for
+//        batches beyond its range a bucketing through global memory and a
+//        sort per bucket): a segment is the items of one row, in (sample,
+//        slot) order.  A segment with one entry is a singleton: its row is
+//        read and written by one sample only.  Every (sample, slot) learns
+//        its position and its segment; segments with two or more entries
+//        ("shared") are listed per batch, by length class, with their first
 //        position, length, row and pair count.
 //
 //   data phase, batch after batch:
