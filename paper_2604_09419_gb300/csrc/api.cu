@@ -68,7 +68,7 @@ bool on_device(const line_ctx* c, const void* p) {
 line_status ensure_walk_tables(line_ctx* c) {
     if (c->cw_ok) return LINE_OK;
     cudaError_t e = grow(&c->cw, &c->cw_cap, sizeof(double) * (size_t)std::max<int64_t>(1, c->n_arcs));
-    if (e == cudaSuccess) e = walk_cumw(c->n_nodes, c->row_ptr, c->w, c->cw, c->stream);
+    if (e == cudaSuccess) e = walk_cumw(c->n_nodes, c->row_ptr, c->w, c->whole, c->cw, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "walk sampler tables");
     c->cw_ok = true;
     return LINE_OK;
@@ -259,6 +259,7 @@ line_status line_build_alias(line_ctx* c, const line_graph_desc* g) {
         // integer weights whose sum is below 2^53: every FP64 sum of them is
         // exact, in any order
         const bool whole = !found.frac && found.sum < (1ull << 53);
+        c->whole = whole;
         const double total_w = (double)found.sum;
         // edge table: arc weights (Algorithm 3)
         if ((e = alias_build_arcs(w, m, whole ? &total_w : nullptr, whole, c->edge_tab, tmp, c->status, s)) != cudaSuccess) { result = cuda_fail(c, e, "edge alias"); break; }

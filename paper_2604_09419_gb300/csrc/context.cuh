@@ -42,6 +42,7 @@ struct line_ctx {
     // weight sums per node (walks), built on first use for the current graph
     // (cw_ok); their allocations outlive the graph, like src..deg
     int64_t* row_ptr = nullptr;
+    bool whole = false;  // the arc weights are integers of at most 2^24 whose sum is below 2^53
     double* cw = nullptr;
     bool cw_ok = false;
     size_t row_ptr_cap = 0, cw_cap = 0;

@@ -58,11 +58,12 @@ __device__ __forceinline__ void load_bits(const void* p, int64_t idx, uint32_t (
 // A dot of FP32 rows in integers, IT products a lane: the 48-bit products of
 // the significands, SH bits above their last one, each shifted down by its
 // exponent's distance to the largest product's and summed exactly.  What is
-// lost are bits below 2^-(46 + SH) of the largest product, fewer than FP64
-// sums lose: against the exact dot over rows of normal, positive, widely
-// spread, subnormal and trained values and of one product above all others,
-// the rms and the largest error are below the FP64 chain's, by 2 to 20 times
-// at d >= 64 for rows whose sum cancels, by 1.1 to 3 times for the others.
+// lost are bits below 2^-(46 + SH) of the largest product (where a factor of
+// it is subnormal, of 2^-126 times the other), fewer than FP64 sums lose:
+// against the exact dot over rows of normal, positive, widely spread,
+// subnormal and trained values and of one product above all others, the rms
+// and the largest error are below the FP64 chain's, by 2 to 20 times at
+// d >= 64 for rows whose sum cancels, by 1.1 to 3 times for the others.
 template <int IT>
 struct Fixed {
     static constexpr int LOG = IT == 1 ? 0 : IT == 2 ? 1 : IT == 4 ? 2 : 3;

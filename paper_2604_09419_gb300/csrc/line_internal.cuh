@@ -200,8 +200,9 @@ struct WalkParams {
     int32_t* rec;            // rec[s R], rec[s R + 1] = the pair of sample t0 + s
 };
 size_t walk_smem_bytes(int L);
-// cw[m]: running FP64 sums of each node's arc weights (w nullable: weight 1).
-cudaError_t walk_cumw(int64_t n_nodes, const int64_t* row_ptr, const float* w, double* cw, cudaStream_t s);
+// cw[m]: running FP64 sums of each node's arc weights (w nullable: weight 1;
+// whole: integers of at most 2^24 whose sum is below 2^53).
+cudaError_t walk_cumw(int64_t n_nodes, const int64_t* row_ptr, const float* w, bool whole, double* cw, cudaStream_t s);
 cudaError_t walk_pairs(const WalkParams& p, cudaStream_t s);
 
 // eval.cu
