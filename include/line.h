@@ -114,8 +114,9 @@ typedef struct {
     int chunk_batches;       /* batches per pre-pass chunk; 0: automatic */
     int warps_per_block;     /* 0: automatic */
     int timing;              /* 1: time the training kernels with CUDA events (line_get_stats) */
-    int graph;               /* 1: batched mode replays each full chunk's launches from a
-                                captured CUDA graph (same results); 0: direct launches */
+    int graph;               /* 1: batched mode replays a chunk's launches from a captured
+                                CUDA graph where the chunk recurs, within a call or from
+                                call to call (same results); 0: direct launches */
     int walk_length;         /* L > 0: positive pairs from random walks of L steps
                                 (Algorithms 2-3, see line_sample_walk_debug); 0: arcs
                                 drawn by weight (Eq. 1).  At most 1024. */
@@ -187,11 +188,11 @@ LINE_API const char* line_last_error(const line_ctx* ctx);
  * are kept when the new graph has the same n_nodes - so training can
  * continue on a changed edge set - and dropped otherwise.  The library
  * keeps its own device copy of src, dst and w (4 bytes per arc each; w only
- * when given), the alias tables and the weighted degrees; per-node arc
- * offsets (8 bytes per node) and the walk sampler's weight sums (8 bytes per
+ * when given), the alias tables, the weighted degrees and the nodes' arc
+ * offsets (8 bytes per node); the walk sampler's weight sums (8 bytes per
  * arc) are added on first use.  A later graph reuses these buffers (and the
- * build's FP64 scratch, 8 bytes per arc or node) when they are large enough;
- * they are freed by line_destroy.
+ * build's scratch) when they are large enough; they are freed by
+ * line_destroy.
  * Errors: LINE_ERR_ARG (sizes), LINE_ERR_VALIDATE (unsorted src, ids out of
  * range, non-positive or non-finite weights, a node set with no positive
  * weight), LINE_ERR_OOM. */
@@ -229,9 +230,8 @@ LINE_API line_status line_sample_debug(line_ctx* ctx, int K, uint64_t seed, uint
  * order.  Negatives are the edge sampler's (domain 0, calls 1..K at counter
  * t).  With reuse r > 1 each walk's pairs serve r passes in a row: sample
  * t takes pair t mod P of walk t / (r P).  The first call on a graph builds
- * the per-node arc offsets and weight sums (12 bytes per arc with the kept
- * weights, 8 per node); their memory is reused by later graphs that fit and
- * freed by line_destroy.
+ * the weight sums (8 bytes per arc); their memory is reused by later graphs
+ * that fit and freed by line_destroy.
  * Errors: LINE_ERR_ARG (K, count, not 1 <= W <= L <= 1024, or reuse
  * outside 1..1024),
  * LINE_ERR_STATE (no graph). */
@@ -322,8 +322,9 @@ LINE_API line_status line_set_embeddings(line_ctx* ctx, int order, int which, co
 
 /* Negative-sampling LINE loss over the first m samples of draw domain 3:
  * L = -sum_t [log sigma(s+) + sum_j log sigma(-s-_j)], s = U[u].Ctx[y]
- * computed in FP64 from the stored values, summed in a fixed order.
- * Result in *out_host (host pointer). */
+ * computed from the stored values to FP64 accuracy (a dot loses only bits
+ * below 2^-58 of its largest product, then rounds once), summed in FP64 in a
+ * fixed order.  Result in *out_host (host pointer). */
 LINE_API line_status line_eval_loss(line_ctx* ctx, int order, int K, uint64_t seed, int64_t m, double* out_host);
 
 /* Link-prediction AUC: held-out edges against non-edges (the paper's own
@@ -346,7 +347,8 @@ LINE_API line_status line_eval_loss(line_ctx* ctx, int order, int K, uint64_t se
  * Errors: LINE_ERR_ARG (bad mask or score, counts, null pointers, or a node
  * id out of range), LINE_ERR_STATE (a requested order has no tables),
  * LINE_ERR_VALIDATE (a score is NaN: non-finite table values), LINE_ERR_OOM,
- * LINE_ERR_CUDA.  Allocates scratch for the pairs per call; synchronises. */
+ * LINE_ERR_CUDA.  Keeps up to 256 MB of scratch for the pairs until
+ * line_destroy (more is allocated for the call); synchronises. */
 LINE_API line_status line_eval_auc(line_ctx* ctx, int orders, int score, const int32_t* pos_src, const int32_t* pos_dst,
                                    int64_t n_pos, const int32_t* neg_src, const int32_t* neg_dst, int64_t n_neg,
                                    float* scores_out, uint64_t* counts_out, double* auc_out);
