@@ -121,8 +121,10 @@ typedef struct {
                                 (Algorithms 2-3, see line_sample_walk_debug); 0: arcs
                                 drawn by weight (Eq. 1).  At most 1024. */
     int window;              /* W: pair window of the walk sampler, 1 <= W <= L */
-    int hogwild_workers;     /* LINE_MODE_HOGWILD: samples in flight at once (>= 0; 0: one
-                                resident wave of the GPU, one worker per lane group) */
+    int hogwild_workers;     /* LINE_MODE_HOGWILD: samples in flight at once (>= 0; 0: a wave of
+                                32 warps per SM, 20 and 16 for FP32 and BF16 rows of 256
+                                values, one worker per lane group; 4,864 at dim 128.  Fewer
+                                where K and dim leave shared memory for fewer.  At most that) */
     int walk_reuse;          /* r: passes over each walk's pairs, 1..1024 (0 means 1): sample t
                                 takes pair t mod P of walk t / (r P) - a single-device form of
                                 the Reuse-Spill variant (§IV-C) */

@@ -30,7 +30,6 @@
 // of the sample's batch.
 #include <algorithm>
 #include <mutex>
-#include <type_traits>
 #include <vector>
 
 #include "bulk.cuh"
@@ -41,6 +40,16 @@ namespace line {
 namespace {
 
 constexpr int kHogWarps = 4;   // warps per block, at most (fewer when a block's stages exceed the shared memory)
+
+// Blocks of the default wave per SM (fewer where the stages leave room for
+// fewer).  The number of samples in flight is part of what the schedule
+// computes, as each works on rows that the others are changing: it is stated
+// here and does not follow from a kernel's registers.  On R-MAT 20 at D = 128
+// nine blocks, which the copying form's 55 registers allow, gave tables
+// 3.1e-3 (U) and 3.6e-3 (C) away from those of eight, whose own runs lie 2.2e-3
+// and 2.3e-3 apart (relative 2-norms after 2^22 samples).
+template <int D, int DT>
+constexpr int kWave = D <= 128 ? 8 : DT == LINE_DTYPE_F32 ? 5 : 4;
 
 // Shared memory per lane group: the staged rows, then the record and the
 // first-occurrence slot of each slot, rounded up to 16 bytes.
@@ -93,11 +102,8 @@ __device__ __forceinline__ void add_row(void* table, int64_t row, int lig, const
     }
 }
 
-// Four consecutive values of a row as they lie in memory, and as floats.
-template <int DT>
-using Packed = std::conditional_t<DT == LINE_DTYPE_F32, float4, uint2>;
-__device__ __forceinline__ float4 unpack(float4 v) { return v; }
-__device__ __forceinline__ float4 unpack(uint2 v) {
+// Four consecutive BF16 values as floats.
+__device__ __forceinline__ float4 widen(uint2 v) {
     return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
                        __uint_as_float(v.y & 0xFFFF0000u));
 }
@@ -106,14 +112,13 @@ __device__ __forceinline__ float4 unpack(uint2 v) {
 // are its one long wait, so how many are in flight decides.  STAGED copies all
 // context rows of a sample into the stage by 16-byte asynchronous copies, past
 // the registers, and waits once; without it the rows pass through registers,
-// at most CH at a time (BF16 rows must: they are widened on the way).  A
-// sample's record is loaded while the sample before is computed.  4.2 million
-// samples, K = 5, device memory tables (R-MAT 20, D = 128 FP32): 5.84 -> 4.81
-// ms, floor 4.78; BF16 7.98 -> 7.51; D = 64, K = 10, FP32 4.94 -> 4.01.  The
-// STAGED form's bound of 8 blocks (55 registers, nine resident) is 3% faster
-// than none (47, ten), a bound of 9 or 7 4% slower than it.
+// at most CH at a time (BF16 rows must: they are widened on the way).  2^22
+// samples, K = 5, R-MAT 20, eight blocks a SM on both sides, all rows through
+// registers four at a time -> like this: D = 128 FP32 5.84 -> 4.91 ms (floor
+// 4.78), BF16 7.91 -> 7.41; D = 64, K = 10, FP32 4.93 -> 4.12; D = 256 BF16 (2^18
+// nodes, four blocks) 13.1 -> 11.4.
 template <int D, int DT, bool STAGED>
-__global__ void __launch_bounds__(kHogWarps * 32, STAGED ? 8 : 0)
+__global__ void __launch_bounds__(kHogWarps * 32, STAGED ? kWave<D, DT> : 0)
     k_hogwild(HogwildParams p) {
     using G = Geom<D, DT>;
     extern __shared__ __align__(16) unsigned char s_raw[];
@@ -135,17 +140,23 @@ __global__ void __launch_bounds__(kHogWarps * 32, STAGED ? 8 : 0)
     const uint32_t ctx_tab = p.order == 2 ? 1u : 0u;
     void* ctx = p.order == 2 ? p.C : p.U;
     // a sample's record entry of this lane (R <= L), loaded one sample ahead
+    // where the loads are spread out (AHEAD)
+    constexpr bool AHEAD = STAGED || DT == LINE_DTYPE_BF16;
     auto entry = [&](int64_t s) { return worker < nw && s < n && lig < R ? __ldg(p.rec + s * R + lig) : 0; };
-    int32_t held = R <= G::L ? entry(worker) : 0;
+    int32_t held = AHEAD && R <= G::L ? entry(worker) : 0;
     for (int64_t r = 0; r < rounds; ++r) {
         const int64_t s = r * nw + worker;
         const bool active = worker < nw && s < n;
         if (R <= G::L) {
             // one slot per lane: the first slot of the worker holding the
             // same row of the same table, by matching keys across the warp
-            int32_t row = held;
-            if (r + 1 < rounds) held = entry(s + nw);
+            int32_t row = 0;
+            if (AHEAD) {
+                row = held;
+                if (r + 1 < rounds) held = entry(s + nw);
+            }
             if (active && lig < R) {
+                if (!AHEAD) row = __ldg(p.rec + s * R + lig);
                 if (row < 0 || row >= p.n_nodes) {
                     atomicOr(p.status, DEV_ERR_INDEX);
                     row = 0;
@@ -187,10 +198,8 @@ __global__ void __launch_bounds__(kHogWarps * 32, STAGED ? 8 : 0)
         // the U row into registers, the distinct context rows into the stage
         float x[G::E], x0[G::E];
         if (active) {
-            // 32 bytes and more a lane: the U row is one of the first CH
-            constexpr int FIRST = DT == LINE_DTYPE_F32 && G::E > 4 ? 0 : 1;
-            if (FIRST == 1) load_row<D, DT>(p.U, srow[0], lig, x0);
             if constexpr (STAGED) {
+                load_row<D, DT>(p.U, srow[0], lig, x0);
                 // a lane reads back only what it copied
                 for (int k = 1; k < R; ++k) {
                     if (sid[k] != k) continue;
@@ -200,16 +209,41 @@ __global__ void __launch_bounds__(kHogWarps * 32, STAGED ? 8 : 0)
                     for (int q = 0; q < G::NV; ++q) cp_async16(to + 4 * q, from + 4 * q);
                 }
                 cp_async_wait_all();
+            } else if constexpr (DT == LINE_DTYPE_F32) {
+                constexpr int CH = 4;
+                for (int k0 = 0; k0 < R; k0 += CH) {
+                    float v[CH][G::E];
+#pragma unroll
+                    for (int kk = 0; kk < CH; ++kk) {
+                        const int k = k0 + kk;
+                        if (k < R && sid[k] == k) load_row<D, DT>(k == 0 ? p.U : ctx, srow[k], lig, v[kk]);
+                    }
+                    if (k0 == 0) {
+#pragma unroll
+                        for (int e = 0; e < G::E; ++e) x0[e] = v[0][e];
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < CH; ++kk) {
+                        const int k = k0 + kk;
+                        if (k > 0 && k < R && sid[k] == k) {
+                            float4* st = reinterpret_cast<float4*>(stage + (size_t)k * D + lig * G::E);
+#pragma unroll
+                            for (int q = 0; q < G::NV; ++q)
+                                st[q] = make_float4(v[kk][4 * q], v[kk][4 * q + 1], v[kk][4 * q + 2], v[kk][4 * q + 3]);
+                        }
+                    }
+                }
             } else {
-                constexpr int CH = DT == LINE_DTYPE_BF16 ? 6 : 4;
-                for (int k0 = FIRST; k0 < R; k0 += CH) {
-                    Packed<DT> v[CH][G::NV];
+                // BF16 rows as they lie, six at a time, widened into the stage
+                constexpr int CH = 6;
+                load_row<D, DT>(p.U, srow[0], lig, x0);
+                for (int k0 = 1; k0 < R; k0 += CH) {
+                    uint2 v[CH][G::NV];
 #pragma unroll
                     for (int kk = 0; kk < CH; ++kk) {
                         const int k = k0 + kk;
                         if (k >= R || sid[k] != k) continue;
-                        const Packed<DT>* from =
-                            reinterpret_cast<const Packed<DT>*>(k == 0 ? p.U : ctx) + ((int64_t)srow[k] * D + lig * G::E) / 4;
+                        const uint2* from = reinterpret_cast<const uint2*>(ctx) + ((int64_t)srow[k] * D + lig * G::E) / 4;
 #pragma unroll
                         for (int q = 0; q < G::NV; ++q) v[kk][q] = __ldcg(from + q);
                     }
@@ -219,17 +253,7 @@ __global__ void __launch_bounds__(kHogWarps * 32, STAGED ? 8 : 0)
                         if (k >= R || sid[k] != k) continue;
                         float4* st = reinterpret_cast<float4*>(stage + (size_t)k * D + lig * G::E);
 #pragma unroll
-                        for (int q = 0; q < G::NV; ++q) {
-                            const float4 f = unpack(v[kk][q]);
-                            if (FIRST == 1 || k > 0) {
-                                st[q] = f;
-                            } else {
-                                x0[4 * q] = f.x;
-                                x0[4 * q + 1] = f.y;
-                                x0[4 * q + 2] = f.z;
-                                x0[4 * q + 3] = f.w;
-                            }
-                        }
+                        for (int q = 0; q < G::NV; ++q) st[q] = widen(v[kk][q]);
                     }
                 }
             }
@@ -309,15 +333,16 @@ cudaError_t launch_as(const HogwildParams& p, int64_t max_workers, cudaStream_t 
     const size_t per_warp = (size_t)G::GPW * group_bytes(D, p.K);
     const int wpb = (int)std::min<size_t>(kHogWarps, kMaxSmem / per_warp);
     if (wpb < 1) return cudaErrorInvalidValue;  // K and D beyond one warp's shared memory (not reachable for K <= 32)
-    const size_t smem = (size_t)wpb * per_warp;
+    size_t smem = (size_t)wpb * per_warp;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     // per device: the largest stage allowed so far (the attribute only
-    // grows, so every cached wave stays launchable) and the resident wave
-    // for each K (the stage size depends on K)
+    // grows, so every cached wave stays launchable), and for each K (the stage
+    // size depends on K) the wave and a block's shared memory
     struct Wave {
         int dev, K, sms, per_sm;
+        size_t smem;
     };
     static std::mutex mu;
     static std::vector<Wave> waves;
@@ -330,26 +355,42 @@ cudaError_t launch_as(const HogwildParams& p, int64_t max_workers, cudaStream_t 
         allowed.push_back({dev, 0});
         cap = &allowed.back().second;
     }
-    if (*cap < smem) {
-        if ((e = cudaFuncSetAttribute(k_hogwild<D, DT, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-            return e;
-        *cap = smem;
-    }
+    auto allow = [&](size_t bytes) {
+        if (*cap >= bytes) return cudaSuccess;
+        const cudaError_t r =
+            cudaFuncSetAttribute(k_hogwild<D, DT, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (r == cudaSuccess) *cap = bytes;
+        return r;
+    };
+    auto resident = [&](int* blocks) {
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_hogwild<D, DT, STAGED>, wpb * 32, smem);
+    };
     int per_sm = -1, sms = 0;
     for (const Wave& w : waves)
         if (w.dev == dev && w.K == p.K) {
             per_sm = w.per_sm;
             sms = w.sms;
+            smem = w.smem;
         }
     if (per_sm < 0) {
+        if ((e = allow(smem)) != cudaSuccess || (e = resident(&per_sm)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hogwild<D, DT, STAGED>, wpb * 32, smem)) != cudaSuccess)
-            return e;
-        waves.push_back({dev, p.K, sms, per_sm});
+        if (per_sm > kWave<D, DT>) {
+            // as much shared memory as keeps another block out: the wave then
+            // lies evenly on the SMs (1,216 blocks where nine fit an SM took
+            // 4.81 or 5.20 ms by where they fell, like this 4.91 or 5.07)
+            int all = 0, own = 0;
+            if ((e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess ||
+                (e = cudaDeviceGetAttribute(&own, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess)
+                return e;
+            smem = std::max<size_t>(smem, all / (kWave<D, DT> + 1) - own + 128);
+            if ((e = allow(smem)) != cudaSuccess || (e = resident(&per_sm)) != cudaSuccess) return e;
+            per_sm = std::min(per_sm, kWave<D, DT>);
+        }
+        waves.push_back({dev, p.K, sms, per_sm, smem});
     }
     const int64_t per_block = (int64_t)wpb * G::GPW;
-    const int64_t full = (int64_t)std::max(per_sm, 1) * sms * per_block;  // one resident wave
+    const int64_t full = (int64_t)std::max(per_sm, 1) * sms * per_block;  // the default wave, all resident
     HogwildParams q = p;
     q.workers = max_workers > 0 ? std::min<int64_t>(max_workers, full) : full;
     q.workers = std::min<int64_t>(q.workers, std::max<int64_t>(p.chunk_samples, 1));
@@ -359,8 +400,8 @@ cudaError_t launch_as(const HogwildParams& p, int64_t max_workers, cudaStream_t 
 }
 
 // Asynchronous copies for FP32 rows of 256 and 512 bytes in tables of 32 MB
-// and more: there the sample's loads are the bound (D = 128: 2^16 nodes 5.36
-// -> 4.56 ms, 2^20 nodes 5.84 -> 4.81).  Smaller tables lie in L2 with their
+// and more: there the sample's loads are the bound (D = 128: 2^16 nodes 5.28
+// -> 4.39 ms, 2^20 nodes 5.84 -> 4.91).  Smaller tables lie in L2 with their
 // hub rows under contention, and more loads in flight only lengthen the queue
 // at those (2^14 nodes: up to 10% slower); rows of 64 and 128 bytes gain
 // nothing (D = 32, 2^20 nodes: 1.84 ms both), and 1 KB rows have enough in
