@@ -79,11 +79,29 @@ __device__ __forceinline__ unsigned long long block_sum(unsigned long long v, un
     return v;
 }
 
+// row_ptr[v] = e for the nodes v in [v0, v1] between two arcs.  In an unsorted
+// graph every ascent begins such a run (2^22 random arcs over 2^20 nodes: 7e11
+// entries), so a long one ends once any thread has found the graph invalid.
+constexpr int64_t kFillShort = 32, kFillPiece = 1024;
+
+__device__ __forceinline__ void fill_offsets(int64_t* __restrict__ row_ptr, int64_t v0, int64_t v1, int64_t e,
+                                             const uint32_t* status) {
+    if (v1 - v0 < kFillShort) {
+        for (int64_t v = v0; v <= v1; ++v) row_ptr[v] = e;
+        return;
+    }
+    for (int64_t v = v0; v <= v1; v += kFillPiece) {
+        if (*(volatile const uint32_t*)status & DEV_ERR_GRAPH) return;
+        for (int64_t q = v, end = min(v1, v + kFillPiece - 1); q <= end; ++q) row_ptr[q] = e;
+    }
+}
+
 // One pass over the arcs: validation (DEV_ERR_GRAPH), the first arc of each
 // node (row_ptr, for a valid graph), whether every weight is an integer in
 // [1, 2^24], and - as if they were - their sum and each node's (degi, zero
 // before).  A thread takes kArcs consecutive arcs: a node's run inside them
-// is added with one atomic (src is sorted).
+// is added with one atomic (src is sorted).  A thread reports an invalid arc
+// before it writes any offset, and then writes none.
 // Bound: HBM (12 bytes an arc) and the run's branches: 185 us for 31.4M arcs;
 // the validation, the row offsets, the integer check and the node sums (a
 // warp a node) took 85 + 64 + 25 + 1,357 us as four kernels.
@@ -94,7 +112,7 @@ __global__ void __launch_bounds__(256) k_graph_scan(int64_t n_nodes, int64_t n_a
                                                     int64_t* __restrict__ row_ptr, unsigned long long* __restrict__ degi,
                                                     GraphScan* __restrict__ out, uint32_t* status) {
     __shared__ unsigned long long part[8];
-    bool bad = false, frac = false;
+    bool frac = false;
     unsigned long long total = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * kArcs;
     for (int64_t e0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * kArcs; e0 < n_arcs; e0 += stride) {
@@ -119,32 +137,38 @@ __global__ void __launch_bounds__(256) k_graph_scan(int64_t n_nodes, int64_t n_a
             }
         }
         int32_t prev = e0 > 0 ? src[e0 - 1] : -1;
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < kArcs; ++k) {
+            if (k >= cnt) continue;
+            ok = ok && s[k] >= 0 && s[k] < n_nodes && s[k] >= (k > 0 ? s[k - 1] : prev) && d[k] >= 0 && d[k] < n_nodes &&
+                 x[k] > 0.0f && isfinite(x[k]);
+        }
+        if (!ok || prev < -1) {
+            if (!(*(volatile const uint32_t*)status & DEV_ERR_GRAPH)) atomicOr(status, DEV_ERR_GRAPH);
+            continue;
+        }
         unsigned long long run = 0;
 #pragma unroll
         for (int k = 0; k < kArcs; ++k) {
             if (k < cnt) {
-                const bool ok = s[k] >= 0 && s[k] < n_nodes && s[k] >= prev && d[k] >= 0 && d[k] < n_nodes;
-                bad |= !ok || !(x[k] > 0.0f) || !isfinite(x[k]);
                 const bool whole = x[k] >= 1.0f && x[k] <= 16777216.0f && x[k] == truncf(x[k]);
                 frac |= !whole;
                 const uint32_t xi = whole ? __float2uint_rz(x[k]) : 0u;
                 total += xi;
                 if (s[k] != prev) {
-                    if (k > 0 && run && prev >= 0 && prev < n_nodes) atomicAdd(degi + prev, run);
+                    if (run) atomicAdd(degi + prev, run);
                     run = 0;
-                    if (ok && prev >= -1)
-                        for (int64_t v = (int64_t)prev + 1; v <= s[k]; ++v) row_ptr[v] = e0 + k;
+                    fill_offsets(row_ptr, (int64_t)prev + 1, s[k], e0 + k, status);
                 }
                 run += xi;
                 prev = s[k];
             }
         }
-        if (run && prev >= 0 && prev < n_nodes) atomicAdd(degi + prev, run);
+        if (run) atomicAdd(degi + prev, run);
         // the nodes after the last arc's
-        if (e0 + cnt == n_arcs && prev >= 0 && prev < n_nodes)
-            for (int64_t v = (int64_t)prev + 1; v <= n_nodes; ++v) row_ptr[v] = n_arcs;
+        if (e0 + cnt == n_arcs) fill_offsets(row_ptr, (int64_t)prev + 1, n_nodes, n_arcs, status);
     }
-    if (bad) atomicOr(status, DEV_ERR_GRAPH);
     if (frac) out->frac = 1u;
     total = block_sum(total, part);
     if (threadIdx.x == 0 && total) atomicAdd(&out->sum, total);
