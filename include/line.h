@@ -324,9 +324,10 @@ LINE_API line_status line_set_embeddings(line_ctx* ctx, int order, int which, co
 
 /* Negative-sampling LINE loss over the first m samples of draw domain 3:
  * L = -sum_t [log sigma(s+) + sum_j log sigma(-s-_j)], s = U[u].Ctx[y]
- * computed from the stored values to FP64 accuracy (a dot loses only bits
- * below 2^-58 of its largest product, then rounds once), summed in FP64 in a
- * fixed order.  Result in *out_host (host pointer). */
+ * computed from the stored values to FP64 accuracy (a dot is off by at most
+ * 2^-56, 2^-55, 2^-54, 2^-52 and 2^-51 of its largest product at dim 16, 32,
+ * 64, 128 and 256, then rounds once; rows with subnormal, infinite or NaN
+ * values are summed in FP64), summed in FP64 in a fixed order.  Result in *out_host (host pointer). */
 LINE_API line_status line_eval_loss(line_ctx* ctx, int order, int K, uint64_t seed, int64_t m, double* out_host);
 
 /* Link-prediction AUC: held-out edges against non-edges (the paper's own

@@ -1,6 +1,7 @@
 // Negative-sampling LINE loss over a fixed set of samples (draw domain 3):
-// terms[t] = -(log sigma(s+) + sum_j log sigma(-s-_j)), s = U[u].Ctx[y] in
-// FP64 from the stored values.  The caller reduces terms[] with the
+// terms[t] = -(log sigma(s+) + sum_j log sigma(-s-_j)), s = U[u].Ctx[y] from
+// the stored values, summed in 64-bit integers (FP64 where that would be less
+// exact) and rounded to FP64.  The caller reduces terms[] with the
 // fixed-order FP64 sum, so the loss is reproducible.
 #include <math.h>
 
@@ -57,45 +58,58 @@ __device__ __forceinline__ void load_bits(const void* p, int64_t idx, uint32_t (
 
 // A dot of FP32 rows in integers, IT products a lane: the 48-bit products of
 // the significands, SH bits above their last one, each shifted down by its
-// exponent's distance to the largest product's and summed exactly.  What is
-// lost are bits below 2^-(46 + SH) of the largest product (where a factor of
-// it is subnormal, of 2^-126 times the other), fewer than FP64 sums lose:
-// against the exact dot over rows of normal, positive, widely spread,
-// subnormal and trained values and of one product above all others, the rms
-// and the largest error are below the FP64 chain's, by 2 to 20 times at
-// d >= 64 for rows whose sum cancels, by 1.1 to 3 times for the others.
+// exponent's distance to the largest exponent's, to nearest, and summed
+// exactly.  A product is off by at most half a unit of 2^-(46 + SH) of the one
+// with the largest exponent, the dot by half of D units: 2^-56, 2^-55, 2^-54,
+// 2^-52 and 2^-51 of it for D = 16, 32, 64, 128 and 256.  Against the exact
+// dot over rows of normal, positive, widely spread and trained values and of
+// one product above all others, 2^9 to 2^62 times, the rms and the largest
+// error are below the FP64 chain's at every width, by 2 to 20 times at D >= 64
+// for rows whose sum cancels, by 1 to 4 times for the others.  (Rounded down,
+// the small products beside one large one all counted on one side: 2^-52 of it
+// at D = 128, where the chain was exact.)  A subnormal factor has no leading
+// bit, and its product would be held to fewer: such rows take FP64 sums.
 template <int IT>
 struct Fixed {
-    static constexpr int LOG = IT == 1 ? 0 : IT == 2 ? 1 : IT == 4 ? 2 : 3;
-    static constexpr int SH = IT == 1 ? 14 : 15 - LOG;  // a lane's sum stays below 2^63, each factor below 2^31
+    // a lane's sum (of twice the products up to IT = 4) stays below 2^63, each
+    // factor below 2^31
+    static constexpr int SH = IT <= 2 ? 13 : 12;
     static constexpr int CUT = 27;       // limbs of the sum over 32 lanes: 32 2^27 fits 32 bits
 
     // This lane's part of a dot; `top`: the largest product's exponent (of all
-    // lanes; twice biased, in place); `big`: |= an infinity or a NaN was met.
-    static __device__ __forceinline__ int64_t lane_sum(const uint32_t (&a)[IT], const uint32_t (&b)[IT], uint32_t& top, bool& big) {
+    // lanes; twice biased, in place); `wide`: |= an infinity, a NaN or a
+    // subnormal value was met.
+    static __device__ __forceinline__ int64_t lane_sum(const uint32_t (&a)[IT], const uint32_t (&b)[IT], uint32_t& top, bool& wide) {
         int64_t p[IT];
-        uint32_t ex[IT], m = 0, mx = 0;
+        uint32_t ex[IT], m = 0, mx = 0, mn = 0xFFFFFFFFu;
 #pragma unroll
         for (int k = 0; k < IT; ++k) {
             const uint32_t ea = a[k] & 0x7F800000u, eb = b[k] & 0x7F800000u;
             mx = max(mx, max(ea, eb));
-            // subnormals: no leading bit, the smallest exponent
+            // (0 for a zero, below 2^23 for a subnormal)
             const uint32_t sa = (a[k] & 0x7FFFFFu) | min(ea, 0x800000u), sb = (b[k] & 0x7FFFFFu) | min(eb, 0x800000u);
-            const int32_t sg = (int32_t)(a[k] ^ b[k]) < 0 ? -(1 << (SH - 7)) : 1 << (SH - 7);
+            mn = min(mn, min(sa - 1u, sb - 1u));
+            constexpr int UP = SH - 7 + (IT <= 4);
+            const int32_t sg = (int32_t)(a[k] ^ b[k]) < 0 ? -(1 << UP) : 1 << UP;
             p[k] = (int64_t)(int32_t)(sa << 7) * ((int32_t)sb * sg);
-            ex[k] = p[k] ? max(ea, 0x800000u) + max(eb, 0x800000u) : 0u;
+            ex[k] = p[k] ? ea + eb : 0u;
             m = max(m, ex[k]);
         }
-        big |= mx >= 0x7F800000u;
+        wide |= mx >= 0x7F800000u || mn < 0x7FFFFFu;
         top = __reduce_max_sync(0xFFFFFFFFu, m);
         int64_t sum = 0;
 #pragma unroll
         for (int k = 0; k < IT; ++k) {
             const uint32_t s = min((top - ex[k]) >> 23, 63u);
-            // eight products a lane leave fewer bits below: to nearest
-            sum += (p[k] + (IT > 4 ? (int64_t)((uint64_t)1 << s >> 1) : 0)) >> s;
+            if constexpr (IT <= 4) {
+                // twice the product, rounded down: t; to nearest it is (t + (t & 1)) / 2
+                const int64_t t = p[k] >> s;
+                sum += t + (t & 1);
+            } else {
+                sum += (p[k] + (int64_t)((uint64_t)1 << s >> 1)) >> s;
+            }
         }
-        return sum;
+        return IT <= 4 ? sum >> 1 : sum;
     }
     // The dot from the limbs' sums over the lanes.
     static __device__ __forceinline__ double value(int64_t h, uint32_t lo, uint32_t top) {
@@ -110,14 +124,16 @@ struct Fixed {
 // values a lane, in integers (Fixed); their limbs are reduced by transposed
 // butterflies (each total in some lanes only); then every lane evaluates the
 // log-sigmoid of its own score, and a sample's are subtracted in order.  Rows
-// with infinities or NaNs take FP64 sums, value k of a row in lane k mod 32.
-// Bound: issue slots of the integer dots (about 30 instructions a product) and
+// with infinities, NaNs or subnormals take FP64 sums, value k of a row in lane
+// k mod 32.
+// Bound: issue slots of the integer dots (about 33 instructions a product) and
 // GB300's FP64 pipe in the log-sigmoids (two lanes a clock and SM, also for
 // conversions).  N = 3 at 64 registers keeps four blocks resident (8 at 117
 // registers: 1.85 ms, 4: 1.48).
 // One warp per sample, with all lanes on the same log-sigmoid and FP64
 // conversions of every value, took 25.2 ms for 2^20 samples of K = 5, d = 128
-// FP32; FP64 sums of values widened by integer instructions 2.77; this 1.40.
+// FP32; FP64 sums of values widened by integer instructions 2.77; this 1.52
+// (1.40 without the rounding and the look for subnormals).
 template <int D, int DT>
 __global__ void __launch_bounds__(256, 4) k_loss_terms(const void* __restrict__ U, const void* __restrict__ Ctx, int K,
                                                     const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
@@ -172,14 +188,14 @@ __global__ void __launch_bounds__(256, 4) k_loss_terms(const void* __restrict__ 
                         for (int k = 0; k < IT; ++k) a[i][k] = c[i][k] = 0u;
                     }
                 }
-                bool big = false;
+                bool wide = false;
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
-                    const int64_t sum = F::lane_sum(a[i], c[i], tops[i], big);
+                    const int64_t sum = F::lane_sum(a[i], c[i], tops[i], wide);
                     low[i] = (uint32_t)sum & ((1u << F::CUT) - 1u);
                     part[i] = sum >> F::CUT;
                 }
-                if (__any_sync(0xFFFFFFFFu, big)) {
+                if (__any_sync(0xFFFFFFFFu, wide)) {
 #pragma unroll 1
                     for (int i = 0; i < N; ++i) {
                         const int q = min(q0 + i, nq - 1);
