@@ -568,11 +568,27 @@ constexpr int kGatherWarps = 4;
 
 
 // JB: context rows held in registers (K + 1 <= JB), or 0 for the staged body.
+// The next kernel may start at once, and its blocks then wait on the SMs.  At
+// D = 256 both kernels' blocks are small enough for those of the next two
+// batches to gather there too, which held up the running ones: FP32 batches of
+// up to 1,600 samples ran up to 25% longer than with larger blocks.  So at D =
+// 256, and with eight rows in registers, the gather lets the apply start after
+// its own wait, and at D = 256 the apply of an FP32 order that trains alone, with
+// batches of up to kLateItems entries, lets the next gather start likewise.
+// 2^18 samples of one order, FP32, D = 256, K = 3: R-MAT 16, B = 768 and 1,024
+// 2.65 and 2.39 ms with both starts at once, 1.86 and 1.64 like this; R-MAT 18,
+// K = 10, B = 1,024 and 1,500: 3.50 and 2.41, 2.71 and 2.34.  D = 128, K = 7, B =
+// 900: 1.77 and 1.62.  The apply's late start costs larger FP32 batches 2% (K =
+// 10, B = 2,048: 1.97 -> 2.02), BF16 ones up to 10% and two orders, which fill
+// the SMs for each other, up to 13%.
+constexpr int64_t kLateItems = 18432;
+
 template <int D, int DT, int JB>
 __global__ void __launch_bounds__(kGatherWarps * 32, 8) k_gather(DataParams p, int b) {
     using G = Geom<D, DT>;
     extern __shared__ float4 smem4[];
-    pdl_launch_dependents();
+    constexpr bool kLate = D > 128 || JB == 8;
+    if constexpr (!kLate) pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = lane / G::L, lig = lane % G::L;
     const int64_t s_begin = (int64_t)b * p.batch;
@@ -587,6 +603,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32, 8) k_gather(DataParams p, i
         Held<G::L, JB> h;
         h.load(p, s_local, lig, active);
         pdl_wait();  // the tables' rows: written by the previous kernel
+        if constexpr (kLate) pdl_launch_dependents();
         sample_body_reg<D, DT, JB>(p, lig, active, bp.eta, bp.salt, gm, h);
     } else {
         const int R = p.K + 2;
@@ -596,6 +613,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32, 8) k_gather(DataParams p, i
         const int32_t r0 = (active && lig < R) ? rec[lig] : 0;
         const uint32_t i0 = (active && lig < R) ? info[lig] : 0u;
         pdl_wait();
+        if constexpr (kLate) pdl_launch_dependents();
         unsigned char* stage = reinterpret_cast<unsigned char*>(smem4) +
                                (size_t)(warp * G::GPW + grp) * (p.K + 1) * D * (DT == LINE_DTYPE_F32 ? 4 : 2);
         sample_body_staged<D, DT>(p, lig, active, bp.eta, bp.salt, gm, r0, i0, rec, info, stage);
@@ -627,7 +645,9 @@ __global__ void __launch_bounds__(NW * 32, D <= 128 ? 32 / NW : 1) k_apply(DataP
     constexpr uint32_t NG = NW * G::GPW, kLogNG = NG == 8 ? 3 : NG == 16 ? 4 : NG == 32 ? 5 : NG == 64 ? 6 : 7;
     static_assert(NG == 1u << kLogNG, "a block's lane groups");
     __shared__ __align__(16) float part[NG * D];
-    pdl_launch_dependents();
+    // (see k_gather)
+    const bool late = D > 128 && DT == LINE_DTYPE_F32 && p.apply_warps == kApplyWarpsAlone && p.batch * (p.K + 2) <= kLateItems;
+    if (!late) pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = lane / G::L, lig = lane % G::L;
     const uint32_t g = (uint32_t)(warp * G::GPW + grp);
@@ -645,6 +665,7 @@ __global__ void __launch_bounds__(NW * 32, D <= 128 ? 32 / NW : 1) k_apply(DataP
     const uint32_t nsb = min(gridDim.x - kLongBlocks, (n0 + NG - 1) / NG);  // blocks with short segments
     if (blockIdx.x - kLongBlocks < nsb) {
         pdl_wait();  // the slab and the rows: written by the gather
+        if (late) pdl_launch_dependents();
         while (m < n0) {
             segment_item<D, DT>(p, d, lig, true, eta, salt);
             m += nsb * NG;
