@@ -170,6 +170,10 @@ LINE_API const char* line_status_string(line_status s);
  * context or NULL on failure.  No paper counterpart: the context holds what
  * one NOMAD process keeps in memory (its graph partition, distributions and
  * embedding rows, Algorithm 1's inputs), here for the whole graph on one GPU.
+ * line_eval_loss, line_eval_auc, and line_get_alias and line_mlp_predict to
+ * host memory keep up to 256 MB of device scratch in the context for the next
+ * such call (more is allocated for the call alone); it is given back when
+ * another allocation of the context has no room, and by line_destroy.
  * Errors: LINE_ERR_ARG (no such device, out NULL), LINE_ERR_CUDA. */
 LINE_API line_status line_create(line_ctx** out, int device, void* cuda_stream);
 LINE_API void line_destroy(line_ctx* ctx);
@@ -350,8 +354,7 @@ LINE_API line_status line_eval_loss(line_ctx* ctx, int order, int K, uint64_t se
  * Errors: LINE_ERR_ARG (bad mask or score, counts, null pointers, or a node
  * id out of range), LINE_ERR_STATE (a requested order has no tables),
  * LINE_ERR_VALIDATE (a score is NaN: non-finite table values), LINE_ERR_OOM,
- * LINE_ERR_CUDA.  Keeps up to 256 MB of scratch for the pairs until
- * line_destroy (more is allocated for the call); synchronises. */
+ * LINE_ERR_CUDA.  Synchronises; scratch for the pairs is kept (line_create). */
 LINE_API line_status line_eval_auc(line_ctx* ctx, int orders, int score, const int32_t* pos_src, const int32_t* pos_dst,
                                    int64_t n_pos, const int32_t* neg_src, const int32_t* neg_dst, int64_t n_neg,
                                    float* scores_out, uint64_t* counts_out, double* auc_out);

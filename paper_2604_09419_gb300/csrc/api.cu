@@ -67,7 +67,7 @@ bool on_device(const line_ctx* c, const void* p) {
 
 line_status ensure_walk_tables(line_ctx* c) {
     if (c->cw_ok) return LINE_OK;
-    cudaError_t e = grow(&c->cw, &c->cw_cap, sizeof(double) * (size_t)std::max<int64_t>(1, c->n_arcs));
+    cudaError_t e = grow(c, &c->cw, &c->cw_cap, sizeof(double) * (size_t)std::max<int64_t>(1, c->n_arcs));
     if (e == cudaSuccess) e = walk_cumw(c->n_nodes, c->row_ptr, c->w, c->whole, c->cw, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "walk sampler tables");
     c->cw_ok = true;
@@ -195,7 +195,7 @@ void line_destroy(line_ctx* c) {
     if (c->side) cudaStreamDestroy(c->side);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
-    if (c->scratch) cudaFree(c->scratch);
+    if (c->scratch.p) cudaFree(c->scratch.p);
     if (c->status) cudaFree(c->status);
     if (c->dscratch) cudaFree(c->dscratch);
     if (c->ev0) cudaEventDestroy(c->ev0);
@@ -221,11 +221,11 @@ line_status line_build_alias(line_ctx* c, const line_graph_desc* g) {
     // the buffers of an earlier graph are reused when large enough; the
     // work queued on the stream before this call may still read them, and
     // the stream orders it before the copies below
-    CK(grow(&c->src, &c->src_cap, sizeof(int32_t) * m), "graph allocation");
-    CK(grow(&c->dst, &c->dst_cap, sizeof(int32_t) * m), "graph allocation");
-    CK(grow(&c->edge_tab, &c->edge_cap, sizeof(uint2) * m), "alias allocation");
-    CK(grow(&c->neg_tab, &c->neg_cap, sizeof(uint2) * n), "alias allocation");
-    CK(grow(&c->deg, &c->deg_cap, sizeof(float) * n), "degree allocation");
+    CK(grow(c, &c->src, &c->src_cap, sizeof(int32_t) * m), "graph allocation");
+    CK(grow(c, &c->dst, &c->dst_cap, sizeof(int32_t) * m), "graph allocation");
+    CK(grow(c, &c->edge_tab, &c->edge_cap, sizeof(uint2) * m), "alias allocation");
+    CK(grow(c, &c->neg_tab, &c->neg_cap, sizeof(uint2) * n), "alias allocation");
+    CK(grow(c, &c->deg, &c->deg_cap, sizeof(float) * n), "degree allocation");
     CK(cudaMemcpyAsync(c->src, g->src, sizeof(int32_t) * m, cudaMemcpyDefault, s), "graph copy");
     CK(cudaMemcpyAsync(c->dst, g->dst, sizeof(int32_t) * m, cudaMemcpyDefault, s), "graph copy");
     float* w = nullptr;
@@ -233,7 +233,7 @@ line_status line_build_alias(line_ctx* c, const line_graph_desc* g) {
     do {
         cudaError_t e;
         if (g->w) {
-            if ((e = grow(&c->w_buf, &c->w_cap, sizeof(float) * m)) != cudaSuccess) { result = cuda_fail(c, e, "weights"); break; }
+            if ((e = grow(c, &c->w_buf, &c->w_cap, sizeof(float) * m)) != cudaSuccess) { result = cuda_fail(c, e, "weights"); break; }
             w = c->w_buf;
             if ((e = cudaMemcpyAsync(w, g->w, sizeof(float) * m, cudaMemcpyDefault, s)) != cudaSuccess) {
                 result = cuda_fail(c, e, "weights copy");
@@ -243,9 +243,9 @@ line_status line_build_alias(line_ctx* c, const line_graph_desc* g) {
         // one pass over the arcs: validation, the row offsets (kept for the
         // walk sampler and the MLP inputs), and the weights' integer sums
         const int64_t big = n > m ? n : m;
-        if ((e = grow(&c->row_ptr, &c->row_ptr_cap, sizeof(int64_t) * (size_t)(n + 1))) != cudaSuccess) { result = cuda_fail(c, e, "row offsets"); break; }
-        if ((e = grow(&c->alias_x, &c->x_cap, sizeof(double) * 2 * n)) != cudaSuccess) { result = cuda_fail(c, e, "alias scratch"); break; }
-        if ((e = grow(&c->alias_tmp, &c->tmp_cap, alias_build_tmp_bytes(big))) != cudaSuccess) { result = cuda_fail(c, e, "alias scratch"); break; }
+        if ((e = grow(c, &c->row_ptr, &c->row_ptr_cap, sizeof(int64_t) * (size_t)(n + 1))) != cudaSuccess) { result = cuda_fail(c, e, "row offsets"); break; }
+        if ((e = grow(c, &c->alias_x, &c->x_cap, sizeof(double) * 2 * n)) != cudaSuccess) { result = cuda_fail(c, e, "alias scratch"); break; }
+        if ((e = grow(c, &c->alias_tmp, &c->tmp_cap, alias_build_tmp_bytes(big))) != cudaSuccess) { result = cuda_fail(c, e, "alias scratch"); break; }
         double* x = c->alias_x;
         unsigned long long* degi = reinterpret_cast<unsigned long long*>(x + n);
         void* tmp = c->alias_tmp;
@@ -327,7 +327,7 @@ line_status line_sample_debug(line_ctx* c, int K, uint64_t seed, uint32_t domain
     cudaPointerAttributes attr;
     bool dev_out = cudaPointerGetAttributes(&attr, out) == cudaSuccess && attr.type == cudaMemoryTypeDevice;
     cudaGetLastError();
-    if (!dev_out) CK(cudaMalloc(&buf, bytes), "sample scratch");
+    if (!dev_out) CK(device_alloc(&buf, bytes, &c->scratch), "sample scratch");
     cudaError_t e = sample_records(c->src, c->dst, c->edge_tab, c->n_arcs, c->neg_tab, c->n_nodes, seed, domain, t0,
                                    count, K, dev_out ? out : buf, c->stream);
     if (e == cudaSuccess && !dev_out) e = cudaMemcpyAsync(out, buf, bytes, cudaMemcpyDefault, c->stream);
@@ -356,7 +356,7 @@ line_status line_sample_walk_debug(line_ctx* c, int K, uint64_t seed, int walk_l
     cudaPointerAttributes attr;
     bool dev_out = cudaPointerGetAttributes(&attr, out) == cudaSuccess && attr.type == cudaMemoryTypeDevice;
     cudaGetLastError();
-    if (!dev_out) CK(cudaMalloc(&buf, bytes), "sample scratch");
+    if (!dev_out) CK(device_alloc(&buf, bytes, &c->scratch), "sample scratch");
     int32_t* rec = dev_out ? out : buf;
     // negatives: the edge sampler's draws (domain 0, calls 1..K); its slots 0
     // and 1 are then overwritten by the walk pairs
@@ -399,9 +399,9 @@ line_status line_init_embeddings(line_ctx* c, int order, int dim, int dtype, uin
     t.ready = false;
     // the tables' earlier allocations are reused when they are large enough
     const size_t bytes = (size_t)c->n_nodes * dim * elem_size(dtype);
-    cudaError_t e = grow(&t.U, &t.u_cap, bytes);
+    cudaError_t e = grow(c, &t.U, &t.u_cap, bytes);
     if (e == cudaSuccess) e = init_table(t.U, dtype, c->n_nodes, dim, seed, c->stream);
-    if (e == cudaSuccess && order == 2) e = grow(&t.C, &t.c_cap, bytes);
+    if (e == cudaSuccess && order == 2) e = grow(c, &t.C, &t.c_cap, bytes);
     if (e == cudaSuccess && order == 2) e = cudaMemsetAsync(t.C, 0, bytes, c->stream);
     if (e != cudaSuccess) {
         free_tables(t);  // nothing of a failed call is kept
@@ -482,6 +482,7 @@ line_status make_train_args(line_ctx* c, const char* what, int order, int dim, i
     a.row_ptr = o.walk_length > 0 ? c->row_ptr : nullptr;
     a.cw = o.walk_length > 0 ? c->cw : nullptr;
     a.graph = o.graph;
+    a.kept = &c->scratch;
     *out = a;
     return LINE_OK;
 }
@@ -601,7 +602,7 @@ line_status line_get_embeddings(line_ctx* c, int order, int which, void* dst, in
         CK(cudaMemcpyAsync(dst, srcp, elems * elem_size(t.dtype), cudaMemcpyDefault, c->stream), "embedding copy");
     } else {
         void* buf = nullptr;
-        CK(cudaMalloc(&buf, elems * 4), "conversion scratch");
+        CK(device_alloc(&buf, elems * 4, &c->scratch), "conversion scratch");
         cudaError_t e = convert_rows(srcp, t.dtype, buf, LINE_DTYPE_F32, nullptr, c->n_nodes, t.dim, c->n_nodes,
                                      c->status, c->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dst, buf, elems * 4, cudaMemcpyDefault, c->stream);
@@ -630,8 +631,8 @@ line_status line_set_embeddings(line_ctx* c, int order, int which, const void* s
     const size_t in_bytes = (size_t)n_rows * t.dim * elem_size(src_dtype);
     void* sbuf = nullptr;
     int32_t* rbuf = nullptr;
-    cudaError_t e = cudaMalloc(&sbuf, in_bytes);
-    if (e == cudaSuccess && rows) e = cudaMalloc(&rbuf, sizeof(int32_t) * n_rows);
+    cudaError_t e = device_alloc(&sbuf, in_bytes, &c->scratch);
+    if (e == cudaSuccess && rows) e = device_alloc(&rbuf, sizeof(int32_t) * n_rows, &c->scratch);
     if (e == cudaSuccess) e = cudaMemcpyAsync(sbuf, src, in_bytes, cudaMemcpyDefault, c->stream);
     if (e == cudaSuccess && rows) e = cudaMemcpyAsync(rbuf, rows, sizeof(int32_t) * n_rows, cudaMemcpyDefault, c->stream);
     if (e == cudaSuccess)

@@ -56,9 +56,8 @@ struct line_ctx {
     void* alias_tmp = nullptr;
     // tables by order (index 1 and 2)
     line::Tables tab[3];
-    // scratch of the synchronous evaluation calls (take_scratch)
-    void* scratch = nullptr;
-    size_t scratch_cap = 0;
+    // scratch of the synchronous calls (Scratch)
+    line::DeviceScratch scratch;
     // device status word and small scratch
     uint32_t* status = nullptr;
     uint32_t* flag = nullptr;
@@ -91,33 +90,35 @@ line_status ensure_walk_tables(line_ctx* c);
 
 // *p holds at least `bytes` (a larger earlier allocation is kept).
 template <typename T>
-cudaError_t grow(T** p, size_t* cap, size_t bytes) {
+cudaError_t grow(line_ctx* c, T** p, size_t* cap, size_t bytes) {
     if (*p && *cap >= bytes) return cudaSuccess;
     if (*p) cudaFree(*p);
     *p = nullptr;
     *cap = 0;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    cudaError_t e = device_alloc(p, bytes, &c->scratch);
     if (e == cudaSuccess) *cap = bytes;
     return e;
 }
 
 // Scratch for one synchronous call: up to kKeptScratch bytes from the
-// context's buffer (grown, kept for later calls, freed by line_destroy: a
-// cudaMalloc and cudaFree per call cost 100-200 us), more from an allocation
-// of the call's own.
+// context's buffer (grown, kept for later calls - a cudaMalloc and cudaFree per
+// call cost 100-200 us - until another allocation has no room or line_destroy),
+// more from an allocation of the call's own.
 constexpr size_t kKeptScratch = (size_t)256 << 20;
 struct Scratch {
     void* p = nullptr;
-    bool own = false;
+    DeviceScratch* from = nullptr;  // null: an allocation of the call's own
     cudaError_t take(line_ctx* c, size_t bytes) {
-        own = bytes > kKeptScratch;
-        if (own) return cudaMalloc(&p, bytes);
-        cudaError_t e = grow(&c->scratch, &c->scratch_cap, bytes);
-        p = c->scratch;
+        if (bytes > kKeptScratch) return device_alloc(&p, bytes, &c->scratch);
+        from = &c->scratch;
+        const cudaError_t e = grow(c, &from->p, &from->bytes, bytes);
+        from->busy = e == cudaSuccess;
+        p = from->p;
         return e;
     }
     ~Scratch() {
-        if (own && p) cudaFree(p);
+        if (from) from->busy = false;
+        else if (p) cudaFree(p);
     }
 };
 inline size_t round256(size_t v) { return (v + 255) & ~(size_t)255; }

@@ -134,10 +134,24 @@ __device__ __forceinline__ uint32_t bf16x2_sr(float lo, float hi, uint32_t r) {
 // ---------------------------------------------------------------------------
 // Launchers (defined in the .cu files).  All enqueue on `s`.
 // ---------------------------------------------------------------------------
+// Device memory that synchronous calls use and keep for the next one (busy: by
+// the call that runs now).
 struct DeviceScratch {
     void* p = nullptr;
     size_t bytes = 0;
+    bool busy = false;
 };
+
+// cudaMalloc; where the device has no room, `kept` is given back first.
+template <typename T>
+cudaError_t device_alloc(T** p, size_t bytes, DeviceScratch* kept) {
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e != cudaErrorMemoryAllocation || !kept->p || kept->busy) return e;
+    cudaGetLastError();
+    cudaFree(kept->p);  // (waits for the work that was queued on it)
+    *kept = DeviceScratch{};
+    return cudaMalloc(reinterpret_cast<void**>(p), bytes);
+}
 
 // alias.cu
 // Block of the fixed-order FP64 sum: blocks of kSumBlock values are each
@@ -282,6 +296,7 @@ struct TrainArgs {
     int walk_len, window, walk_reuse;
     int64_t hogwild_workers;  // LINE_MODE_HOGWILD: concurrent workers (0: one resident wave)
     bool concurrent;          // another order trains at the same time (line_train_orders)
+    DeviceScratch* kept;      // given back if the call's own scratch does not fit
 };
 
 struct TrainTimes {

@@ -39,6 +39,7 @@ constexpr int64_t kMlpMaxBatch = 1 << 16;
 
 struct MlpState {
     int order = 0, dim = 0, hidden = 0, P = 0, act = 0;
+    DeviceScratch* kept = nullptr;  // the context's, given back if an allocation here does not fit
     int64_t n_params = 0;
     float* params = nullptr;  // [W1 (hidden x P) | b1 (hidden) | W2 (dim x hidden) | b2 (dim)];
                               // grads, m and v follow in the same allocation
@@ -1197,7 +1198,7 @@ cudaError_t ensure_weight_tiles(MlpState& s) {
     if (s.wt) cudaFree(s.wt);
     s.wt = nullptr;
     s.wt_elems = 0;
-    cudaError_t e = cudaMalloc(&s.wt, sizeof(float) * need);
+    cudaError_t e = device_alloc(&s.wt, sizeof(float) * need, s.kept);
     if (e == cudaSuccess) s.wt_elems = need;
     return e;
 }
@@ -1215,7 +1216,7 @@ cudaError_t ensure_w16(MlpState& s) {
     if (s.w16) cudaFree(s.w16);
     s.w16 = nullptr;
     s.w16_elems = 0;
-    cudaError_t e = cudaMalloc(&s.w16, sizeof(__nv_bfloat16) * need);
+    cudaError_t e = device_alloc(&s.w16, sizeof(__nv_bfloat16) * need, s.kept);
     if (e == cudaSuccess) s.w16_elems = need;
     return e;
 }
@@ -1249,7 +1250,7 @@ cudaError_t ensure_cap(MlpState& s, int64_t rows) {
         total += (sizes[i] + 255) / 256 * 256;
     }
     void* arena = nullptr;
-    cudaError_t e = cudaMalloc(&arena, total);
+    cudaError_t e = device_alloc(&arena, total, s.kept);
     if (e != cudaSuccess) return e;
     unsigned char* b = reinterpret_cast<unsigned char*>(arena);
     s.arena = arena;
@@ -1458,7 +1459,7 @@ cudaError_t ensure_rowloss(MlpState& s, int64_t rows, int64_t B, cudaStream_t st
         if (s.rowloss) cudaFree(s.rowloss);
         s.rowloss = nullptr;
         s.rowloss_cap = 0;
-        const cudaError_t e = cudaMalloc(&s.rowloss, need);
+        const cudaError_t e = device_alloc(&s.rowloss, need, s.kept);
         if (e != cudaSuccess) return e;
         s.rowloss_cap = need;
     }
@@ -1497,7 +1498,7 @@ cudaError_t upload_nodes(MlpState& s, const int32_t* nodes, int64_t n, cudaStrea
         if (s.nodes) cudaFree(s.nodes);
         s.nodes = nullptr;
         s.nodes_cap = 0;
-        cudaError_t e = cudaMalloc(&s.nodes, sizeof(int32_t) * n);
+        cudaError_t e = device_alloc(&s.nodes, sizeof(int32_t) * n, s.kept);
         if (e != cudaSuccess) return e;
         s.nodes_cap = n;
     }
@@ -1530,6 +1531,7 @@ line_status line_mlp_create(line_ctx* c, int order, int hidden, int act_dtype, u
     } else {
         mlp_destroy(s);
         s = new MlpState();
+        s->kept = &c->scratch;
         s->order = order;
         s->dim = t.dim;
         s->hidden = hidden;
@@ -1540,14 +1542,14 @@ line_status line_mlp_create(line_ctx* c, int order, int hidden, int act_dtype, u
         s->n_params = L0.n;
         // params, grads, m and v in one allocation, each at a 256-byte boundary
         const size_t pbs = (sizeof(float) * L0.n + 255) / 256 * 256;
-        e = cudaMalloc(&s->params, 4 * pbs);
+        e = device_alloc(&s->params, 4 * pbs, s->kept);
         if (e == cudaSuccess) {
             unsigned char* b = reinterpret_cast<unsigned char*>(s->params);
             s->grads = reinterpret_cast<float*>(b + pbs);
             s->m = reinterpret_cast<float*>(b + 2 * pbs);
             s->v = reinterpret_cast<float*>(b + 3 * pbs);
         }
-        if (e == cudaSuccess) e = cudaMalloc(&s->X, (size_t)c->n_nodes * s->P * elem_size(act_dtype));
+        if (e == cudaSuccess) e = device_alloc(&s->X, (size_t)c->n_nodes * s->P * elem_size(act_dtype), s->kept);
     }
     const Layout L(*s);
     const size_t pb = sizeof(float) * L.n;
@@ -1585,21 +1587,21 @@ static line_status mlp_features_impl(line_ctx* c, const char* what, const uint8_
     // scratch kept in the MLP state (grown, never shrunk)
     const int64_t max_hubs = HubScratch(c->n_nodes, c->n_arcs).max_hubs;
     cudaError_t e = cudaSuccess;
-    if (!s.kmask) e = cudaMalloc(&s.kmask, (size_t)c->n_nodes);
-    if (e == cudaSuccess && !s.flag) e = cudaMalloc(&s.flag, sizeof(uint32_t));
+    if (!s.kmask) e = device_alloc(&s.kmask, (size_t)c->n_nodes, s.kept);
+    if (e == cudaSuccess && !s.flag) e = device_alloc(&s.flag, sizeof(uint32_t), s.kept);
     const HubScratch hs(c->n_nodes, c->n_arcs);
     const size_t hub_bytes = hs.bytes(s.dim);
     if (e == cudaSuccess && s.hubs_cap < (int64_t)hub_bytes) {
         if (s.hubs) cudaFree(s.hubs);
         s.hubs = nullptr;
         s.hubs_cap = 0;
-        if ((e = cudaMalloc(&s.hubs, hub_bytes)) == cudaSuccess) s.hubs_cap = (int64_t)hub_bytes;
+        if ((e = device_alloc(&s.hubs, hub_bytes, s.kept)) == cudaSuccess) s.hubs_cap = (int64_t)hub_bytes;
     }
     if (e == cudaSuccess && rows && s.frows_cap < n_rows) {
         if (s.frows) cudaFree(s.frows);
         s.frows = nullptr;
         s.frows_cap = 0;
-        if ((e = cudaMalloc(&s.frows, sizeof(int32_t) * (size_t)n_rows)) == cudaSuccess) s.frows_cap = n_rows;
+        if ((e = device_alloc(&s.frows, sizeof(int32_t) * (size_t)n_rows, s.kept)) == cudaSuccess) s.frows_cap = n_rows;
     }
     if (e != cudaSuccess) return cuda_fail(c, e, what);
     cudaStream_t str = c->stream;
@@ -1662,7 +1664,7 @@ line_status line_mlp_get_features(line_ctx* c, float* out) {
         return LINE_OK;
     }
     void* buf = nullptr;
-    CK(cudaMalloc(&buf, n * 4), "line_mlp_get_features");
+    CK(device_alloc(&buf, n * 4, s.kept), "line_mlp_get_features");
     cudaError_t e = convert_rows(s.X, LINE_DTYPE_BF16, buf, LINE_DTYPE_F32, nullptr, c->n_nodes, s.P, c->n_nodes,
                                  c->status, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, buf, n * 4, cudaMemcpyDefault, c->stream);
@@ -1755,7 +1757,7 @@ line_status line_mlp_train(line_ctx* c, const int32_t* nodes, int64_t n_nodes, i
         if (s.losses) cudaFree(s.losses);
         s.losses = nullptr;
         s.loss_cap = 0;
-        CK(cudaMalloc(&s.losses, sizeof(double) * steps), "line_mlp_train");
+        CK(device_alloc(&s.losses, sizeof(double) * steps, s.kept), "line_mlp_train");
         s.loss_cap = steps;
     }
     // node ids out of range are reported by the gather (status word)
@@ -1812,7 +1814,7 @@ line_status line_mlp_predict(line_ctx* c, const int32_t* rows, int64_t n_rows, f
         if (s.frows) cudaFree(s.frows);
         s.frows = nullptr;
         s.frows_cap = 0;
-        if ((e = cudaMalloc(&s.frows, sizeof(int32_t) * (size_t)n_rows)) == cudaSuccess) s.frows_cap = n_rows;
+        if ((e = device_alloc(&s.frows, sizeof(int32_t) * (size_t)n_rows, s.kept)) == cudaSuccess) s.frows_cap = n_rows;
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.frows, rows, sizeof(int32_t) * n_rows, cudaMemcpyDefault, str);
     if (e == cudaSuccess) e = tile_weights(s, str);

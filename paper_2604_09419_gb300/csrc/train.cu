@@ -1778,12 +1778,12 @@ __global__ void __launch_bounds__(kPartThreads) k_group_parts(GroupParams q, int
 struct Buf {
     void* p = nullptr;
     size_t cap = 0;
-    cudaError_t ensure(size_t bytes) {
+    cudaError_t ensure(size_t bytes, DeviceScratch* kept) {
         if (bytes <= cap) return cudaSuccess;
         if (p) cudaFree(p);
         p = nullptr;
         cap = 0;
-        cudaError_t e = cudaMalloc(&p, bytes);
+        cudaError_t e = device_alloc(&p, bytes, kept);
         if (e == cudaSuccess) cap = bytes;
         return e;
     }
@@ -2058,7 +2058,7 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
 
     cudaError_t e;
     auto ensure = [&](Buf& b, size_t bytes) -> bool {
-        if ((e = b.ensure(bytes)) != cudaSuccess) {
+        if ((e = b.ensure(bytes, a.kept)) != cudaSuccess) {
             *err = "device allocation failed (training scratch)";
             return false;
         }

@@ -64,10 +64,10 @@ line_status line_autotune(line_ctx* c, int order, int dim, int K, const line_lr*
         const size_t bytes = (size_t)c->n_nodes * dim * elem_size(t.dtype);
         void* sU = nullptr;
         void* sC = nullptr;
-        if (e == cudaSuccess) e = cudaMalloc(&sU, bytes);
+        if (e == cudaSuccess) e = device_alloc(&sU, bytes, &c->scratch);
         if (sU) scratch.push_back(sU);
         if (e == cudaSuccess) e = cudaMemcpyAsync(sU, t.U, bytes, cudaMemcpyDeviceToDevice, c->stream);
-        if (e == cudaSuccess && t.C) e = cudaMalloc(&sC, bytes);
+        if (e == cudaSuccess && t.C) e = device_alloc(&sC, bytes, &c->scratch);
         if (sC) scratch.push_back(sC);
         if (e == cudaSuccess && t.C) e = cudaMemcpyAsync(sC, t.C, bytes, cudaMemcpyDeviceToDevice, c->stream);
         if (e != cudaSuccess) break;
