@@ -37,8 +37,9 @@
 //   a counter hash of seed, table, row, batch and column group).
 //
 // The order of every floating-point sum is fixed, so results are bitwise
-// reproducible, and a singleton row gets exactly the value the apply step
-// would give it.  Two schedules run the same per-sample and per-segment code:
+// reproducible.  A singleton U row gets exactly the value the apply step would
+// give it; a singleton context row is rounded once less, as its contribution
+// g_j U_b[u] is added by a fused multiply-add.  Two schedules run the same per-sample and per-segment code:
 //   LINE_MODE_BATCHED     two launches per batch, chained with programmatic
 //                         dependent launch;
 //   LINE_MODE_PERSISTENT  one cooperative launch per chunk: resident CTAs
@@ -818,10 +819,9 @@ __device__ __forceinline__ void sample_body_slot(const DataParams& p, int lig, b
             const int32_t y = rec_entry<G::L>(gm, r0, rec, 1 + j, active);
             if (active) {
                 if (inf & kSingleBit) {
-                    const float decay = 1.0f * etalam;
                     float x[G::E];
 #pragma unroll
-                    for (int e = 0; e < G::E; ++e) x[e] = fmaf(-decay, c[e], c[e]) + g * xu[e];
+                    for (int e = 0; e < G::E; ++e) x[e] = fmaf(g, xu[e], fmaf(-etalam, c[e], c[e]));
                     store_row<D, DT>(p.C, y, lig, x, salt, ctx_table);
                 } else {
                     float4* dst = reinterpret_cast<float4*>(p.slab + (int64_t)inf * D + lig * G::E);
