@@ -117,13 +117,6 @@ __device__ __forceinline__ float from_f<float>(float x) { return x; }
 template <>
 __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
 
-
-__device__ __forceinline__ float load_row_elem(const void* U, int dtype, int64_t idx) {
-    return dtype == LINE_DTYPE_F32 ? reinterpret_cast<const float*>(U)[idx]
-                                   : __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(U)[idx]);
-}
-
-
 // ---- initialisation --------------------------------------------------------
 __global__ void k_mlp_init(float* __restrict__ p, int H, int P, int D, uint64_t seed, float s1, float s2) {
     const int64_t n1 = (int64_t)H * P, n2 = (int64_t)D * H;

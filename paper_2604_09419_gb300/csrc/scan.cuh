@@ -1,8 +1,7 @@
-// Device-wide scans over an index space, used by the alias construction and
-// the per-chunk segment build.  Three launches: per-tile reduction, a scan of
-// the tile totals in one block, and a per-tile rescan that hands every index
-// its exclusive and inclusive prefix to an output functor.  The summation
-// order is fixed by the tiling, so integer and FP results are reproducible.
+// Device-wide scans of integers over an index space, used by the alias
+// construction.  Three launches: per-tile reduction, a scan of the tile totals
+// in one block, and a per-tile rescan that hands every index its exclusive and
+// inclusive prefix to an output functor.
 #pragma once
 
 #include <cuda_runtime.h>

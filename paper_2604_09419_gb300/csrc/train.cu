@@ -56,7 +56,6 @@
 #include "line_internal.cuh"
 #include "pdl.cuh"
 #include "rows.cuh"
-#include "scan.cuh"
 
 namespace line {
 
@@ -1200,7 +1199,6 @@ struct GroupParams {
     int64_t batch;
     int64_t chunk_samples;
     uint32_t R, K, parts;  // parts: bucketing CTAs per batch
-    uint32_t row_bits;
     uint32_t R_magic;       // floor(2^32 / R) + 1: i / R = mulhi(i, R_magic) for i < 2^32 / R
     uint32_t ctx_off;       // row id of the context table's first row
     const int32_t* rec;     // draws, (sample, slot) order
@@ -1833,7 +1831,6 @@ struct TrainWorkspace {
     cudaStream_t cap = nullptr;     // stream the data-phase graphs are captured on
     bool graph_failed = false;      // a capture failed: direct launches from then on
     cudaEvent_t start = nullptr;    // caller-stream work before the call
-    cudaEvent_t prep_end = nullptr; // last pre-pass of the call
     std::vector<cudaEvent_t> events;  // timing events
     cudaError_t event(size_t i, cudaEvent_t* out) {
         while (events.size() <= i) {
@@ -1856,7 +1853,6 @@ struct TrainWorkspace {
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&cs.data_done, cudaEventDisableTiming);
         }
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&start, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&prep_end, cudaEventDisableTiming);
         (void)device;
         return e;
     }
@@ -1873,7 +1869,6 @@ struct TrainWorkspace {
                 if (g.exec) cudaGraphExecDestroy(g.exec);
         }
         if (start) cudaEventDestroy(start);
-        if (prep_end) cudaEventDestroy(prep_end);
         for (auto e : events) cudaEventDestroy(e);
     }
 };
@@ -2162,7 +2157,6 @@ cudaError_t train_run(const TrainArgs& a, TrainWorkspace* ws, uint32_t* status, 
     gq.R = (uint32_t)R;
     gq.K = (uint32_t)a.K;
     gq.parts = parts;
-    gq.row_bits = row_bits;
     gq.R_magic = (uint32_t)(((uint64_t)1 << 32) / (uint32_t)R) + 1u;
     gq.ctx_off = a.order == 2 ? (uint32_t)a.n_nodes : 0u;
     gq.bucketed = (uint64_t*)ws->items1.p;
