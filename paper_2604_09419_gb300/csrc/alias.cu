@@ -79,20 +79,18 @@ __device__ __forceinline__ unsigned long long block_sum(unsigned long long v, un
     return v;
 }
 
-// row_ptr[v] = e for the nodes v in [v0, v1] between two arcs.  In an unsorted
+// row_ptr[v] = e for the nodes v in [v0, v1] between two arcs, written by a
+// whole warp (by one thread a run of 2^24 nodes took 56 ms).  In an unsorted
 // graph every ascent begins such a run (2^22 random arcs over 2^20 nodes: 7e11
-// entries), so a long one ends once any thread has found the graph invalid.
+// entries), so one ends once any thread has found the graph invalid.
 constexpr int64_t kFillShort = 32, kFillPiece = 1024;
 
 __device__ __forceinline__ void fill_offsets(int64_t* __restrict__ row_ptr, int64_t v0, int64_t v1, int64_t e,
                                              const uint32_t* status) {
-    if (v1 - v0 < kFillShort) {
-        for (int64_t v = v0; v <= v1; ++v) row_ptr[v] = e;
-        return;
-    }
+    const int lane = threadIdx.x & 31;
     for (int64_t v = v0; v <= v1; v += kFillPiece) {
         if (*(volatile const uint32_t*)status & DEV_ERR_GRAPH) return;
-        for (int64_t q = v, end = min(v1, v + kFillPiece - 1); q <= end; ++q) row_ptr[q] = e;
+        for (int64_t q = v + lane, end = min(v1, v + kFillPiece - 1); q <= end; q += 32) row_ptr[q] = e;
     }
 }
 
@@ -112,13 +110,16 @@ __global__ void __launch_bounds__(256) k_graph_scan(int64_t n_nodes, int64_t n_a
                                                     int64_t* __restrict__ row_ptr, unsigned long long* __restrict__ degi,
                                                     GraphScan* __restrict__ out, uint32_t* status) {
     __shared__ unsigned long long part[8];
+    const int lane = threadIdx.x & 31;
     bool frac = false;
     unsigned long long total = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * kArcs;
-    for (int64_t e0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * kArcs; e0 < n_arcs; e0 += stride) {
+    // (whole warps go round)
+    for (int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane) * kArcs; w0 < n_arcs; w0 += stride) {
+        const int64_t e0 = w0 + lane * kArcs;
         int32_t s[kArcs], d[kArcs];
         float x[kArcs];
-        const int cnt = (int)min((int64_t)kArcs, n_arcs - e0);
+        const int cnt = (int)max((int64_t)0, min((int64_t)kArcs, n_arcs - e0));
         if (cnt == kArcs) {  // (the library's own copies: 256-byte aligned)
 #pragma unroll
             for (int q = 0; q < kArcs / 4; ++q) {
@@ -136,38 +137,55 @@ __global__ void __launch_bounds__(256) k_graph_scan(int64_t n_nodes, int64_t n_a
                 x[k] = k < cnt && w ? w[e0 + k] : 1.0f;
             }
         }
-        int32_t prev = e0 > 0 ? src[e0 - 1] : -1;
-        bool ok = true;
+        const int32_t before = cnt && e0 > 0 ? src[e0 - 1] : -1;
+        bool ok = before >= -1;
 #pragma unroll
         for (int k = 0; k < kArcs; ++k) {
             if (k >= cnt) continue;
-            ok = ok && s[k] >= 0 && s[k] < n_nodes && s[k] >= (k > 0 ? s[k - 1] : prev) && d[k] >= 0 && d[k] < n_nodes &&
+            ok = ok && s[k] >= 0 && s[k] < n_nodes && s[k] >= (k > 0 ? s[k - 1] : before) && d[k] >= 0 && d[k] < n_nodes &&
                  x[k] > 0.0f && isfinite(x[k]);
         }
-        if (!ok || prev < -1) {
-            if (!(*(volatile const uint32_t*)status & DEV_ERR_GRAPH)) atomicOr(status, DEV_ERR_GRAPH);
-            continue;
-        }
-        unsigned long long run = 0;
+        if (!ok && !(*(volatile const uint32_t*)status & DEV_ERR_GRAPH)) atomicOr(status, DEV_ERR_GRAPH);
+        const bool last = e0 + cnt == n_arcs;  // the nodes after the last arc's follow
+        bool far = false;                      // a run too long for one thread
+        if (ok && cnt) {
+            int32_t prev = before;
+            unsigned long long run = 0;
 #pragma unroll
-        for (int k = 0; k < kArcs; ++k) {
-            if (k < cnt) {
-                const bool whole = x[k] >= 1.0f && x[k] <= 16777216.0f && x[k] == truncf(x[k]);
-                frac |= !whole;
-                const uint32_t xi = whole ? __float2uint_rz(x[k]) : 0u;
-                total += xi;
-                if (s[k] != prev) {
-                    if (run) atomicAdd(degi + prev, run);
-                    run = 0;
-                    fill_offsets(row_ptr, (int64_t)prev + 1, s[k], e0 + k, status);
+            for (int k = 0; k < kArcs; ++k) {
+                if (k < cnt) {
+                    const bool whole = x[k] >= 1.0f && x[k] <= 16777216.0f && x[k] == truncf(x[k]);
+                    frac |= !whole;
+                    const uint32_t xi = whole ? __float2uint_rz(x[k]) : 0u;
+                    total += xi;
+                    if (s[k] != prev) {
+                        if (run) atomicAdd(degi + prev, run);
+                        run = 0;
+                        if ((int64_t)s[k] - prev > kFillShort) far = true;
+                        else
+                            for (int64_t v = (int64_t)prev + 1; v <= s[k]; ++v) row_ptr[v] = e0 + k;
+                    }
+                    run += xi;
+                    prev = s[k];
                 }
-                run += xi;
-                prev = s[k];
+            }
+            if (run) atomicAdd(degi + prev, run);
+            far |= last;
+        }
+        if (__any_sync(0xFFFFFFFFu, far)) {
+#pragma unroll
+            for (int k = 0; k <= kArcs; ++k) {
+                // the run before arc k; k = cnt: the one after the last arc
+                const int64_t lo = (int64_t)(k > 0 ? s[k > 0 ? k - 1 : 0] : before) + 1;
+                const int64_t hi = k < cnt ? (int64_t)s[k < kArcs ? k : 0] : n_nodes;
+                const bool mine = ok && cnt && (k < cnt ? hi - lo >= kFillShort : k == cnt && last);
+                for (uint32_t mask = __ballot_sync(0xFFFFFFFFu, mine); mask; mask &= mask - 1) {
+                    const int l = __ffs(mask) - 1;
+                    fill_offsets(row_ptr, __shfl_sync(0xFFFFFFFFu, lo, l), __shfl_sync(0xFFFFFFFFu, hi, l),
+                                 __shfl_sync(0xFFFFFFFFu, e0 + k, l), status);
+                }
             }
         }
-        if (run) atomicAdd(degi + prev, run);
-        // the nodes after the last arc's
-        if (e0 + cnt == n_arcs) fill_offsets(row_ptr, (int64_t)prev + 1, n_nodes, n_arcs, status);
     }
     if (frac) out->frac = 1u;
     total = block_sum(total, part);
