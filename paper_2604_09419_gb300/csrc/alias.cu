@@ -100,7 +100,7 @@ __device__ __forceinline__ void fill_offsets(int64_t* __restrict__ row_ptr, int6
 // before).  A thread takes kArcs consecutive arcs: a node's run inside them
 // is added with one atomic (src is sorted).  A thread reports an invalid arc
 // before it writes any offset, and then writes none.
-// Bound: HBM (12 bytes an arc) and the run's branches: 185 us for 31.4M arcs;
+// Bound: HBM (12 bytes an arc) and the run's branches: 200 us for 31.4M arcs;
 // the validation, the row offsets, the integer check and the node sums (a
 // warp a node) took 85 + 64 + 25 + 1,357 us as four kernels.
 constexpr int kArcs = 8;

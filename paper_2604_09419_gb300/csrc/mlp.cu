@@ -382,8 +382,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_hub_plan(FeatParams p) {
 // for rows of 256, which hold more registers).  Chunks and nodes in one kernel
 // fill each other's tails; a chunk's hub is found by a 32-way search, and the
 // block goes on to its next chunk while warp 0 adds the warps' sums.  R-MAT
-// 20, BF16 rows of 128: a sample of 65,536 nodes 243 -> 121 us, the 104,857
-// new nodes 340 -> 180 (two kernels, a binary search, two barriers a chunk).
+// 20, BF16 rows of 128: a sample of 65,536 nodes 243 -> 120 us, the 104,857
+// new nodes 340 -> 188 (two kernels, a binary search, two barriers a chunk).
 template <int D>
 constexpr int kFeatureBlocks = D <= 128 ? 4 : 3;
 
@@ -1104,8 +1104,8 @@ __global__ void __launch_bounds__(32 * kColGroups) k_colsum_slices(const float* 
 // The end of a step in one kernel: every parameter's gradient, its slices
 // summed in order, then (Adam) the parameter's update and its place in the
 // tensor-core tiles of the next forward pass.  As a kernel each - four sums,
-// Adam, three tilings - they took 26 us a step and eight launches, this
-// 5 us and one (18 MB of partial sums from L2).
+// Adam, three tilings - they took 26 us a step and eight launches, this 9 us
+// with cold caches and one (18 MB of partial sums).
 struct UpdateArgs {
     const float *w2, *w1, *b1, *b2;  // partial sums
     int SW, SB;                      // their slices: weights, biases
